@@ -608,8 +608,9 @@ int hdmc_batch_psi6(hdmc_batch_t* b, double r_cut, double* out) {
     const size_t el = b->prec == HDMC_FP64 ? sizeof(double) : sizeof(float);
     std::vector<size_t> off(b->R + 1, 0);
     for (int r = 0; r < b->R; ++r) off[r + 1] = off[r] + 4 * (size_t)psi6_blocks(b->sys[r].g);
-    if (sizeof(double) * off[b->R] > b->lay.arena) return HDMC_EINVAL;
+    if (sizeof(double) * (off[b->R] + 4 * (size_t)b->R) > b->lay.arena) return HDMC_EINVAL;
     double* partial = reinterpret_cast<double*>(b->arena[b->cur ^ 1]);
+    double* totals = partial + off[b->R];   // 4 per replica, behind the block sums
     const char* cur = static_cast<const char*>(b->arena[b->cur]);
     int e = HDMC_OK;
     for (int r = 0; r < b->R && !e; ++r) {
@@ -617,21 +618,17 @@ int hdmc_batch_psi6(hdmc_batch_t* b, double r_cut, double* out) {
         c.g = b->sys[r].g;
         c.stream = s;
         const void* cells = cur + (size_t)b->cell_off[r] * 8 * el;
-        if (b->prec == HDMC_FP64) launch_psi6_f64(c, cells, r_cut * r_cut, nullptr, partial + off[r]);
-        else launch_psi6_f32(c, cells, r_cut * r_cut, nullptr, partial + off[r]);
+        if (b->prec == HDMC_FP64) launch_psi6_f64(c, cells, r_cut * r_cut, nullptr, partial + off[r], totals + 4 * r);
+        else launch_psi6_f32(c, cells, r_cut * r_cut, nullptr, partial + off[r], totals + 4 * r);
         e = cuda_code(cudaGetLastError());
     }
-    std::vector<double> part(off[b->R]);
+    std::vector<double> part(4 * (size_t)b->R);
     if (!e)
-        e = cuda_code(cudaMemcpyAsync(part.data(), partial, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, s));
+        e = cuda_code(cudaMemcpyAsync(part.data(), totals, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, s));
     if (!e) e = cuda_code(cudaStreamSynchronize(s));
     if (e) return e;
-    for (int r = 0; r < b->R; ++r) {
-        double sum[4] = {0, 0, 0, 0};
-        for (size_t i = off[r]; i < off[r + 1]; i += 4)
-            for (int k = 0; k < 4; ++k) sum[k] += part[i + k];
-        for (int k = 0; k < 4; ++k) out[4 * r + k] = sum[k] / (double)b->sys[r].N;
-    }
+    for (int r = 0; r < b->R; ++r)
+        for (int k = 0; k < 4; ++k) out[4 * r + k] = part[4 * (size_t)r + k] / (double)b->sys[r].N;
     return HDMC_OK;
 }
 

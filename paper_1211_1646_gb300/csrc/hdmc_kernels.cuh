@@ -391,56 +391,196 @@ k_hist(const Geometry g, const T* __restrict__ cells, const double* __restrict__
 // z = dx + i dy from cell-local coordinates as in the histogram, 0 without
 // neighbours.  Pairs in the order dy, dx, slot and every binary64 operation
 // explicitly rounded, so psi_6(j) is the same number whatever the launch.
-// One thread per cell (grid of the histogram); block sums of
-// {re, im, |psi_6|, n} in a fixed order to partial[4 * block].
+//
+// The binary64 pipe binds this kernel (1/64 of the binary32 rate, about 50
+// binary64 instructions per neighbour), so it is given only neighbours, and
+// full warps of them: a binary32 estimate with a margin above its error
+// selects each disk's candidates (6 of the 23 disks of 25 cells at r_cut =
+// 1.4 sigma) into a list per lane; the lists of a warp are laid end to end
+// and evaluated 32 at a time, and each lane then adds its own terms up in
+// list order, which is the order dy, dx, slot.  Coordinates are widened to
+// binary64 on the integer pipe.  N = 1M, phi = 0.716, r_cut = 1.4 sigma,
+// binary32, one histogram, pressure and psi_6: 3.25 -> 0.96 ms (the pair loop
+// in binary64 over every disk of the 25 cells had 18.7 of 32 lanes active).
+// One thread per cell, one warp per 32 cells of a set row; block sums of
+// {re, im, |psi_6|, n} in a fixed order to partial[4 * block]; k_psi6_sum adds
+// them up, so that the host reads four numbers.
+constexpr int kPsiBX = 32, kPsiBY = 4;
+constexpr int kPsiList = 32;    // candidates a lane holds; a cell adds at most 16
+constexpr int kPsiFlat = 256;   // terms evaluated between two rounds of sums
+
+// Exact binary32 -> binary64 on the integer pipe (conversions run on the
+// binary64 pipe); subnormal binary32 values, not met in earnest, convert.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
+    if (m < 0x00800000u && m != 0u) return (double)v;
+    const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// 2 v exactly as __dmul_rn(2.0, v) gives it, on the integer pipe (v finite
+// and far below overflow; a subnormal v, not met in earnest, is multiplied).
+__device__ __forceinline__ double twice(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), e = hi & 0x7FF00000u;
+    if (e == 0u) return __dmul_rn(2.0, v);
+    return __hiloint2double((int)(hi + 0x00100000u), __double2loint(v));
+}
+
+struct PsiShared {
+    uint16_t list[kPsiList][kPsiBX];   // entry: own slot (2 bits), slot (2), dx + 2 (3), dy + 2 (3)
+    uint32_t flat[kPsiFlat];           // entry | lane << 10, bit 31 set once found within r_cut
+    double2 term[kPsiFlat];            // z^6 / |z|^6
+};
+
+// Evaluates the warp's listed candidates and adds each lane's terms to its
+// disks' sums in list order (warp-uniform call).
 template <typename T>
-__global__ void __launch_bounds__(kHistBX * kHistBY)
+__device__ __forceinline__ void psi6_flush(const Geometry& g, const T* __restrict__ cells, PsiShared& s, int count,
+                                           long long own0, int cx0, int cy, double rc2, const double* shx,
+                                           const double* shy, double are[4], double aim[4], int nb[4]) {
+    const int lane = threadIdx.x;
+    int first = count;   // exclusive prefix sum of the counts
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, first, o);
+        first += lane >= o ? v : 0;
+    }
+    const int total = __shfl_sync(0xffffffffu, first, 31);
+    first -= count;
+    for (int base = 0; base < total; base += kPsiFlat) {
+        const int k0 = max(0, base - first), k1 = min(count, base + kPsiFlat - first);   // my share of this part
+        for (int k = k0; k < k1; ++k) s.flat[first + k - base] = (uint32_t)s.list[k][lane] | ((uint32_t)lane << 10);
+        __syncwarp();
+        const int n = min(kPsiFlat, total - base);
+        for (int f = lane; f < n; f += 32) {
+            const uint32_t e = s.flat[f];
+            const int i = e & 3, j = (e >> 2) & 3, dx = (int)((e >> 4) & 7) - 2, dy = (int)((e >> 7) & 7) - 2;
+            const int src = (e >> 10) & 31;
+            const T* own = cells + 8 * (own0 + src);
+            const T* q = cells + 8 * storage_index(g, wrap(cx0 + 2 * src + dx, g.mx), wrap(cy + dy, g.my));
+            const double ddx = __dsub_rn(widen(__ldg(own + i)), __dadd_rn(widen(__ldg(q + j)), shx[dx + 2]));
+            const double ddy = __dsub_rn(widen(__ldg(own + 4 + i)), __dadd_rn(widen(__ldg(q + 4 + j)), shy[dy + 2]));
+            const double xx = __dmul_rn(ddx, ddx), yy = __dmul_rn(ddy, ddy);
+            const double r2 = __dadd_rn(xx, yy);
+            // r2 >= +0 and rc2 > 0: their bit patterns order as they do
+            if (__double_as_longlong(r2) < __double_as_longlong(rc2)) {
+                const double ar = __dsub_rn(xx, yy);   // z^2
+                const double ai = twice(__dmul_rn(ddx, ddy));
+                const double br = __dsub_rn(__dmul_rn(ar, ddx), __dmul_rn(ai, ddy));   // z^3
+                const double bi = __dadd_rn(__dmul_rn(ar, ddy), __dmul_rn(ai, ddx));
+                const double zr = __dsub_rn(__dmul_rn(br, br), __dmul_rn(bi, bi));   // z^6
+                const double zi = twice(__dmul_rn(br, bi));
+                const double r6 = __dmul_rn(__dmul_rn(r2, r2), r2);
+                s.term[f] = make_double2(__ddiv_rn(zr, r6), __ddiv_rn(zi, r6));
+                s.flat[f] = e | 0x80000000u;
+            }
+        }
+        __syncwarp();
+        for (int k = k0; k < k1; ++k) {
+            const uint32_t e = s.flat[first + k - base];
+            if (e >> 31) {
+                const int i = e & 3;
+                const double2 t = s.term[first + k - base];
+                const double r = __dadd_rn(pick(are, i), t.x), m = __dadd_rn(pick(aim, i), t.y);
+                put_if(are, i, r, true);
+                put_if(aim, i, m, true);
+                put_if(nb, i, pick(nb, i) + 1, true);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPsiBX * kPsiBY)
 k_psi6(const Geometry g, const T* __restrict__ cells, double rc2, double* __restrict__ psi,
        double* __restrict__ partial) {
-    __shared__ double red[kHistBY][4];
+    __shared__ PsiShared sh[kPsiBY];
+    __shared__ double red[kPsiBY][3];
+    __shared__ int redn[kPsiBY];
+    __shared__ double shx[5], shy[5];   // cell offsets (dx - 2) wx, (dy - 2) wy
+    const int lane = threadIdx.x;
     const int q = blockIdx.z;
-    const int hx = blockIdx.x * kHistBX + threadIdx.x, hy = blockIdx.y * kHistBY + threadIdx.y;
+    const int hx = blockIdx.x * kPsiBX + lane, hy = blockIdx.y * kPsiBY + threadIdx.y;
+    if (threadIdx.y == 0 && lane < 10) {
+        const int k = lane % 5;
+        const double w = lane < 5 ? (double)Prm<T>::wx(g) : (double)Prm<T>::wy(g);
+        (lane < 5 ? shx : shy)[k] = (double)(k - 2) * w;
+    }
+    __syncthreads();
     const bool live = hx < g.hx && hy < g.hy;
     const int cx = 2 * hx + (q & 1), cy = 2 * hy + (q >> 1);
-    const double wxd = (double)Prm<T>::wx(g), wyd = (double)Prm<T>::wy(g);
+    const long long own0 = (long long)q * g.cq + (long long)hy * g.hx + (long long)blockIdx.x * kPsiBX;
     Cell<T> own;
 #pragma unroll
     for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = T(kEmpty);
-    if (live) load_cell_ro(cells + 8 * ((long long)q * g.cq + (long long)hy * g.hx + hx), own);
+    if (live) load_cell_ro(cells + 8 * (own0 + lane), own);
     double are[4] = {0, 0, 0, 0}, aim[4] = {0, 0, 0, 0};
     int nb[4] = {0, 0, 0, 0};
-    if (live) {
-        for (int dy = -2; dy <= 2; ++dy)
+    if (__any_sync(0xffffffffu, Prm<T>::ge0(own.x[0]))) {
+        PsiShared& s = sh[threadIdx.y];
+        const float wxf = (float)Prm<T>::wx(g), wyf = (float)Prm<T>::wy(g);
+        // estimate: |error of a difference| < 1e-6 (wx + wy), below the margin on r_cut
+        const float rcf = sqrtf((float)rc2) * 1.00001f + 1.0e-5f * (wxf + wyf);
+        const f2x nt = pk(-rcf * rcf, -rcf * rcf);
+        const bool own23 = __any_sync(0xffffffffu, Prm<T>::ge0(own.x[2]));
+        const bool corners = rcf * rcf > wxf * wxf + wyf * wyf;   // cells (+-2, +-2) start sqrt(wx^2 + wy^2) away
+        float ox[4], oy[4];
+        uint32_t occupied = 0;   // bits 4i..4i+3 set when own slot i holds a disk
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ox[i] = to_f32(own.x[i]);
+            oy[i] = to_f32(own.y[i]);
+            occupied |= Prm<T>::ge0(own.x[i]) ? (0xFu << (4 * i)) : 0u;
+        }
+        int count = 0;
+        for (int dy = -2; dy <= 2; ++dy) {
+            const int ny = wrap(cy + dy, g.my);
             for (int dx = -2; dx <= 2; ++dx) {
+                if (!corners && (dx == -2 || dx == 2) && (dy == -2 || dy == 2)) continue;
                 Cell<T> c;
-                load_cell_ro(cells + 8 * storage_index(g, wrap(cx + dx, g.mx), wrap(cy + dy, g.my)), c);
-                const double sx = (double)dx * wxd, sy = (double)dy * wyd;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) c.x[j] = c.y[j] = T(kEmpty);
+                if (live) load_cell_ro(cells + 8 * storage_index(g, wrap(cx + dx, g.mx), ny), c);
+                const float sxf = (float)dx * wxf, syf = (float)dy * wyf;
+                const f2x qx01 = add2(pk(to_f32(c.x[0]), to_f32(c.x[1])), pk(sxf, sxf));
+                const f2x qx23 = add2(pk(to_f32(c.x[2]), to_f32(c.x[3])), pk(sxf, sxf));
+                const f2x qy01 = add2(pk(to_f32(c.y[0]), to_f32(c.y[1])), pk(syf, syf));
+                const f2x qy23 = add2(pk(to_f32(c.y[2]), to_f32(c.y[3])), pk(syf, syf));
+                const bool c23 = __any_sync(0xffffffffu, Prm<T>::ge0(c.x[2]));
+                uint32_t cand = 0, there = 0;   // bit 4i+j: pair (own i, neighbour slot j)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) there |= Prm<T>::ge0(c.x[j]) ? (0x1111u << j) : 0u;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    if (!Prm<T>::ge0(own.x[i])) continue;
-                    const double px = (double)own.x[i], py = (double)own.y[i];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (!Prm<T>::ge0(c.x[j]) || (dx == 0 && dy == 0 && j == i)) continue;
-                        const double ddx = __dsub_rn(px, __dadd_rn((double)c.x[j], sx));
-                        const double ddy = __dsub_rn(py, __dadd_rn((double)c.y[j], sy));
-                        const double r2 = __dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy));
-                        if (!(r2 < rc2)) continue;
-                        const double ar = __dsub_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy));   // z^2
-                        const double ai = __dmul_rn(2.0, __dmul_rn(ddx, ddy));
-                        const double br = __dsub_rn(__dmul_rn(ar, ddx), __dmul_rn(ai, ddy));     // z^3
-                        const double bi = __dadd_rn(__dmul_rn(ar, ddy), __dmul_rn(ai, ddx));
-                        const double zr = __dsub_rn(__dmul_rn(br, br), __dmul_rn(bi, bi));      // z^6
-                        const double zi = __dmul_rn(2.0, __dmul_rn(br, bi));
-                        const double r6 = __dmul_rn(__dmul_rn(r2, r2), r2);
-                        are[i] = __dadd_rn(are[i], __ddiv_rn(zr, r6));
-                        aim[i] = __dadd_rn(aim[i], __ddiv_rn(zi, r6));
-                        nb[i] += 1;
+                    if (i >= 2 && !own23) continue;
+                    const f2x tx2 = pk(ox[i], ox[i]), ty2 = pk(oy[i], oy[i]);
+                    f2x z = zpair(tx2, ty2, qx01, qy01, nt);
+                    cand |= ((lo32(z) >> 31) << (4 * i)) | ((hi32(z) >> 31) << (4 * i + 1));
+                    if (c23) {
+                        z = zpair(tx2, ty2, qx23, qy23, nt);
+                        cand |= ((lo32(z) >> 31) << (4 * i + 2)) | ((hi32(z) >> 31) << (4 * i + 3));
                     }
                 }
+                cand &= occupied & there;
+                if (dx == 0 && dy == 0) cand &= ~0x8421u;
+                const uint32_t tag = ((uint32_t)(dx + 2) << 4) | ((uint32_t)(dy + 2) << 7);
+                while (cand) {
+                    const int b = __ffs(cand) - 1;
+                    cand &= cand - 1;
+                    s.list[count++][lane] = (uint16_t)(tag | (uint32_t)(b >> 2) | ((uint32_t)(b & 3) << 2));
+                }
+                if (__any_sync(0xffffffffu, count > kPsiList - 16)) {
+                    psi6_flush<T>(g, cells, s, count, own0, cx - 2 * lane, cy, rc2, shx, shy, are, aim, nb);
+                    count = 0;
+                }
             }
+        }
+        psi6_flush<T>(g, cells, s, count, own0, cx - 2 * lane, cy, rc2, shx, shy, are, aim, nb);
     }
-    double t[4] = {0, 0, 0, 0};   // re, im, |psi_6|, neighbours of this thread's disks
+    double t[3] = {0, 0, 0};   // re, im, |psi_6| of this thread's disks
+    int tn = 0;                // their neighbours
     const long long cc = (long long)cy * g.mx + cx;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -453,26 +593,47 @@ k_psi6(const Geometry g, const T* __restrict__ cells, double rc2, double* __rest
             t[1] = __dadd_rn(t[1], pi);
             t[2] = __dadd_rn(t[2], __dsqrt_rn(__dadd_rn(__dmul_rn(pr, pr), __dmul_rn(pi, pi))));
         }
-        t[3] = __dadd_rn(t[3], (double)nb[i]);
+        tn += nb[i];
         if (psi) {
             psi[(4 * cc + i) * 2] = pr;
             psi[(4 * cc + i) * 2 + 1] = pi;
         }
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 3; ++k)
         for (int o = 16; o > 0; o >>= 1) t[k] = __dadd_rn(t[k], __shfl_down_sync(0xffffffffu, t[k], o));
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 4; ++k) red[threadIdx.y][k] = t[k];
-    __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        for (int k = 0; k < 4; ++k) {
-            double v = 0.0;
-            for (int w = 0; w < kHistBY; ++w) v = __dadd_rn(v, red[w][k]);
-            partial[4 * b + k] = v;
-        }
+    tn = __reduce_add_sync(0xffffffffu, tn);
+    if (lane == 0) {
+        for (int k = 0; k < 3; ++k) red[threadIdx.y][k] = t[k];
+        redn[threadIdx.y] = tn;
     }
+    __syncthreads();
+    if (lane < 4 && threadIdx.y == 0) {
+        const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        double v = 0.0;
+        int n = 0;
+        for (int w = 0; w < kPsiBY; ++w) {
+            if (lane < 3) v = __dadd_rn(v, red[w][lane]);
+            n += redn[w];
+        }
+        partial[4 * b + lane] = lane < 3 ? v : (double)n;
+    }
+}
+
+// Sums of the nb block sums into out[0..3], in an order fixed by nb alone
+// (one block; out does not overlap the partials).
+static __global__ void __launch_bounds__(256) k_psi6_sum(const double* __restrict__ partial, unsigned nb,
+                                                         double* __restrict__ out) {
+    __shared__ double red[256];
+    const int k = threadIdx.x & 3;
+    double v = 0.0;
+    for (unsigned b = threadIdx.x >> 2; b < nb; b += 64) v = __dadd_rn(v, partial[4 * (size_t)b + k]);
+    red[threadIdx.x] = v;
+    for (int o = 128; o >= 4; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) red[threadIdx.x] = __dadd_rn(red[threadIdx.x], red[threadIdx.x + o]);
+    }
+    if (threadIdx.x < 4) out[k] = red[k];
 }
 
 // ---- batched replicas ------------------------------------------------------------------
@@ -549,10 +710,12 @@ void launch_shift_t(const LaunchCtx& c, const void* src, void* dst, const SweepD
 }
 
 template <typename T>
-void launch_psi6_t(const LaunchCtx& c, const void* cells, double rc2, double* psi, double* partial) {
-    const dim3 block(kHistBX, kHistBY);
-    k_psi6<T><<<set_grid(c.g, block), block, 0, c.stream>>>(c.g, reinterpret_cast<const T*>(cells), rc2, psi,
-                                                             partial);
+void launch_psi6_t(const LaunchCtx& c, const void* cells, double rc2, double* psi, double* partial, double* out) {
+    const dim3 block(kPsiBX, kPsiBY);
+    const dim3 grid = set_grid(c.g, block);
+    const unsigned nb = grid.x * grid.y * grid.z;
+    k_psi6<T><<<grid, block, 0, c.stream>>>(c.g, reinterpret_cast<const T*>(cells), rc2, psi, partial);
+    k_psi6_sum<<<1, 256, 0, c.stream>>>(partial, nb, out);
 }
 
 template <typename T>
