@@ -341,6 +341,7 @@ struct hdmc3_handle {
     int cur;
     Draw3* table;              // kDrawChunk3 sweep draws + 1 extra entry
     Dev3* st;
+    unsigned long long* ctr;   // kCtr3 x 4 trial counters since creation or load
     unsigned long long* hist;  // kHistBins accumulator
     double* edges2;            // kHistBins + 1 squared bin edges
     float* binf;               // binary32 bin bounds that decide a bin for certain (certified_bins)
@@ -358,6 +359,15 @@ int finish3(hdmc3_t* h) {
     e = cudaMemcpy(&err, &h->st->error, sizeof(err), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_code(e);
     return error_code(err);
+}
+
+// Adds the counter slots to the counters of st (the handle's stream is idle).
+int add_counters3(hdmc3_t* h, Dev3& st) {
+    unsigned long long c[4 * kCtr3];
+    const cudaError_t e = cudaMemcpy(c, h->ctr, sizeof(c), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_code(e);
+    for (int i = 0; i < 4 * kCtr3; ++i) st.ctr[i & 3] += c[i];
+    return HDMC_OK;
 }
 
 bool make_grid3(const double L[3], double sigma, int m[3], double w[3]) {
@@ -539,11 +549,30 @@ int download3(hdmc3_t* h, std::vector<double>& loc, std::vector<uint8_t>& cnt) {
 }
 
 void launch_sub3(hdmc3_t* h, int jd, int k) {
-    const unsigned blocks = (h->g.cq + kSubB3 - 1) / kSubB3;
-    if (h->prec == HDMC_FP64)
-        k_sub3<double><<<blocks, kSubB3, 0, h->stream>>>(h->g, (double*)h->cells[h->cur], h->table, jd, k, h->st);
-    else
-        k_sub3<float><<<blocks, kSubB3, 0, h->stream>>>(h->g, (float*)h->cells[h->cur], h->table, jd, k, h->st);
+    auto run = [&](auto kernel, auto* cells, unsigned G) {
+        const unsigned per = kSubB3 / G;
+        kernel<<<(h->g.cq + per - 1) / per, kSubB3, 0, h->stream>>>(h->g, cells, h->table, jd, k, h->ctr);
+    };
+    // Lanes per cell: few active cells leave the chip idle and the chain of
+    // one cell update binds, so its work is spread over a warp; many are bound
+    // by instructions, of which wide groups need more.  us per sub-sweep at
+    // n_M = 4 with 32 / 8 / 4 / 2 lanes, binary32 then binary64:
+    //     2,197 active cells   6.2 / 6.7 / 8.2 / 8.6       9.2 / 11.6 / 13.2 / 17.1
+    //     7,000               10.3 / 8.3 / 8.5 / 10.3     16.0 / 14.1 / 15.7 / 18.6
+    //    32,768               29.0 / 19.3 / 15.7 / 16.2   46.8 / 34.7 / 29.8 / 31.8
+    //   132,651              103.2 / 55.4 / 39.7 / 37.1   172 / 108 / 93.2 / 93.9
+    const unsigned cq = h->g.cq;
+    if (h->prec == HDMC_FP64) {
+        double* a = (double*)h->cells[h->cur];
+        if (cq <= 4096) run(k_sub3<double, 32>, a, 32);
+        else if (cq <= 16384) run(k_sub3<double, 8>, a, 8);
+        else run(k_sub3<double, 4>, a, 4);
+    } else {
+        float* a = (float*)h->cells[h->cur];
+        if (cq <= 4096) run(k_sub3<float, 32>, a, 32);
+        else if (cq <= 16384) run(k_sub3<float, 8>, a, 8);
+        else run(k_sub3<float, 2>, a, 2);
+    }
 }
 
 void launch_shift3(hdmc3_t* h, int jd) {
@@ -563,6 +592,7 @@ void free3(hdmc3_t* h) {
     cudaFree(h->cells[1]);
     cudaFree(h->table);
     cudaFree(h->st);
+    cudaFree(h->ctr);
     cudaFree(h->hist);
     cudaFree(h->edges2);
     cudaFree(h->binf);
@@ -621,6 +651,12 @@ int enqueue_sweeps3(hdmc3_t* h, int64_t n, double* ms_sub, double* ms_shift) {
     return HDMC_OK;
 }
 
+void set_move3(G3& g, double d) {
+    g.d = d;
+    g.df = (float)d;
+    g.d52 = d * 0x1p-52;
+}
+
 int set_geometry3(G3& g, const double L[3], double sigma, double d, int nselect, uint64_t seed) {
     int m[3];
     double w[3];
@@ -642,11 +678,18 @@ int set_geometry3(G3& g, const double L[3], double sigma, double d, int nselect,
     g.sigma = sigma;
     g.sig2 = sigma * sigma;
     g.sig2f = (float)(sigma * sigma);
-    g.keep2f = (float)(sigma * sigma * (1.0 + 1.0e-3));
-    g.band_lo = (float)(sigma * sigma * (1.0 - 0x1p-14));
-    g.band_hi = (float)(sigma * sigma * (1.0 + 0x1p-14));
-    g.d = d;
-    g.df = (float)d;
+    g.band_lo = (float)(sigma * sigma * (1.0 - 0x1p-16));
+    g.band_hi = (float)(sigma * sigma * (1.0 + 0x1p-16));
+    // quotient by D of any s < 2^30: floor(s (floor(2^(30+l)/D) + 1) / 2^(30+l)) with 2^l >= D
+    // (Granlund and Montgomery, Division by invariant integers using multiplication, PLDI 1994)
+    for (int a = 0; a < 2; ++a) {
+        const unsigned D = (unsigned)g.h[a];
+        unsigned l = 0;
+        while ((1u << l) < D) ++l;
+        g.dm[a] = (unsigned)((1ull << (30 + l)) / D + 1u);
+        g.dsh[a] = 30 + l;
+    }
+    set_move3(g, d);
     g.nsel = nselect;
     g.key0 = (uint32_t)seed;
     g.key1 = (uint32_t)(seed >> 32);
@@ -733,6 +776,9 @@ int hdmc3_save(hdmc3_t* h, void* buf, size_t bytes) {
     if (e) return e;
     Dev3 st;
     std::memcpy(&st, b + L.state, sizeof(st));
+    e = add_counters3(h, st);
+    if (e) return e;
+    std::memcpy(b + L.state, &st, sizeof(st));
     return error_code(st.error);
 }
 
@@ -778,14 +824,14 @@ int hdmc3_load(hdmc3_t* h, const void* buf, size_t bytes) {
     if (r[1] != 0 || r[0] != (unsigned long long)h->N) return HDMC_EINVAL;
     // commit
     e = cuda_code(cudaMemcpyAsync(h->st, &st, sizeof(Dev3), cudaMemcpyHostToDevice, s));
+    if (!e) e = cuda_code(cudaMemsetAsync(h->ctr, 0, sizeof(unsigned long long) * 4 * kCtr3, s));
     if (!e)
         e = cuda_code(cudaMemcpyAsync(h->hist, b + L.hist, sizeof(unsigned long long) * kHistBins,
                                       cudaMemcpyHostToDevice, s));
     if (!e) e = cuda_code(cudaStreamSynchronize(s));
     if (e) return e;
     h->cur = 1 - h->cur;
-    h->g.d = hd.d;
-    h->g.df = (float)hd.d;
+    set_move3(h->g, hd.d);
     h->g.nsel = hd.nsel;
     h->g.key0 = hd.key0;
     h->g.key1 = hd.key1;
@@ -838,11 +884,13 @@ int hdmc3_create(hdmc3_t** out, int64_t N, double Lx, double Ly, double Lz, doub
     if (ce == cudaSuccess) ce = cudaMalloc(&h->cells[1], bytes);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->table, sizeof(Draw3) * (kDrawChunk3 + 1));
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->st, sizeof(Dev3));
+    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->ctr, sizeof(unsigned long long) * 4 * kCtr3);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->hist, sizeof(unsigned long long) * kHistBins);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->edges2, sizeof(double) * (kHistBins + 1));
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->binf, sizeof(float) * (2 * kHistBins + 2));
     if (ce == cudaSuccess) ce = cudaMemcpy(h->cells[0], raw.data(), bytes, cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) ce = cudaMemset(h->st, 0, sizeof(Dev3));
+    if (ce == cudaSuccess) ce = cudaMemset(h->ctr, 0, sizeof(unsigned long long) * 4 * kCtr3);
     if (ce == cudaSuccess) ce = cudaMemset(h->hist, 0, sizeof(unsigned long long) * kHistBins);
     double E[kHistBins + 1];
     squared_edges(sigma, E);
@@ -1037,6 +1085,8 @@ int hdmc3_counters(hdmc3_t* h, uint64_t out[4]) {
     Dev3 st;
     const cudaError_t ce = cudaMemcpy(&st, h->st, sizeof(st), cudaMemcpyDeviceToHost);
     if (ce != cudaSuccess) return cuda_code(ce);
+    const int ec = add_counters3(h, st);
+    if (ec) return ec;
     for (int k = 0; k < 4; ++k) out[k] = st.ctr[k];
     return e;
 }
@@ -1062,8 +1112,7 @@ int hdmc3_set_move_size(hdmc3_t* h, double d) {
     if (!h) return HDMC_EINVAL;
     for (int a = 0; a < 3; ++a)
         if (!(d > 0) || !(d < 0.5 * h->g.w[a])) return HDMC_EINVAL;
-    h->g.d = d;
-    h->g.df = (float)d;
+    set_move3(h->g, d);
     return HDMC_OK;
 }
 

@@ -24,8 +24,6 @@ namespace hdmc {
 constexpr int kSlots3 = 8;          // sum of w^2 < 4 sigma^2 => at most 8 centres per cell
 constexpr int kCell3 = 3 * kSlots3;  // coordinates per cell
 constexpr int kHalf3 = 12;           // coordinates per half cell (4 slots)
-constexpr int kSubB3 = 64;          // sub-sweep block: 64 active cells
-constexpr int kCand3 = 24;          // gathered neighbour spheres per cell (more: read from global)
 constexpr int kShiftB3 = 256;
 constexpr int kHistB3 = 128;
 constexpr int kDrawChunk3 = 64;     // sweeps per draws launch
@@ -41,14 +39,20 @@ struct G3 {
     float wprevf[3];       // largest binary32 below wf
     double sigma, sig2;
     float sig2f;
-    float keep2f;          // gather threshold sigma^2 (1 + 1e-3), binary32
-    float band_lo, band_hi;   // sigma^2 (1 -+ 2^-14): binary32 pair tests outside decide (binary64 mode)
-    double d;
+    float band_lo, band_hi;   // sigma^2 (1 -+ 2^-16): binary32 pair tests outside decide (binary64 mode)
+    double d, d52;         // d, d 2^-52
     float df;
     int nsel;
     uint32_t key0, key1;
     uint32_t flags;        // kNoParticleShuffle | kNoSetShuffle
     unsigned int* check;   // builds with -DHDMC_CHECK: device word that collects failed index checks
+    unsigned dm[2], dsh[2];   // division of a cell number below 2^30 by h[0], h[1]: (s dm) >> dsh
+    __host__ __device__ __forceinline__ unsigned div0(unsigned s) const {
+        return (unsigned)(((unsigned long long)s * dm[0]) >> dsh[0]);
+    }
+    __host__ __device__ __forceinline__ unsigned div1(unsigned s) const {
+        return (unsigned)(((unsigned long long)s * dm[1]) >> dsh[1]);
+    }
 };
 
 struct alignas(8) Draw3 {
@@ -58,8 +62,13 @@ struct alignas(8) Draw3 {
     double ds;
 };
 
+// Trial counters {trials, accepted, left the cell, overlap} are added up in
+// kCtr3 slots (block b in slot b mod kCtr3), so that the sub-sweep's warps do
+// not queue at four addresses; the host adds the slots to Dev3::ctr.
+constexpr int kCtr3 = 64;
+
 struct Dev3 {
-    unsigned long long ctr[4];   // trials, accepted, left the cell, overlap
+    unsigned long long ctr[4];   // counters of a loaded snapshot (the slots hold the rest)
     double origin[3];
     unsigned int error;          // bit 0: a cell received more than 8 spheres
     unsigned int pad;

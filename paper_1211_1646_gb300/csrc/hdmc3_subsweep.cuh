@@ -1,10 +1,23 @@
 // hdmc3_subsweep.cuh -- the three-dimensional sub-sweep (Alg. 1 and Alg. 2
-// with eight checkerboard sets): one thread per active cell.  Before its
-// trials a thread gathers, into shared memory, the spheres of its 26
-// neighbour cells within reach of the box that holds all its trial positions;
-// no other sphere can overlap a trial position, so the decisions are those of
-// testing the whole neighbourhood, and every test keeps the arithmetic of the
-// serial form.
+// with eight checkerboard sets): a group of G lanes per active cell.  Each
+// lane keeps slots 0 and 1 of its share of the 26 neighbour cells in
+// registers, as packed binary32 pairs, and tests every trial position against
+// them; a vote of the group decides the trial.  The group's lanes draw the
+// trial directions together, one Philox block (binary64: three) per lane and
+// round, and the first round also draws the shuffle.  Third spheres of a cell
+// are rare (flagged per warp, read when present).
+//
+// What binds it: with few active cells the chain of one cell update (loads,
+// Philox, n_M dependent trials), which wide groups shorten; with many the
+// instructions (binary32: issue and the L1 wavefronts of the cell loads, 48 %
+// of peak) and in binary64 also the binary64 pipe, which has two instructions
+// per trial coordinate.  One thread per cell, which first gathered the
+// neighbours within reach of its trials into shared memory, took (us per
+// sub-sweep, n_M = 4, before -> now):
+//     216 active cells (N = 2048)       binary32 14.1 ->  6.2   binary64  46.3 ->  8.2
+//   2,197             (N = 16384)                14.4 ->  6.2             45.6 ->  9.2
+//  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
+// 132,651             (N = 1,048,576)            39.4 -> 37.1            165.3 -> 93.2
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -27,395 +40,567 @@ __device__ __forceinline__ bool inside_ball(const uint32_t (&w)[6]) {
     return (u0 * u0 + u1 * u1) + u2 * u2 < 1.0;
 }
 
-// Trial directions of one cell update, uniform in the unit ball by
-// rejection from (-1,1)^3.
-//   binary64: consecutive words of the trial stream, six per attempt,
-//             three sym52 variates;
+constexpr float kFar3 = -1.0e18f;   // stands for no sphere: farther than any cell
+
+// Precision-specific parts of a cell update.
+//
+// Trial directions, uniform in the unit ball by rejection from (-1,1)^3:
+//   binary64: consecutive words of the trial stream, six per attempt, three
+//             sym52 variates u = m 2^-52 (m odd, |m| < 2^52); a lane takes
+//             three Philox blocks, two attempts.  A variate is kept as the
+//             binary64 with the sign of m and the magnitude 2^52 + |m|, put
+//             together from its bits, and d u is RN(d u) =
+//             fma(d 2^-52, 2^52 + |m|, -d), with the sign of m: the product
+//             is exactly d + d |m| 2^-52, so one instruction of the slow
+//             binary64 pipe gives the correctly rounded product.
 //   binary32: each Philox block of the trial stream cut into six 21-bit
 //             fields, two attempts of three sym21 variates per block, kept
-//             when fma(u, u, fma(v, v, s*s)) < 1.
-template <typename T> struct TrialDir;
-template <> struct TrialDir<double> {
-    WordStream ws;
-    __device__ TrialDir(const G3& g, uint32_t sweep, uint32_t c, uint32_t dom) : ws(g.key0, g.key1, sweep, c, dom) {}
-    // The next `want` kept directions into column threadIdx.x of u, with the
-    // lanes that still need one drawing their attempts together (from a
-    // common start they stay at the same word of their streams, so the
-    // Philox blocks are computed converged).
-    __device__ __forceinline__ void fill(int want, double (*u)[3][kSubB3]) {
-        for (int have = 0; have < want;) {
-            uint32_t wd[6];
+//             when fma(u, u, fma(v, v, s*s)) < 1; a lane takes one block.
+//
+// Overlap test of a trial position with two slots at once, on binary32
+// coordinates.  binary32: the method's own test.  binary64: the coordinates
+// are truncated copies and r^2 is estimated; every difference is within
+// 6e-7 sigma of the binary64 one (truncations 2 x 1.7e-7, the offset's and
+// the sums' roundings 2.6e-7, coordinates below 1.42 sigma), r^2 near
+// contact within 2.4e-6 sigma^2, and the band of 2^-16 sigma^2 on either side
+// is decided in binary64.
+template <typename T> struct Sub3;
+
+template <> struct Sub3<float> {
+    static constexpr bool kExact = true;   // the pair test decides
+    struct Draw {
+        float u[2][3];
+        bool keep[2];
+    };
+    static __device__ __forceinline__ uint32_t attempts(const G3& g, uint32_t sweep, uint32_t c, uint32_t dom,
+                                                        uint32_t lane_block, Draw& d) {
+        uint32_t f[6];
+        const uint4 r = philox4x32_10(make_uint4(sweep, c, dom, lane_block), g.key0, g.key1);
+        fields21(r, f);
 #pragma unroll
-            for (int q = 0; q < 6; ++q) wd[q] = ws.next();
-            if (inside_ball(wd)) {
-                u[have][0][threadIdx.x] = sym52(wd[0], wd[1]);
-                u[have][1][threadIdx.x] = sym52(wd[2], wd[3]);
-                u[have][2][threadIdx.x] = sym52(wd[4], wd[5]);
-                ++have;
-            }
-        }
-    }
-};
-template <> struct TrialDir<float> {
-    uint32_t k0, k1, sweep, c, dom, block;
-    uint32_t f[6];
-    int triple;
-    __device__ TrialDir(const G3& g, uint32_t sweep_, uint32_t c_, uint32_t dom_)
-        : k0(g.key0), k1(g.key1), sweep(sweep_), c(c_), dom(dom_), block(0), triple(2) {}
-    // The next `want` kept directions (attempts in stream order: the field
-    // triples (0,1,2) and (3,4,5) of block 0, then of block 1, ...) into
-    // column threadIdx.x of u.  Lanes that still need a direction compute
-    // their next Philox block together, so the generator runs with the warp
-    // converged, not once for every lane that happens to need a block in a
-    // given trial.
-    __device__ __forceinline__ void fill(int want, float (*u)[3][kSubB3]) {
-        int have = 0;
-        for (;;) {
+        for (int a = 0; a < 2; ++a) {
 #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                if (triple == a && have < want) {
-                    const float u0 = sym21(f[3 * a]), u1 = sym21(f[3 * a + 1]), u2 = sym21(f[3 * a + 2]);
-                    ++triple;
-                    if (fmaf(u0, u0, fmaf(u1, u1, u2 * u2)) < 1.0f) {
-                        u[have][0][threadIdx.x] = u0;
-                        u[have][1][threadIdx.x] = u1;
-                        u[have][2][threadIdx.x] = u2;
-                        ++have;
-                    }
-                }
-            }
-            if (have >= want) break;
-            fields21(philox4x32_10(make_uint4(sweep, c, dom, block), k0, k1), f);
-            ++block;
-            triple = 0;
+            for (int q = 0; q < 3; ++q) d.u[a][q] = sym21(f[3 * a + q]);
+            d.keep[a] = fmaf(d.u[a][0], d.u[a][0], fmaf(d.u[a][1], d.u[a][1], d.u[a][2] * d.u[a][2])) < 1.0f;
         }
+        return r.x;
     }
+    static __device__ __forceinline__ float trial(const G3& g, float x, float u) { return fmaf(g.df, u, x); }
+    static __device__ __forceinline__ bool inside(float p, float w) { return p >= 0.0f && p < w; }
+    static __device__ __forceinline__ float est(float v) { return v; }
+    static __device__ __forceinline__ float est_or_far(float v) { return v; }   // an empty slot's sentinel is far away
 };
 
-// Trial directions drawn ahead per thread (shared memory).
-constexpr int kDir3 = 4;
-template <typename T> struct DirBuf { T u[kDir3][3][kSubB3]; };
+template <> struct Sub3<double> {
+    static constexpr bool kExact = false;
+    struct Draw {
+        double u[2][3];
+        bool keep[2];
+    };
+    static __device__ __forceinline__ double variate(uint32_t hi, uint32_t lo) {
+        const long long m = (long long)(2 * ((((unsigned long long)hi << 32) | lo) >> 12) + 1) - (1ll << 52);
+        const unsigned long long a = (unsigned long long)(m < 0 ? -m : m);
+        return __longlong_as_double((long long)(a | 0x4330000000000000ull | ((unsigned long long)m & 0x8000000000000000ull)));
+    }
+    static __device__ __forceinline__ uint32_t attempts(const G3& g, uint32_t sweep, uint32_t c, uint32_t dom,
+                                                        uint32_t lane_block, Draw& d) {
+        uint32_t w[12];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const uint4 r = philox4x32_10(make_uint4(sweep, c, dom, 3 * lane_block + b), g.key0, g.key1);
+            w[4 * b] = r.x;
+            w[4 * b + 1] = r.y;
+            w[4 * b + 2] = r.z;
+            w[4 * b + 3] = r.w;
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const uint32_t v[6] = {w[6 * a], w[6 * a + 1], w[6 * a + 2], w[6 * a + 3], w[6 * a + 4], w[6 * a + 5]};
+            d.keep[a] = inside_ball(v);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) d.u[a][q] = variate(v[2 * q], v[2 * q + 1]);
+        }
+        return w[0];
+    }
+    static __device__ __forceinline__ double trial(const G3& g, double x, double v) {
+        const double c = __longlong_as_double(__double_as_longlong(g.d) ^
+                                              ((__double_as_longlong(v) & (1ll << 63)) ^ (1ll << 63)));   // -d with v's sign
+        return __dadd_rn(x, __fma_rn(g.d52, v, c));
+    }
+    static __device__ __forceinline__ bool inside(double p, double w) {
+        return Prm<double>::ge0(p) && Prm<double>::lt(p, w);
+    }
+    static __device__ __forceinline__ float est(double v) { return approx_f32(v); }
+    static __device__ __forceinline__ float est_or_far(double v) { return v == kEmpty ? kFar3 : approx_f32(v); }
+};
 
-// Pair test on binary32 copies of the coordinates: 1 overlap, 0 none, 2 too
-// close to contact for binary32 to decide (binary64 only; the copies are
-// within 3e-7 of the binary64 values, so r^2 is within 1e-5 of the binary64
-// one, well inside the 2^-14 sigma^2 band).  In binary32 mode the copies are
-// the coordinates and this is the method's own test.
+// Slots 0 and 1 of a cell, moved by (sx, sy, sz), as packed pairs, and
+// whether slot 2 is occupied.  Slots 2 and 3 likewise (OFF = 2).
+struct Pair3 {
+    f2x x, y, z;
+};
 template <typename T>
-__device__ __forceinline__ int quick_hit(const G3& g, float dx, float dy, float dz);
-template <>
-__device__ __forceinline__ int quick_hit<float>(const G3& g, float dx, float dy, float dz) {
-    return fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -g.sig2f))) < 0.0f;
+__device__ __forceinline__ void ld2(const T* p, T& a, T& b);
+template <> __device__ __forceinline__ void ld2(const float* p, float& a, float& b) {
+    const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+    a = v.x;
+    b = v.y;
 }
-template <>
-__device__ __forceinline__ int quick_hit<double>(const G3& g, float dx, float dy, float dz) {
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    return r2 < g.band_lo ? 1 : (r2 > g.band_hi ? 0 : 2);
+template <> __device__ __forceinline__ void ld2(const double* p, double& a, double& b) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    a = v.x;
+    b = v.y;
+}
+template <typename T>
+__device__ __forceinline__ Pair3 pair_at(const T* p, float sx, float sy, float sz, T& x2) {
+    T x0, x1, y0, y1, z0, z1;
+    if constexpr (sizeof(T) == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+        x0 = v.x;
+        x1 = v.y;
+        x2 = v.z;
+    } else {
+        ld2(p, x0, x1);
+        x2 = __ldg(p + 2);
+    }
+    ld2(p + 4, y0, y1);
+    ld2(p + 8, z0, z1);
+    Pair3 r;
+    r.x = add2(pk(Sub3<T>::est_or_far(x0), Sub3<T>::est_or_far(x1)), pk(sx, sx));
+    r.y = add2(pk(Sub3<T>::est(y0), Sub3<T>::est(y1)), pk(sy, sy));
+    r.z = add2(pk(Sub3<T>::est(z0), Sub3<T>::est(z1)), pk(sz, sz));
+    return r;
 }
 
-// Exact test of the trial position against every sphere of the neighbour
-// cell with storage index sn (its offset from the cell (cx,cy,cz) is
-// recovered from the grid: m >= 4 makes it unique).
 template <typename T>
-__device__ bool cell_hit_exact(const G3& g, const T* cells, unsigned sn, int cx, int cy, int cz, T px, T py, T pz) {
+__device__ __forceinline__ Pair3 pair23_at(const T* p, float sx, float sy, float sz) {
+    T x0, x1, y0, y1, z0, z1;
+    ld2(p + 2, x0, x1);
+    ld2(p + 6, y0, y1);
+    ld2(p + 10, z0, z1);
+    Pair3 r;
+    r.x = add2(pk(Sub3<T>::est_or_far(x0), Sub3<T>::est_or_far(x1)), pk(sx, sx));
+    r.y = add2(pk(Sub3<T>::est(y0), Sub3<T>::est(y1)), pk(sy, sy));
+    r.z = add2(pk(Sub3<T>::est(z0), Sub3<T>::est(z1)), pk(sz, sz));
+    return r;
+}
+
+// fma(dx, dx, fma(dy, dy, fma(dz, dz, ns2))) for both slots of a pair.
+__device__ __forceinline__ f2x ztriple(const Pair3& q, f2x px, f2x py, f2x pz, f2x ns2) {
+    const f2x dx = sub2(px, q.x), dy = sub2(py, q.y), dz = sub2(pz, q.z);
+    return fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, ns2)));
+}
+
+// Where a cell's neighbours are: the storage index of the neighbour at offset
+// (dx, dy, dz) is x[dx + 1] + y[dy + 1] + z[dz + 1] (the set number and the
+// half-grid position both separate by axis; periodic).
+struct Axes3 {
+    unsigned x[3], y[3], z[3];
+    __device__ __forceinline__ static void axis(int i, int q, int h, unsigned stride, unsigned set, unsigned (&v)[3]) {
+        int lo = i - 1 + q, hi = i + q;
+        lo = lo < 0 ? h - 1 : lo;
+        hi = hi >= h ? 0 : hi;
+        v[0] = (unsigned)lo * stride + (unsigned)(q ^ 1) * set;
+        v[1] = (unsigned)i * stride + (unsigned)q * set;
+        v[2] = (unsigned)hi * stride + (unsigned)(q ^ 1) * set;
+    }
+    __device__ __forceinline__ Axes3(const G3& g, int Q, int ix, int iy, int iz) {
+        axis(ix, Q & 1, g.h[0], 1u, g.cq, x);
+        axis(iy, (Q >> 1) & 1, g.h[1], (unsigned)g.h[0], 2u * g.cq, y);
+        axis(iz, Q >> 2, g.h[2], (unsigned)g.h[0] * (unsigned)g.h[1], 4u * g.cq, z);
+    }
+    // Neighbours 0..25: 3 row + (dx + 1) for the eight x-rows (dy, dz) != (0, 0)
+    // in the order (dz, dy), then dx = -1 and dx = 1 of the cell's own row.
+    __device__ __forceinline__ unsigned at(const G3& g, int num, int& dx, int& dy, int& dz) const {
+        int row = (num * 11) >> 5;   // num / 3 for num < 32
+        dx = num >= 24 ? 2 * (num - 24) : num - 3 * row;
+        row = num >= 24 ? 4 : row + (row >= 4);   // 4: the own row
+        dz = (row * 11) >> 5;
+        dy = row - 3 * dz;
+        const unsigned i = (dx == 0 ? x[0] : dx == 1 ? x[1] : x[2]) + (dy == 0 ? y[0] : dy == 1 ? y[1] : y[2]) +
+                           (dz == 0 ? z[0] : dz == 1 ? z[1] : z[2]);
+        --dx;
+        --dy;
+        --dz;
+        return (unsigned)checked_cell(g.check, i, g.C);
+    }
+};
+
+// The method's test of the trial position against slots first..last of one
+// neighbour cell, up to its first empty slot.
+template <typename T>
+__device__ __forceinline__ bool slots_hit(const G3& g, const T* cells, unsigned sn, int dx, int dy, int dz, int first, int last,
+                                          const T* p) {
     using A = Ar3<T>;
-    const unsigned Q = sn / g.cq, r0 = sn % g.cq;
-    const int ix = (int)(r0 % (unsigned)g.h[0]);
-    const unsigned r1 = r0 / (unsigned)g.h[0];
-    const int iy = (int)(r1 % (unsigned)g.h[1]), iz = (int)(r1 / (unsigned)g.h[1]);
-    int dd[3] = {2 * ix + (int)(Q & 1) - cx, 2 * iy + (int)((Q >> 1) & 1) - cy, 2 * iz + (int)(Q >> 2) - cz};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) dd[a] = dd[a] > 1 ? dd[a] - g.m[a] : (dd[a] < -1 ? dd[a] + g.m[a] : dd[a]);
-    const T sx = (T)dd[0] * A::w(g, 0), sy = (T)dd[1] * A::w(g, 1), sz = (T)dd[2] * A::w(g, 2);
+    const T sx = (T)dx * A::w(g, 0), sy = (T)dy * A::w(g, 1), sz = (T)dz * A::w(g, 2);
     bool hit = false;
-    for (int j = 0; j < kSlots3; ++j) {
+    for (int j = first; j <= last; ++j) {
         const T* q = slot3(cells, g, sn, j);
         if (q[0] == (T)kEmpty) break;
-        hit |= A::hit(g, px - (q[0] + sx), py - (q[4] + sy), pz - (q[8] + sz));
+        hit |= A::hit(g, p[0] - (q[0] + sx), p[1] - (q[4] + sy), p[2] - (q[8] + sz));
     }
     return hit;
 }
 
-// Does the trial position hit a sphere of the 26 neighbour cells?  Reads
-// global memory (used when a cell has more than kCand3 gathered spheres).
-template <typename T>
-__device__ bool neighbour_hit_global(const G3& g, const T* cells, int cx, int cy, int cz, T px, T py, T pz) {
-    using A = Ar3<T>;
-    bool hit = false;
-    for (int dz = -1; dz <= 1; ++dz)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                if (dx == 0 && dy == 0 && dz == 0) continue;
-                const unsigned sn = sidx3(g, wrap3(cx + dx, g.m[0]), wrap3(cy + dy, g.m[1]), wrap3(cz + dz, g.m[2]));
-                const T sx = (T)dx * A::w(g, 0), sy = (T)dy * A::w(g, 1), sz = (T)dz * A::w(g, 2);
-                for (int j = 0; j < kSlots3; ++j) {
-                    const T* q = slot3(cells, g, sn, j);
-                    if (q[0] == (T)kEmpty) break;
-                    const T ex = q[0] + sx, ey = q[4] + sy, ez = q[8] + sz;
-                    hit |= A::hit(g, px - ex, py - ey, pz - ez);
-                }
-            }
-    return hit;
-}
+constexpr int kSubB3 = 32;     // threads of a sub-sweep block: one warp, no block barrier (blocks of 4 warps: 41.0 us)
+constexpr int kDir3 = 8;       // trial directions drawn ahead per cell
 
-// Per-thread candidate lists in shared memory, column t for thread t:
-// binary32 keeps the three coordinates (12 bytes a candidate); binary64 adds
-// the neighbour cell's storage index for the exact test near contact.
-template <typename T> struct Cand;
-template <> struct Cand<float> {
-    float x[kCand3][kSubB3], y[kCand3][kSubB3], z[kCand3][kSubB3];
-    __device__ __forceinline__ void put(int q, float a, float b, float c, unsigned) {
-        x[q][threadIdx.x] = a;
-        y[q][threadIdx.x] = b;
-        z[q][threadIdx.x] = c;
-    }
-    __device__ __forceinline__ float4 get(int q) const {
-        return make_float4(x[q][threadIdx.x], y[q][threadIdx.x], z[q][threadIdx.x], 0.0f);
-    }
+// Shared memory of one warp's cells.
+template <typename T, int G> struct Warp3 {
+    static constexpr int kCells = 32 / G;
+    // kept directions, a ring: fewer than kDir3 left over, 2 G more per round
+    static constexpr int kRing = G <= 4 ? 16 : G <= 8 ? 32 : G <= 16 ? 64 : 128;
+    static_assert(kRing >= kDir3 - 1 + 2 * G, "direction ring");
+    T dir[kCells][kRing][3];
+    T own[kCells][kSlots3][3];   // own spheres, slot order before the shuffle
+    T trial[kCells][4];          // the current trial position
 };
-template <> struct Cand<double> {
-    float4 v[kCand3][kSubB3];
-    __device__ __forceinline__ void put(int q, float a, float b, float c, unsigned sn) {
-        v[q][threadIdx.x] = make_float4(a, b, c, __uint_as_float(sn));
-    }
-    __device__ __forceinline__ float4 get(int q) const { return v[q][threadIdx.x]; }
-};
-
-// Gather the occupied slots of one half of a neighbour cell (offset
-// dx,dy,dz, storage index sn) that lie within reach of the box [lo, hi] that
-// holds every trial position of this cell update: their binary32 image
-// coordinates (and sn in binary64) go to the thread's candidate list.
-template <typename T>
-__device__ __forceinline__ void gather_half(const G3& g, const T (&qx)[4], const T (&qy)[4], const T (&qz)[4],
-                                            int dx, int dy, int dz, unsigned sn, const float (&lo)[3],
-                                            const float (&hi)[3], Cand<T>& cand, int& nc) {
-    const float sx = (float)dx * g.wf[0], sy = (float)dy * g.wf[1], sz = (float)dz * g.wf[2];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if constexpr (sizeof(T) == 4) {
-            // without branches: an empty slot's sentinel lies far outside the
-            // reach of any box, and a candidate that is not kept is
-            // overwritten by the next one (3 % faster than the branches)
-            const float ex = qx[j] + sx, ey = qy[j] + sy, ez = qz[j] + sz;
-            const float gx = fmaxf(fmaxf(lo[0] - ex, ex - hi[0]), 0.0f);
-            const float gy = fmaxf(fmaxf(lo[1] - ey, ey - hi[1]), 0.0f);
-            const float gz = fmaxf(fmaxf(lo[2] - ez, ez - hi[2]), 0.0f);
-            const bool keep = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < g.keep2f;
-            if (nc < kCand3) cand.put(nc, ex, ey, ez, sn);
-            nc += keep;
-        } else if (qx[j] != (T)kEmpty) {   // binary64: convert only occupied slots
-            const float ex = (float)qx[j] + sx, ey = (float)qy[j] + sy, ez = (float)qz[j] + sz;
-            const float gx = fmaxf(fmaxf(lo[0] - ex, ex - hi[0]), 0.0f);
-            const float gy = fmaxf(fmaxf(lo[1] - ey, ey - hi[1]), 0.0f);
-            const float gz = fmaxf(fmaxf(lo[2] - ez, ez - hi[2]), 0.0f);
-            if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < g.keep2f) {
-                if (nc < kCand3) cand.put(nc, ex, ey, ez, sn);
-                ++nc;
-            }
-        }
-    }
-}
-
-// Both halves of a neighbour cell whose primary half is already loaded.
-template <typename T>
-__device__ __forceinline__ void gather_cell(const G3& g, const T* cells, const T (&qx)[4], const T (&qy)[4],
-                                            const T (&qz)[4], int dx, int dy, int dz, unsigned sn,
-                                            const float (&lo)[3], const float (&hi)[3], Cand<T>& cand, int& nc) {
-    gather_half(g, qx, qy, qz, dx, dy, dz, sn, lo, hi, cand, nc);
-    if (qx[3] != (T)kEmpty) {
-        const T* p = cells + secondary3(g, sn);
-        T rx[4], ry[4], rz[4];
-        ld4(p, rx);
-        ld4(p + 4, ry);
-        ld4(p + 8, rz);
-        gather_half(g, rx, ry, rz, dx, dy, dz, sn, lo, hi, cand, nc);
-    }
-}
 
 // One sub-sweep: every cell of set Q = table[jd].perm[k] (Alg. 1, Alg. 2).
-// binary32: the neighbour cells of one x-row are loaded together (256-bit
-// loads) before they are scanned; binary64: one cell at a time.
-template <typename T>
+template <typename T, int G>
 __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, const Draw3* __restrict__ table, int jd,
-                                           int k, Dev3* st) {
+                                           int k, unsigned long long* __restrict__ ctr) {
+    using S = Sub3<T>;
     using A = Ar3<T>;
-    __shared__ Cand<T> cand;
-    __shared__ DirBuf<T> dirs;
+    using W = Warp3<T, G>;
+    constexpr int NC = G <= 8 ? 24 / G + 1 : 1;    // neighbour cells of a lane
+    static_assert(G == 2 || G == 4 || G == 8 || G == 32, "lanes per cell");
+    constexpr unsigned kFull = 0xFFFFFFFFu;
+    __shared__ W warps[kSubB3 / 32];
+    W& sw = warps[threadIdx.x / 32];
+    const int lane = threadIdx.x & 31, grp = lane / G, L = lane % G, gb = grp * G;
+    const unsigned gm = (G == 32 ? kFull : ((1u << G) - 1u) << gb);   // lanes of my group
+    const unsigned below = gm & ((1u << lane) - 1u);                    // those before me
     const Draw3& dr = table[jd];
     const int Q = dr.perm[k];
-    const unsigned s = blockIdx.x * kSubB3 + threadIdx.x;
-    uint32_t n_tr = 0, n_ac = 0, n_lf = 0, n_ov = 0;
-    if (s < g.cq) {
-        const int ix = (int)(s % (unsigned)g.h[0]);
-        const unsigned r = s / (unsigned)g.h[0];
-        const int iy = (int)(r % (unsigned)g.h[1]);
-        const int iz = (int)(r / (unsigned)g.h[1]);
-        const int cx = 2 * ix + (Q & 1), cy = 2 * iy + ((Q >> 1) & 1), cz = 2 * iz + (Q >> 2);
-        const unsigned sown = (unsigned)Q * g.cq + s;
-        T x[8], y[8], z[8];
-        ld_cell3(cells, g, sown, x, y, z);
-        int n = 0;
+    const uint32_t sweep = dr.sweep;
+    const unsigned s = (blockIdx.x * (kSubB3 / 32) + threadIdx.x / 32) * W::kCells + grp;
+    const bool live = s < g.cq;
+    const unsigned r1 = g.div0(s), ix = s - r1 * (unsigned)g.h[0];
+    const unsigned iz = g.div1(r1), iy = r1 - iz * (unsigned)g.h[1];
+    const Axes3 ax(g, Q, (int)ix, (int)iy, (int)iz);
+    const int cx = 2 * (int)ix + (Q & 1), cy = 2 * (int)iy + ((Q >> 1) & 1), cz = 2 * (int)iz + (Q >> 2);
+    const uint32_t c = ((uint32_t)cz * (uint32_t)g.m[1] + (uint32_t)cy) * (uint32_t)g.m[0] + (uint32_t)cx;
+    const unsigned sown = (unsigned)checked_cell(g.check, live ? ax.x[1] + ax.y[1] + ax.z[1] : 0u, g.C);
+
+    // own spheres: the primary half's slots L, L + G
+    constexpr int NO = G < 4 ? 4 / G : 1;
+    T own[NO][3];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) n += x[j] != (T)kEmpty;
-        if (n > 0) {
-            const uint32_t c = ((uint32_t)cz * (uint32_t)g.m[1] + (uint32_t)cy) * (uint32_t)g.m[0] + (uint32_t)cx;
-            const uint32_t setbits = (uint32_t)Q << 24;
-            if (n >= 2 && !(g.flags & kNoParticleShuffle)) {
-                WordStream S(g.key0, g.key1, dr.sweep, c, (kDomShuffle << 28) | setbits);
-                shuffle3(x, y, z, n, S.bounded(factorial8(n)));
-            }
-            // Every trial position lies in the box [lo, hi]: a sphere makes at
-            // most K = ceil(n_M / n) trials, each moving it by less than d per
-            // axis from where the previous accepted one left it, and positions
-            // outside [0, w) are rejected before any overlap test.
-            float lo[3], hi[3];
-            {
-                const int K = (g.nsel + n - 1) / n;
-                const float reach = (float)K * g.df * (1.0f + 1.0e-5f) + 1.0e-6f;
-                float mn[3] = {3.0e38f, 3.0e38f, 3.0e38f}, mx[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (j < n) {
-                        const float v[3] = {(float)x[j], (float)y[j], (float)z[j]};
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            mn[a] = fminf(mn[a], v[a]);
-                            mx[a] = fmaxf(mx[a], v[a]);
-                        }
-                    }
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    lo[a] = fmaxf(0.0f, mn[a] - reach);
-                    hi[a] = fminf(g.wf[a], mx[a] + reach);
-                }
-            }
-            int nc = 0;
-#pragma unroll 1
-            for (int row = 0; row < 9; ++row) {
-                const int dz = row / 3 - 1, dy = row % 3 - 1;
-                const int ny = wrap3(cy + dy, g.m[1]), nz = wrap3(cz + dz, g.m[2]);
-                if (sizeof(T) == 4) {
-                    T ax[3][4], ay[3][4], az[3][4];
-                    unsigned sn[3];
-#pragma unroll
-                    for (int e = 0; e < 3; ++e) {
-                        sn[e] = sidx3(g, wrap3(cx + e - 1, g.m[0]), ny, nz);
-                        const T* p = cells + primary3(sn[e]);
-                        ld4(p, ax[e]);
-                        ld4(p + 4, ay[e]);
-                        ld4(p + 8, az[e]);
-                    }
-#pragma unroll
-                    for (int e = 0; e < 3; ++e)
-                        if (e != 1 || row != 4)
-                            gather_cell(g, cells, ax[e], ay[e], az[e], e - 1, dy, dz, sn[e], lo, hi, cand, nc);
-                } else {
-#pragma unroll 1
-                    for (int e = 0; e < 3; ++e) {
-                        if (e == 1 && row == 4) continue;
-                        const unsigned sn = sidx3(g, wrap3(cx + e - 1, g.m[0]), ny, nz);
-                        const T* p = cells + primary3(sn);
-                        T ax[4], ay[4], az[4];
-                        ld4(p, ax);
-                        ld4(p + 4, ay);
-                        ld4(p + 8, az);
-                        gather_cell(g, cells, ax, ay, az, e - 1, dy, dz, sn, lo, hi, cand, nc);
-                    }
-                }
-            }
-            const bool spill = nc > kCand3;
-            float fx[8], fy[8], fz[8];   // binary32 copies of the own coordinates
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                fx[j] = (float)x[j];
-                fy[j] = (float)y[j];
-                fz[j] = (float)z[j];
-            }
-            const T w0 = A::w(g, 0), w1 = A::w(g, 1), w2 = A::w(g, 2);
-            TrialDir<T> TD(g, dr.sweep, c, (kDomTrial << 28) | setbits);
-            int i = 0;
-            for (int t = 0; t < g.nsel; ++t) {
-                T u0, u1, u2;
-                {   // drawn ahead, kDir3 at a time
-                    const int tt = t % kDir3;
-                    if (tt == 0) TD.fill(min(kDir3, g.nsel - t), dirs.u);
-                    u0 = dirs.u[tt][0][threadIdx.x];
-                    u1 = dirs.u[tt][1][threadIdx.x];
-                    u2 = dirs.u[tt][2][threadIdx.x];
-                }
-                const T px = A::trial(g, pick8(x, i), u0);
-                const T py = A::trial(g, pick8(y, i), u1);
-                const T pz = A::trial(g, pick8(z, i), u2);
-                ++n_tr;
-                if (!(px >= (T)0 && px < w0 && py >= (T)0 && py < w1 && pz >= (T)0 && pz < w2)) {
-                    ++n_lf;
-                } else {
-                    const float pfx = (float)px, pfy = (float)py, pfz = (float)pz;
-                    bool hit = false;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (j < n && j != i) {
-                            int h = quick_hit<T>(g, pfx - fx[j], pfy - fy[j], pfz - fz[j]);
-                            if (h == 2) h = A::hit(g, px - x[j], py - y[j], pz - z[j]);
-                            hit |= h != 0;
-                        }
-                    if (!spill) {
-                        int q = 0;
-                        for (; q + 1 < nc && !hit; q += 2) {
-                            const float4 e0 = cand.get(q), e1 = cand.get(q + 1);
-                            int h0 = quick_hit<T>(g, pfx - e0.x, pfy - e0.y, pfz - e0.z);
-                            int h1 = quick_hit<T>(g, pfx - e1.x, pfy - e1.y, pfz - e1.z);
-                            if (h0 == 2) h0 = cell_hit_exact(g, cells, __float_as_uint(e0.w), cx, cy, cz, px, py, pz);
-                            if (h1 == 2) h1 = cell_hit_exact(g, cells, __float_as_uint(e1.w), cx, cy, cz, px, py, pz);
-                            hit = (h0 | h1) != 0;
-                        }
-                        if (q < nc && !hit) {
-                            const float4 e = cand.get(q);
-                            int h = quick_hit<T>(g, pfx - e.x, pfy - e.y, pfz - e.z);
-                            if (h == 2) h = cell_hit_exact(g, cells, __float_as_uint(e.w), cx, cy, cz, px, py, pz);
-                            hit = h != 0;
-                        }
-                    } else if (!hit) {
-                        hit = neighbour_hit_global(g, cells, cx, cy, cz, px, py, pz);
-                    }
-                    if (hit) {
-                        ++n_ov;
-                    } else {
-                        put8(x, i, px);
-                        put8(y, i, py);
-                        put8(z, i, pz);
-                        put8(fx, i, pfx);
-                        put8(fy, i, pfy);
-                        put8(fz, i, pfz);
-                        ++n_ac;
-                    }
-                }
-                i = i + 1 == n ? 0 : i + 1;
-            }
-            st_cell3(cells, g, sown, x, y, z, n > 4);
+    for (int r = 0; r < NO; ++r) {
+        own[r][0] = (T)kEmpty;
+        own[r][1] = own[r][2] = (T)0;
+        if (live && L + r * G < 4) {
+            const T* p = cells + primary3(sown) + (L + r * G);
+            own[r][0] = p[0];
+            own[r][1] = p[4];
+            own[r][2] = p[8];
         }
     }
-    const unsigned a = __reduce_add_sync(0xFFFFFFFFu, n_tr), b = __reduce_add_sync(0xFFFFFFFFu, n_ac);
-    const unsigned cc = __reduce_add_sync(0xFFFFFFFFu, n_lf), d = __reduce_add_sync(0xFFFFFFFFu, n_ov);
-    if ((threadIdx.x & 31) == 0 && a) {
-        atomicAdd(&st->ctr[0], (unsigned long long)a);
-        atomicAdd(&st->ctr[1], (unsigned long long)b);
-        atomicAdd(&st->ctr[2], (unsigned long long)cc);
-        atomicAdd(&st->ctr[3], (unsigned long long)d);
+    // my neighbour cells: slots 0 and 1 in registers; has2: bit c set when
+    // the c-th of them has a third sphere
+    Pair3 nb[NC];
+    unsigned has2 = 0;
+    // the number (Axes3::at) of my j-th neighbour: whole x-rows, then one of the own row
+    auto number = [&](int j) { return G > 8 ? j * G + L : j < 3 * (8 / G) ? 3 * (L + (j / 3) * G) + j % 3 : 24 + L; };
+    auto neighbour = [&](int j, unsigned sn, float sx, float sy, float sz) {
+        T x2;
+        nb[j] = pair_at(cells + primary3(sn), sx, sy, sz, x2);
+        has2 |= x2 != (T)kEmpty ? 1u << j : 0u;
+    };
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        nb[j].x = pk(kFar3, kFar3);
+        nb[j].y = nb[j].z = 0;
+    }
+    if (live) {
+        if constexpr (G <= 8) {
+#pragma unroll
+            for (int r = 0; r < 8 / G; ++r) {
+                const int num = 3 * (L + r * G);
+                int dx, dy, dz;
+                const unsigned row = ax.at(g, num, dx, dy, dz) - ax.x[0];
+                const float sy = (float)dy * g.wf[1], sz = (float)dz * g.wf[2];
+#pragma unroll
+                for (int e = 0; e < 3; ++e)
+                    neighbour(3 * r + e, (unsigned)checked_cell(g.check, row + ax.x[e], g.C), (float)(e - 1) * g.wf[0], sy, sz);
+            }
+            if (L < 2) {
+                int dx, dy, dz;
+                const unsigned sn = ax.at(g, 24 + L, dx, dy, dz);
+                neighbour(NC - 1, sn, (float)dx * g.wf[0], 0.0f, 0.0f);
+            }
+        } else if (L < 26) {
+            int dx, dy, dz;
+            const unsigned sn = ax.at(g, L, dx, dy, dz);
+            neighbour(0, sn, (float)dx * g.wf[0], (float)dy * g.wf[1], (float)dz * g.wf[2]);
+        }
+    }
+
+    // the first trial directions, while the loads are under way
+    const uint32_t setbits = (uint32_t)Q << 24;
+    unsigned have = 0, used = 0;   // directions kept so far, lane blocks used
+    auto keep = [&](bool need, const typename S::Draw& d) {
+        const bool k0 = need && d.keep[0], k1 = need && d.keep[1];
+        const unsigned b0 = __ballot_sync(kFull, k0), b1 = __ballot_sync(kFull, k1);
+        const unsigned pos = have + __popc(b0 & below) + __popc(b1 & below);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            if (k0) sw.dir[grp][pos % W::kRing][q] = d.u[0][q];
+            if (k1) sw.dir[grp][(pos + k0) % W::kRing][q] = d.u[1][q];
+        }
+        have += __popc(b0 & gm) + __popc(b1 & gm);
+    };
+    auto draw = [&](unsigned upto) {
+#pragma unroll 1
+        for (;;) {
+            const bool need = live && have < upto;
+            if (!__any_sync(kFull, need)) break;
+            typename S::Draw d;
+            S::attempts(g, sweep, c, (kDomTrial << 28) | setbits, used + L, d);
+            keep(need, d);
+            used += need ? G : 0;
+        }
+        __syncwarp();
+    };
+    // first round: the group's last lane draws the first word of the shuffle
+    // stream instead, the others the first G - 1 lane blocks
+    uint32_t word;
+    {
+        typename S::Draw d;
+        const bool last = L == G - 1;
+        word = S::attempts(g, sweep, c, ((last ? kDomShuffle : kDomTrial) << 28) | setbits, last ? 0u : (uint32_t)L, d);
+        keep(live && !last, d);
+        used = G - 1;
+        word = __shfl_sync(kFull, word, gb + G - 1);
+    }
+    draw((unsigned)min(kDir3, g.nsel));
+
+    // own cell: number of spheres, slots 4..7 when slot 3 is occupied
+    int n = 0;
+#pragma unroll
+    for (int r = 0; r < NO; ++r) {
+        n += __popc(__ballot_sync(kFull, own[r][0] != (T)kEmpty) & gm);
+        if (L + r * G < 4) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) sw.own[grp][L + r * G][q] = own[r][q];
+        }
+    }
+    if (__any_sync(kFull, n == 4)) {
+        int more4 = 0;
+        if (n == 4)
+            for (int j = L; j < 4; j += G) {
+                const T* p = cells + secondary3(g, sown) + j;
+                if (p[0] == (T)kEmpty) break;
+                sw.own[grp][4 + j][0] = p[0];
+                sw.own[grp][4 + j][1] = p[4];
+                sw.own[grp][4 + j][2] = p[8];
+                ++more4;
+            }
+#pragma unroll
+        for (int o = 1; o < (G < 4 ? G : 4); o <<= 1) more4 += __shfl_xor_sync(kFull, more4, o);
+        n += __shfl_sync(kFull, more4, gb);
+    }
+    // shuffle (Alg. 1): slot j of the shuffled cell is old slot (perm >> 4j) & 7
+    unsigned perm = 0x76543210u;
+    if (n >= 2 && !(g.flags & kNoParticleShuffle)) {
+        const uint32_t range = factorial8(n);
+        const unsigned long long m = (unsigned long long)word * range;
+        uint32_t kk = (uint32_t)(m >> 32);
+        if ((uint32_t)m < range) {   // as good as never: WordStream::bounded from the start
+            WordStream ws(g.key0, g.key1, sweep, c, (kDomShuffle << 28) | setbits);
+            kk = ws.bounded(range);
+        }
+#pragma unroll 1
+        for (int j = n - 1; j >= 3; --j) {   // swap slots j and kk mod (j+1)
+            const unsigned qt = kk / (uint32_t)(j + 1), r = kk - qt * (uint32_t)(j + 1);
+            kk = qt;
+            const unsigned x = ((perm >> (4 * j)) ^ (perm >> (4 * r))) & 7u;   // 0 when j == r
+            perm ^= (x << (4 * j)) ^ (x << (4 * r));
+        }
+        if (n >= 3) {   // kk < 6: slots 2 and kk mod 3
+            const unsigned r = kk >= 3u ? kk - 3u : kk;
+            kk = kk >= 3u ? 1u : 0u;
+            const unsigned x = ((perm >> 8) ^ (perm >> (4 * r))) & 7u;
+            perm ^= (x << 8) ^ (x << (4 * r));
+        }
+        if (kk == 0u) {   // kk < 2: slots 1 and kk
+            const unsigned x = ((perm >> 4) ^ perm) & 7u;
+            perm ^= (x << 4) ^ x;
+        }
+    }
+    // slots 2 and 3 of the first flagged neighbour cell; further flagged cells
+    // and slots 4..7 (rare) are read in the trial loop
+    Pair3 f23;
+    f23.x = pk(kFar3, kFar3);
+    f23.y = f23.z = 0;
+    const bool any23 = __any_sync(kFull, has2 != 0);
+    unsigned more = has2 & (has2 - 1u);   // bit 31: slots 4..7 of the first flagged cell may be occupied
+    if (has2) {
+        int dx, dy, dz;
+        const T* p = cells + primary3(ax.at(g, number(__ffs(has2) - 1), dx, dy, dz));
+        f23 = pair23_at(p, (float)dx * g.wf[0], (float)dy * g.wf[1], (float)dz * g.wf[2]);
+        more |= __ldg(p + 3) != (T)kEmpty ? 0x80000000u : 0u;
+    }
+    const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots3 && __any_sync(kFull, n > G);
+    __syncwarp();
+
+    // binary64: lane L computes trial coordinate L (two lanes: the first also coordinate 2)
+    const int a0 = L < 3 ? L : 0;
+    const T w0 = A::w(g, 0), w1 = A::w(g, 1), w2 = A::w(g, 2);
+    const T wa = a0 == 0 ? w0 : a0 == 1 ? w1 : w2;
+    const f2x lo2 = S::kExact ? pk(-g.sig2f, -g.sig2f) : pk(-g.band_lo, -g.band_lo);
+    const f2x band2 = pk(g.band_lo - g.band_hi, g.band_lo - g.band_hi);
+    unsigned n_ac = 0, n_lf = 0;
+    int i = 0;
+#pragma unroll 1
+    for (int t = 0; t < g.nsel; ++t) {
+        if (t > 0 && t % kDir3 == 0) draw((unsigned)min(t + kDir3, g.nsel));
+        const int cur = (int)((perm >> (4 * i)) & 7u);
+        T* const me = sw.own[grp][cur];
+        const T* const u = sw.dir[grp][(unsigned)t % W::kRing];
+        float px, py, pz;
+        bool inside;
+        if constexpr (S::kExact) {
+            px = S::trial(g, me[0], u[0]);
+            py = S::trial(g, me[1], u[1]);
+            pz = S::trial(g, me[2], u[2]);
+            inside = S::inside(px, w0) && S::inside(py, w1) && S::inside(pz, w2);
+        } else {
+            const T p = S::trial(g, me[a0], u[a0]);
+            bool in = S::inside(p, wa);
+            const float pf = S::est(p);
+            px = __shfl_sync(kFull, pf, gb);
+            py = __shfl_sync(kFull, pf, gb + 1);
+            if constexpr (G >= 4) {
+                pz = __shfl_sync(kFull, pf, gb + 2);
+            } else {
+                const T pc = S::trial(g, me[2], u[2]);
+                in = in && S::inside(pc, w2);
+                pz = S::est(pc);
+                if (L == 0) sw.trial[grp][2] = pc;
+            }
+            constexpr unsigned m3 = G >= 4 ? 7u : 3u;
+            inside = ((__ballot_sync(kFull, in) >> gb) & m3) == m3;
+            if (L < 3) sw.trial[grp][L] = p;
+            __syncwarp();
+        }
+        const f2x px2 = pk(px, px), py2 = pk(py, py), pz2 = pk(pz, pz);
+        uint32_t sure = 0, maybe = 0;   // sign bits: certainly / possibly overlapping
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const f2x z = ztriple(nb[j], px2, py2, pz2, lo2);
+            sure |= lo32(z) | hi32(z);
+            if (!S::kExact) {
+                const f2x y = add2(z, band2);
+                maybe |= lo32(y) | hi32(y);
+            }
+        }
+        if (any23) {
+            const f2x z = ztriple(f23, px2, py2, pz2, lo2);
+            sure |= lo32(z) | hi32(z);
+            if (!S::kExact) {
+                const f2x y = add2(z, band2);
+                maybe |= lo32(y) | hi32(y);
+            }
+        }
+        bool hit = (sure >> 31) != 0;
+        // own cell: the other spheres, one per lane
+        if (crowd) {
+            auto own_hit = [&](int j) {
+                const T* q = sw.own[grp][j];
+                if constexpr (S::kExact) {
+                    return A::hit(g, px - q[0], py - q[1], pz - q[2]);
+                } else {
+                    const float ex = px - S::est(q[0]), ey = py - S::est(q[1]), ez = pz - S::est(q[2]);
+                    const float r2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+                    if (r2 < g.band_lo || r2 > g.band_hi) return r2 < g.band_lo;
+                    const T* tp = sw.trial[grp];
+                    return A::hit(g, tp[0] - q[0], tp[1] - q[1], tp[2] - q[2]);
+                }
+            };
+            if (L < n && L != cur) hit |= own_hit(L);
+            if (crowdG)
+                for (int j = L + G; j < n; j += G)
+                    if (j != cur) hit |= own_hit(j);
+        }
+        if (!S::kExact && !hit && inside && (maybe >> 31)) {
+            // some slot is too close to contact for the estimates: decide those slots in binary64
+            unsigned close = 0;   // bits 2j, 2j+1: slots 0, 1 of neighbour j; bits 30, 31: the flagged pair
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const f2x y = add2(ztriple(nb[j], px2, py2, pz2, lo2), band2);
+                close |= ((lo32(y) >> 31) << (2 * j)) | ((hi32(y) >> 31) << (2 * j + 1));
+            }
+            const f2x y = add2(ztriple(f23, px2, py2, pz2, lo2), band2);
+            close |= ((lo32(y) >> 31) << 30) | (hi32(y) & 0x80000000u);
+            while (close) {
+                const int b = __ffs(close) - 1;
+                close &= close - 1u;
+                const int j = b >= 30 ? __ffs(has2) - 1 : b >> 1, slot = b >= 30 ? b - 28 : b & 1;
+                int dx, dy, dz;
+                const unsigned sn = ax.at(g, number(j), dx, dy, dz);
+                hit |= slots_hit(g, cells, sn, dx, dy, dz, slot, slot, sw.trial[grp]);
+            }
+        }
+        if (more && !hit && inside) {   // rare: slots 2..7 of further flagged cells, slots 4..7 of the first
+            for (unsigned m = more; m; m &= m - 1u) {
+                const int b = __ffs(m) - 1;
+                int dx, dy, dz;
+                const unsigned sn = ax.at(g, number(b == 31 ? __ffs(has2) - 1 : b), dx, dy, dz);
+                T tp[3];
+                if constexpr (S::kExact) {
+                    tp[0] = px;
+                    tp[1] = py;
+                    tp[2] = pz;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) tp[q] = sw.trial[grp][q];
+                }
+                hit |= slots_hit(g, cells, sn, dx, dy, dz, b == 31 ? 4 : 2, kSlots3 - 1, tp);
+            }
+        }
+        const bool overlap = (__ballot_sync(kFull, hit) & gm) != 0;
+        if (n > 0 && inside && !overlap) {
+            if (L == 0) {
+                if constexpr (S::kExact) {
+                    me[0] = px;
+                    me[1] = py;
+                    me[2] = pz;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) me[q] = sw.trial[grp][q];
+                }
+            }
+            ++n_ac;
+        }
+        n_lf += !inside;
+        __syncwarp();
+        i = i + 1 >= n ? 0 : i + 1;
+    }
+    // the shuffled slots back; unused slots keep their sentinels
+#pragma unroll 1
+    for (int j = L; j < n; j += G) {
+        const T* q = sw.own[grp][(perm >> (4 * j)) & 7u];
+        T* p = cells + (j < 4 ? primary3(sown) + j : secondary3(g, sown) + (j - 4));
+        p[0] = q[0];
+        p[4] = q[1];
+        p[8] = q[2];
+    }
+    // counters: one lane per cell
+    const bool count = L == 0 && n > 0;
+    const unsigned tr = __reduce_add_sync(kFull, count ? (unsigned)g.nsel : 0u);
+    const unsigned ac = __reduce_add_sync(kFull, count ? n_ac : 0u), lf = __reduce_add_sync(kFull, count ? n_lf : 0u);
+    if (lane < 4 && tr) {
+        const unsigned v = lane == 0 ? tr : lane == 1 ? ac : lane == 2 ? lf : tr - ac - lf;
+        atomicAdd(ctr + 4 * (blockIdx.x % kCtr3) + lane, (unsigned long long)v);
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSubB3) k_sub3(G3 g, T* __restrict__ cells, const Draw3* __restrict__ table, int jd,
-                                                 int k, Dev3* st) {
-    sub3_cells<T>(g, cells, table, jd, k, st);
-}
-// binary32: eight blocks per SM (128 registers; ten blocks at 96 registers
-// spill and measured slower, 46.8 against 41.5 us)
-template <>
-__global__ void __launch_bounds__(kSubB3, 8) k_sub3<float>(G3 g, float* __restrict__ cells,
-                                                            const Draw3* __restrict__ table, int jd, int k, Dev3* st) {
-    sub3_cells<float>(g, cells, table, jd, k, st);
+template <typename T, int G>
+__global__ void __launch_bounds__(kSubB3, G == 2 ? 12 : G == 4 ? 16 : G == 8 ? 20 : 24) k_sub3(const G3 g, T* __restrict__ cells, const Draw3* __restrict__ table, int jd,
+                                                 int k, unsigned long long* __restrict__ ctr) {
+    sub3_cells<T, G>(g, cells, table, jd, k, ctr);
 }
 
 }  // namespace hdmc
