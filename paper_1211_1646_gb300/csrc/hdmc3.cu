@@ -24,6 +24,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <utility>
 #include <vector>
 
 #include "hdmc.h"
@@ -38,9 +40,17 @@ void bin_axis(double x, double w, int m, int& cell, double& loc);
 double poly_intercept(const std::vector<double>& t, const std::vector<double>& y, int deg);
 void squared_edges(double sigma, double* E);
 
-// Sweep or shift draws for `count` consecutive indices starting at `first`.
-__global__ void k_draws3(G3 g, Draw3* table, uint32_t first, int count, int sweep_mode) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Sweep or shift draws for `count` consecutive indices (one block).  Shifts
+// start at `first`; sweeps start at *next, which is advanced, so that a
+// recorded graph of many sweeps can be replayed unchanged.
+__global__ void __launch_bounds__(kDrawChunk3) k_draws3(const G3 g, Draw3* table, uint32_t first, uint32_t* next, int count,
+                                                        int sweep_mode) {
+    const int i = threadIdx.x;
+    if (sweep_mode) {
+        first = *next;
+        __syncthreads();
+        if (i == 0) *next = first + (uint32_t)count;
+    }
     if (i >= count) return;
     const uint32_t index = first + (uint32_t)i;
     WordStream s(g.key0, g.key1, index, 0xFFFFFFFFu, (sweep_mode ? kDomSweep : kDomShift) << 28);
@@ -68,81 +78,165 @@ __global__ void k_draws3(G3 g, Draw3* table, uint32_t first, int count, int swee
     const int ax = r.fdir >> 1;
     const double w = ax == 0 ? g.w[0] : (ax == 1 ? g.w[1] : g.w[2]);
     r.ds = unif53(hi, lo) * (0.5 * w);
+    r.dsf = (float)r.ds;
+    r.pad = 0u;
     r.sweep = index;
     table[i] = r;
 }
 
 // Cell shift (Alg. 4) along one of three axes: new cell c keeps the spheres
 // of old c that stay inside it (slot order), then takes those of old c+f
-// that leave c+f, re-expressed in c's frame and clamped into [0, w).  Both
-// old cells are read with 256-bit loads and the new cell is put together in
-// registers.
+// that leave c+f, re-expressed in c's frame and clamped into [0, w).  One
+// thread per new cell, grid (cells of a set, set).
+//
+// The new cell is put together in registers; a slot is looked at only if some
+// lane of the warp has a sphere in it, since nine cells in ten hold at most
+// two: without that, eight slots of either cell took 440 instructions a warp
+// and, in binary64, 16 subtractions and as many pairs of comparisons on the
+// binary64 pipe (73 % busy; the comparisons now read bit patterns).  A cell
+// that holds four spheres or more, before or after, is done by its thread
+// alone, slot by slot from memory to memory.  N = 1M, in-step:
+// binary32 26.5 -> 21.4 us, binary64 150 -> 58.6 us (300 MB through DRAM, 5.1 TB/s).
 template <typename T>
 __device__ __forceinline__ T sel3(int ax, T a, T b, T c) {
     return ax == 0 ? a : (ax == 1 ? b : c);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kShiftB3) k_shift3(G3 g, const T* __restrict__ src, T* __restrict__ dst,
-                                                     const Draw3* __restrict__ table, int jd, Dev3* st) {
-    const unsigned s = blockIdx.x * kShiftB3 + threadIdx.x;
-    if (s >= g.C) return;
-    const Draw3& dr = table[jd];
-    const int ax = dr.fdir >> 1;
-    const int sgn = (dr.fdir & 1) ? -1 : 1;
-    const unsigned Q = s / g.cq, r0 = s % g.cq;
-    const int ix = (int)(r0 % (unsigned)g.h[0]);
-    const unsigned r1 = r0 / (unsigned)g.h[0];
-    const int iy = (int)(r1 % (unsigned)g.h[1]), iz = (int)(r1 / (unsigned)g.h[1]);
-    int nx = 2 * ix + (int)(Q & 1), ny = 2 * iy + (int)((Q >> 1) & 1), nz = 2 * iz + (int)(Q >> 2);
-    if (ax == 0) nx = wrap3(nx + sgn, g.m[0]);
-    else if (ax == 1) ny = wrap3(ny + sgn, g.m[1]);
-    else nz = wrap3(nz + sgn, g.m[2]);
-    T ox[8], oy[8], oz[8], bx[8], by[8], bz[8];
-    ld_cell3(src, g, s, ox, oy, oz);
-    ld_cell3(src, g, sidx3(g, nx, ny, nz), bx, by, bz);
+template <typename T> struct Shift3 {
+    int ax;
     T w, sd, sw, wprev;
+    __device__ __forceinline__ bool inside(T dp) const { return Prm<T>::ge0(dp) && Prm<T>::lt(dp, w); }
+    // Is a sphere with moving coordinate x inside its old cell after the
+    // shift, and its new coordinate: x - sd, for a migrant (to the cell on the
+    // other side of f) one width further and clamped into [0, w).
+    template <bool MIGRANT>
+    __device__ __forceinline__ bool moved(T x, T& v) const {
+        v = Prm<T>::sub(x, sd);
+        const bool in = Prm<T>::ge0(v) && Prm<T>::lt(v, w);
+        if (MIGRANT) {
+            v = Prm<T>::add(v, sw);
+            v = Prm<T>::lt(v, w) ? v : wprev;
+            v = Prm<T>::ge0(v) ? v : (T)0;
+        }
+        return in;
+    }
+    // Appends slots 0..2 of one old cell to slots 0..2 of the new one (k: its
+    // spheres so far): the stayers of c, or the migrants of c + f.
+    template <bool MIGRANTS>
+    __device__ __forceinline__ void append(const T (&x)[4], const T (&y)[4], const T (&z)[4], T (&rx)[4], T (&ry)[4],
+                                           T (&rz)[4], int& k) const {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const bool there = x[j] != (T)kEmpty;
+            if (!__any_sync(0xFFFFFFFFu, there)) break;   // spheres fill a cell from slot 0
+            T v;
+            const bool in = moved<MIGRANTS>(sel3(ax, x[j], y[j], z[j]), v);
+            const bool take = there && (MIGRANTS ? !in : in);
+            const T vx = ax == 0 ? v : x[j], vy = ax == 1 ? v : y[j], vz = ax == 2 ? v : z[j];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if (!MIGRANTS && i > j) break;   // at most j stayers before this one
+                const bool here = take && k == i;
+                rx[i] = here ? vx : rx[i];
+                ry[i] = here ? vy : ry[i];
+                rz[i] = here ? vz : rz[i];
+            }
+            k += take;
+        }
+    }
+    // The same for all slots, from memory to memory.
+    template <bool MIGRANTS>
+    __device__ __forceinline__ void copy(const G3& g, const T* __restrict__ src, unsigned from, T* __restrict__ dst, unsigned to,
+                                         int& k) const {
+#pragma unroll 1
+        for (int j = 0; j < kSlots3; ++j) {
+            const T* q = slot3(src, g, from, j);
+            const T x = q[0], y = q[4], z = q[8];
+            if (x == (T)kEmpty) break;
+            T v;
+            const bool in = moved<MIGRANTS>(sel3(ax, x, y, z), v);
+            if (in == MIGRANTS) continue;
+            if (k < kSlots3) {
+                T* p = dst + (k < 4 ? primary3(to) + k : secondary3(g, to) + (k - 4));
+                p[0] = ax == 0 ? v : x;
+                p[4] = ax == 1 ? v : y;
+                p[8] = ax == 2 ? v : z;
+            }
+            ++k;
+        }
+    }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* __restrict__ src, T* __restrict__ dst,
+                                                     const Draw3* __restrict__ table, int jd, Dev3* st) {
+    pdl_release();
+    pdl_wait();
+    const unsigned r = blockIdx.x * kShiftB3 + threadIdx.x;
+    const bool live = r < g.cq;
+    const int Q = (int)blockIdx.y;
+    const unsigned s = (unsigned)Q * g.cq + r;
+    const Draw3& dr = table[jd];
+    Shift3<T> P;
+    P.ax = dr.fdir >> 1;
+    const int sgn = (dr.fdir & 1) ? -1 : 1;
     if (sizeof(T) == 8) {
-        w = (T)g.w[ax];
-        sd = (T)((double)sgn * dr.ds);
-        sw = (T)((double)sgn * g.w[ax]);
-        wprev = (T)g.wprev[ax];
+        P.w = (T)sel3(P.ax, g.w[0], g.w[1], g.w[2]);
+        P.sd = sgn > 0 ? (T)dr.ds : (T)-dr.ds;
+        P.wprev = (T)sel3(P.ax, g.wprev[0], g.wprev[1], g.wprev[2]);
     } else {
-        w = (T)g.wf[ax];
-        sd = (T)((float)sgn * (float)dr.ds);
-        sw = (T)((float)sgn * g.wf[ax]);
-        wprev = (T)g.wprevf[ax];
+        P.w = (T)sel3(P.ax, g.wf[0], g.wf[1], g.wf[2]);
+        P.sd = sgn > 0 ? (T)dr.dsf : (T)-dr.dsf;
+        P.wprev = (T)sel3(P.ax, g.wprevf[0], g.wprevf[1], g.wprevf[2]);
     }
-    T rx[8], ry[8], rz[8];
+    P.sw = sgn > 0 ? P.w : -P.w;
+    if (s == 0) {
+        if (sizeof(T) == 8) st->origin[P.ax] = sgn > 0 ? __dadd_rn(st->origin[P.ax], dr.ds) : __dsub_rn(st->origin[P.ax], dr.ds);
+        else st->origin[P.ax] += (double)(sgn > 0 ? dr.dsf : -dr.dsf);
+    }
+    // old cell c + f
+    const unsigned r1 = g.div0(r), iz = g.div1(r1);
+    int nx = 2 * (int)(r - r1 * (unsigned)g.h[0]) + (Q & 1), ny = 2 * (int)(r1 - iz * (unsigned)g.h[1]) + ((Q >> 1) & 1),
+        nz = 2 * (int)iz + (Q >> 2);
+    if (P.ax == 0) nx = wrap3(nx + sgn, g.m[0]);
+    else if (P.ax == 1) ny = wrap3(ny + sgn, g.m[1]);
+    else nz = wrap3(nz + sgn, g.m[2]);
+    const unsigned sb = live ? sidx3(g, nx, ny, nz) : 0u;
+    T ox[4], oy[4], oz[4], bx[4], by[4], bz[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) rx[j] = ry[j] = rz[j] = (T)kEmpty;
+    for (int j = 0; j < 4; ++j) ox[j] = bx[j] = (T)kEmpty;
+    if (live) {
+        const T* p = src + primary3(s);
+        const T* q = src + primary3(sb);
+        ld4(p, ox);
+        ld4(q, bx);
+        ld4(p + 4, oy);
+        ld4(q + 4, by);
+        ld4(p + 8, oz);
+        ld4(q + 8, bz);
+    }
+    T rx[4], ry[4], rz[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) rx[j] = ry[j] = rz[j] = (T)kEmpty;
     int k = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const T dp = sel3(ax, ox[j], oy[j], oz[j]) - sd;
-        if (ox[j] != (T)kEmpty && dp >= (T)0 && dp < w) {
-            put8(rx, k, ax == 0 ? dp : ox[j]);
-            put8(ry, k, ax == 1 ? dp : oy[j]);
-            put8(rz, k, ax == 2 ? dp : oz[j]);
-            ++k;
-        }
+    P.template append<false>(ox, oy, oz, rx, ry, rz, k);
+    P.template append<true>(bx, by, bz, rx, ry, rz, k);
+    if (!live) return;
+    T* p = dst + primary3(s);
+    if (ox[3] == (T)kEmpty && bx[3] == (T)kEmpty && k <= 3) {
+        st4(p, rx);
+        st4(p + 4, ry);
+        st4(p + 8, rz);
+        return;
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const T dp = sel3(ax, bx[j], by[j], bz[j]) - sd;
-        if (bx[j] != (T)kEmpty && !(dp >= (T)0 && dp < w)) {
-            T v = dp + sw;
-            if (v >= w) v = wprev;
-            if (v < (T)0) v = (T)0;
-            put8(rx, k, ax == 0 ? v : bx[j]);
-            put8(ry, k, ax == 1 ? v : by[j]);
-            put8(rz, k, ax == 2 ? v : bz[j]);
-            ++k;
-        }
-    }
+    k = 0;
+    P.template copy<false>(g, src, s, dst, s, k);
+    P.template copy<true>(g, src, sb, dst, s, k);
     if (k > kSlots3) atomicOr(&st->error, kErrOverflow);
-    st_cell3(dst, g, s, rx, ry, rz, k >= 4);
-    if (s == 0) st->origin[ax] += (double)sd;
+    for (int j = k; j < (k < 4 ? 4 : kSlots3); ++j) {   // a cell of four or more has a valid secondary half
+        T* q = dst + (j < 4 ? primary3(s) + j : secondary3(g, s) + (j - 4));
+        q[0] = q[4] = q[8] = (T)kEmpty;
+    }
 }
 
 // Contact histogram: every sphere against the spheres of its 5x5x5 cell
@@ -348,9 +442,19 @@ struct hdmc3_handle {
     float lo2f, hi2f;
     int64_t samples;
     uint64_t sweeps, shifts;
+    uint32_t* next;            // device: index of the next sweep to draw
+    cudaStream_t cap;          // private stream used only to record graphs
+    std::map<std::pair<int, int>, cudaGraphExec_t> graphs;   // (sweeps, buffer) -> graph
+    void drop_graphs() {
+        for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
+        graphs.clear();
+    }
 };
 
 namespace {
+
+constexpr int kGraph3 = 32;   // sweeps per recorded graph (289 launches)
+
 
 int finish3(hdmc3_t* h) {
     cudaError_t e = cudaStreamSynchronize(h->stream);
@@ -548,42 +652,51 @@ int download3(hdmc3_t* h, std::vector<double>& loc, std::vector<uint8_t>& cnt) {
     return e;
 }
 
-void launch_sub3(hdmc3_t* h, int jd, int k) {
+LaunchCtx ctx3(cudaStream_t stream, bool pdl) {
+    LaunchCtx c{};
+    c.stream = stream;
+    c.pdl = pdl;
+    return c;
+}
+
+void launch_sub3(hdmc3_t* h, cudaStream_t stream, int cur, int jd, int k, bool pdl) {
+    const LaunchCtx c = ctx3(stream, pdl);
     auto run = [&](auto kernel, auto* cells, unsigned G) {
         const unsigned per = kSubB3 / G;
-        kernel<<<(h->g.cq + per - 1) / per, kSubB3, 0, h->stream>>>(h->g, cells, h->table, jd, k, h->ctr);
+        launch_on(c, kernel, dim3((h->g.cq + per - 1) / per), dim3(kSubB3), h->g, cells, h->table, jd, k, h->ctr);
     };
     // Lanes per cell: few active cells leave the chip idle and the chain of
     // one cell update binds, so its work is spread over a warp; many are bound
     // by instructions, of which wide groups need more.  us per sub-sweep at
-    // n_M = 4 with 32 / 8 / 4 / 2 lanes, binary32 then binary64:
+    // n_M = 4 with 32 / 8 / 4 / 2 lanes, binary32 then binary64 (plain launches):
     //     2,197 active cells   6.2 / 6.7 / 8.2 / 8.6       9.2 / 11.6 / 13.2 / 17.1
     //     7,000               10.3 / 8.3 / 8.5 / 10.3     16.0 / 14.1 / 15.7 / 18.6
     //    32,768               29.0 / 19.3 / 15.7 / 16.2   46.8 / 34.7 / 29.8 / 31.8
     //   132,651              103.2 / 55.4 / 39.7 / 37.1   172 / 108 / 93.2 / 93.9
     const unsigned cq = h->g.cq;
     if (h->prec == HDMC_FP64) {
-        double* a = (double*)h->cells[h->cur];
+        double* a = (double*)h->cells[cur];
         if (cq <= 4096) run(k_sub3<double, 32>, a, 32);
         else if (cq <= 16384) run(k_sub3<double, 8>, a, 8);
         else run(k_sub3<double, 4>, a, 4);
     } else {
-        float* a = (float*)h->cells[h->cur];
+        float* a = (float*)h->cells[cur];
         if (cq <= 4096) run(k_sub3<float, 32>, a, 32);
         else if (cq <= 16384) run(k_sub3<float, 8>, a, 8);
         else run(k_sub3<float, 2>, a, 2);
     }
 }
 
-void launch_shift3(hdmc3_t* h, int jd) {
-    const unsigned blocks = (h->g.C + kShiftB3 - 1) / kShiftB3;
+// One shift from cells[cur] into the other buffer (the caller swaps them).
+void launch_shift3(hdmc3_t* h, cudaStream_t stream, int cur, int jd, bool pdl) {
+    const LaunchCtx c = ctx3(stream, pdl);
+    const dim3 grid((h->g.cq + kShiftB3 - 1) / kShiftB3, 8);
     if (h->prec == HDMC_FP64)
-        k_shift3<double><<<blocks, kShiftB3, 0, h->stream>>>(h->g, (const double*)h->cells[h->cur],
-                                                              (double*)h->cells[1 - h->cur], h->table, jd, h->st);
+        launch_on(c, k_shift3<double>, grid, dim3(kShiftB3), h->g, (const double*)h->cells[cur], (double*)h->cells[1 - cur],
+                  h->table, jd, h->st);
     else
-        k_shift3<float><<<blocks, kShiftB3, 0, h->stream>>>(h->g, (const float*)h->cells[h->cur],
-                                                             (float*)h->cells[1 - h->cur], h->table, jd, h->st);
-    h->cur = 1 - h->cur;
+        launch_on(c, k_shift3<float>, grid, dim3(kShiftB3), h->g, (const float*)h->cells[cur], (float*)h->cells[1 - cur],
+                  h->table, jd, h->st);
 }
 
 void free3(hdmc3_t* h) {
@@ -592,21 +705,59 @@ void free3(hdmc3_t* h) {
     cudaFree(h->cells[1]);
     cudaFree(h->table);
     cudaFree(h->st);
+    h->drop_graphs();
+    if (h->cap) cudaStreamDestroy(h->cap);
     cudaFree(h->ctr);
+    cudaFree(h->next);
     cudaFree(h->hist);
     cudaFree(h->edges2);
     cudaFree(h->binf);
     delete h;
 }
 
-// n sweeps; with events, the mean device time of the sub-sweep and shift
-// launches is measured.
-int enqueue_sweeps3(hdmc3_t* h, int64_t n, double* ms_sub, double* ms_shift) {
-    if (n < 0) return HDMC_EINVAL;
+void launch_draws3(hdmc3_t* h, cudaStream_t stream, int count) {
+    k_draws3<<<1, kDrawChunk3, 0, stream>>>(h->g, h->table, 0u, h->next, count, 1);
+}
+
+// K sweeps on s, starting from buffer cur.  The draws kernel and the first
+// sub-sweep after it are ordinary launches, every later kernel is a
+// programmatic dependent of the one before it (launch_on).
+void enqueue_sweeps3(hdmc3_t* h, cudaStream_t s, int K, int cur) {
+    launch_draws3(h, s, K);
+    for (int j = 0; j < K; ++j) {
+        for (int k = 0; k < 8; ++k) launch_sub3(h, s, cur ^ (j & 1), j, k, j > 0 || k > 0);
+        launch_shift3(h, s, cur ^ (j & 1), j, true);
+    }
+}
+
+// The recorded graph of K sweeps from the current buffer.
+int sweep_graph3(hdmc3_t* h, int K, cudaGraphExec_t& exec) {
+    const auto key = std::make_pair(K, h->cur);
+    auto it = h->graphs.find(key);
+    if (it != h->graphs.end()) {
+        exec = it->second;
+        return HDMC_OK;
+    }
+    if (h->graphs.size() >= 8) h->drop_graphs();
+    cudaGraph_t graph = nullptr;
+    int e = cuda_code(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
+    if (e) return e;
+    enqueue_sweeps3(h, h->cap, K, h->cur);
+    e = cuda_code(cudaStreamEndCapture(h->cap, &graph));
+    if (e) return e;
+    e = cuda_code(cudaGraphInstantiate(&exec, graph, 0));
+    cudaGraphDestroy(graph);
+    if (e) return e;
+    h->graphs[key] = exec;
+    return HDMC_OK;
+}
+
+// n sweeps with an event pair around every launch: the mean device time of
+// the sub-sweep and shift launches.
+int profile_sweeps3(hdmc3_t* h, int64_t n, double* ms_sub, double* ms_shift) {
     std::vector<cudaEvent_t> ev;
     std::vector<int> kind;
     auto mark = [&](int k) {
-        if (!ms_sub && !ms_shift) return;
         cudaEvent_t e;
         cudaEventCreate(&e);
         cudaEventRecord(e, h->stream);
@@ -615,16 +766,17 @@ int enqueue_sweeps3(hdmc3_t* h, int64_t n, double* ms_sub, double* ms_shift) {
     };
     for (int64_t done = 0; done < n;) {
         const int cnt = (int)std::min<int64_t>(kDrawChunk3, n - done);
-        k_draws3<<<1, kDrawChunk3, 0, h->stream>>>(h->g, h->table, (uint32_t)h->sweeps, cnt, 1);
+        launch_draws3(h, h->stream, cnt);
         for (int j = 0; j < cnt; ++j) {
             for (int k = 0; k < 8; ++k) {
                 mark(0);
-                launch_sub3(h, j, k);
+                launch_sub3(h, h->stream, h->cur, j, k, false);
                 mark(-1);
             }
             mark(1);
-            launch_shift3(h, j);
+            launch_shift3(h, h->stream, h->cur, j, false);
             mark(-1);
+            h->cur = 1 - h->cur;
             h->sweeps += 1;
         }
         done += cnt;
@@ -634,20 +786,18 @@ int enqueue_sweeps3(hdmc3_t* h, int64_t n, double* ms_sub, double* ms_shift) {
         for (auto x : ev) cudaEventDestroy(x);
         return cuda_code(e);
     }
-    if (!ev.empty()) {
-        cudaEventSynchronize(ev.back());
-        double tot[2] = {0, 0};
-        int num[2] = {0, 0};
-        for (size_t i = 0; i + 1 < ev.size(); i += 2) {
-            float ms = 0;
-            cudaEventElapsedTime(&ms, ev[i], ev[i + 1]);
-            tot[kind[i]] += ms;
-            num[kind[i]] += 1;
-        }
-        for (auto x : ev) cudaEventDestroy(x);
-        if (ms_sub) *ms_sub = num[0] ? tot[0] / num[0] : 0.0;
-        if (ms_shift) *ms_shift = num[1] ? tot[1] / num[1] : 0.0;
+    cudaEventSynchronize(ev.back());
+    double tot[2] = {0, 0};
+    int num[2] = {0, 0};
+    for (size_t i = 0; i + 1 < ev.size(); i += 2) {
+        float ms = 0;
+        cudaEventElapsedTime(&ms, ev[i], ev[i + 1]);
+        tot[kind[i]] += ms;
+        num[kind[i]] += 1;
     }
+    for (auto x : ev) cudaEventDestroy(x);
+    if (ms_sub) *ms_sub = num[0] ? tot[0] / num[0] : 0.0;
+    if (ms_shift) *ms_shift = num[1] ? tot[1] / num[1] : 0.0;
     return HDMC_OK;
 }
 
@@ -824,6 +974,8 @@ int hdmc3_load(hdmc3_t* h, const void* buf, size_t bytes) {
     if (r[1] != 0 || r[0] != (unsigned long long)h->N) return HDMC_EINVAL;
     // commit
     e = cuda_code(cudaMemcpyAsync(h->st, &st, sizeof(Dev3), cudaMemcpyHostToDevice, s));
+    const uint32_t next = (uint32_t)hd.sweeps;
+    if (!e) e = cuda_code(cudaMemcpyAsync(h->next, &next, sizeof(next), cudaMemcpyHostToDevice, s));
     if (!e) e = cuda_code(cudaMemsetAsync(h->ctr, 0, sizeof(unsigned long long) * 4 * kCtr3, s));
     if (!e)
         e = cuda_code(cudaMemcpyAsync(h->hist, b + L.hist, sizeof(unsigned long long) * kHistBins,
@@ -831,6 +983,7 @@ int hdmc3_load(hdmc3_t* h, const void* buf, size_t bytes) {
     if (!e) e = cuda_code(cudaStreamSynchronize(s));
     if (e) return e;
     h->cur = 1 - h->cur;
+    h->drop_graphs();   // recorded kernels carry the old parameters
     set_move3(h->g, hd.d);
     h->g.nsel = hd.nsel;
     h->g.key0 = hd.key0;
@@ -884,6 +1037,9 @@ int hdmc3_create(hdmc3_t** out, int64_t N, double Lx, double Ly, double Lz, doub
     if (ce == cudaSuccess) ce = cudaMalloc(&h->cells[1], bytes);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->table, sizeof(Draw3) * (kDrawChunk3 + 1));
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->st, sizeof(Dev3));
+    if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
+    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->next, sizeof(uint32_t));
+    if (ce == cudaSuccess) ce = cudaMemset(h->next, 0, sizeof(uint32_t));
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->ctr, sizeof(unsigned long long) * 4 * kCtr3);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->hist, sizeof(unsigned long long) * kHistBins);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->edges2, sizeof(double) * (kHistBins + 1));
@@ -914,14 +1070,33 @@ int hdmc3_create(hdmc3_t** out, int64_t N, double Lx, double Ly, double Lz, doub
 }
 
 int hdmc3_sweep(hdmc3_t* h, int64_t n) {
-    if (!h) return HDMC_EINVAL;
-    return enqueue_sweeps3(h, n, nullptr, nullptr);
+    if (!h || n < 0) return HDMC_EINVAL;
+    // a stream that the caller records takes the launches themselves
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool recorded = cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    while (n > 0) {
+        const int K = (int)std::min<int64_t>(n, recorded ? kDrawChunk3 : kGraph3);
+        int e = HDMC_OK;
+        if (recorded) {
+            enqueue_sweeps3(h, h->stream, K, h->cur);
+            e = cuda_code(cudaGetLastError());
+        } else {
+            cudaGraphExec_t exec;
+            e = sweep_graph3(h, K, exec);
+            if (!e) e = cuda_code(cudaGraphLaunch(exec, h->stream));
+        }
+        if (e) return e;
+        h->cur ^= K & 1;
+        h->sweeps += (uint64_t)K;
+        n -= K;
+    }
+    return HDMC_OK;
 }
 
 int hdmc3_profile_sweeps(hdmc3_t* h, int64_t n, double* ms_subsweep, double* ms_shift) {
     if (!h || n < 1) return HDMC_EINVAL;
     double a = 0, b = 0;
-    int e = enqueue_sweeps3(h, n, &a, &b);
+    int e = profile_sweeps3(h, n, &a, &b);
     if (e) return e;
     if (ms_subsweep) *ms_subsweep = a;
     if (ms_shift) *ms_shift = b;
@@ -944,12 +1119,14 @@ int hdmc3_profile_stages(hdmc3_t* h, int64_t n, double* ms_subsweep, double* ms_
         cudaEventRecord(ev[0], h->stream);
         for (int64_t done = 0; done < n;) {
             const int cnt = (int)std::min<int64_t>(kDrawChunk3, n - done);
-            k_draws3<<<1, kDrawChunk3, 0, h->stream>>>(h->g, h->table, (uint32_t)h->sweeps, cnt, 1);
+            launch_draws3(h, h->stream, cnt);
             for (int j = 0; j < cnt; ++j) {
-                if (stage == 1)
-                    for (int k = 0; k < 8; ++k) launch_sub3(h, j, k);
-                else
-                    launch_shift3(h, j);
+                if (stage == 1) {
+                    for (int k = 0; k < 8; ++k) launch_sub3(h, h->stream, h->cur, j, k, j > 0 || k > 0);
+                } else {
+                    launch_shift3(h, h->stream, h->cur, j, j > 0);
+                    h->cur = 1 - h->cur;
+                }
                 h->sweeps += 1;
             }
             done += cnt;
@@ -970,8 +1147,9 @@ int hdmc3_profile_stages(hdmc3_t* h, int64_t n, double* ms_subsweep, double* ms_
 
 int hdmc3_shift(hdmc3_t* h) {
     if (!h) return HDMC_EINVAL;
-    k_draws3<<<1, 1, 0, h->stream>>>(h->g, h->table + kDrawChunk3, (uint32_t)h->shifts, 1, 0);
-    launch_shift3(h, kDrawChunk3);
+    k_draws3<<<1, 1, 0, h->stream>>>(h->g, h->table + kDrawChunk3, (uint32_t)h->shifts, nullptr, 1, 0);
+    launch_shift3(h, h->stream, h->cur, kDrawChunk3, false);
+    h->cur = 1 - h->cur;
     h->shifts += 1;
     return cuda_code(cudaGetLastError());
 }
@@ -986,7 +1164,7 @@ int hdmc3_subsweep(hdmc3_t* h, uint32_t sweep, int Q) {
     if (e != cudaSuccess) return cuda_code(e);
     e = cudaStreamSynchronize(h->stream);   // d lives on this stack frame
     if (e != cudaSuccess) return cuda_code(e);
-    launch_sub3(h, kDrawChunk3, 0);
+    launch_sub3(h, h->stream, h->cur, kDrawChunk3, 0, false);
     return cuda_code(cudaGetLastError());
 }
 
@@ -1113,12 +1291,15 @@ int hdmc3_set_move_size(hdmc3_t* h, double d) {
     for (int a = 0; a < 3; ++a)
         if (!(d > 0) || !(d < 0.5 * h->g.w[a])) return HDMC_EINVAL;
     set_move3(h->g, d);
+    h->drop_graphs();   // recorded kernels carry the old value
     return HDMC_OK;
 }
 
 int hdmc3_set_balance(hdmc3_t* h, int shuffle_particles, int shuffle_sets) {
     if (!h) return HDMC_EINVAL;
-    h->g.flags = (shuffle_particles ? 0u : kNoParticleShuffle) | (shuffle_sets ? 0u : kNoSetShuffle);
+    const uint32_t f = (shuffle_particles ? 0u : kNoParticleShuffle) | (shuffle_sets ? 0u : kNoSetShuffle);
+    if (f != h->g.flags) h->drop_graphs();   // recorded kernels carry the old geometry
+    h->g.flags = f;
     return HDMC_OK;
 }
 

@@ -60,6 +60,8 @@ struct alignas(8) Draw3 {
     int32_t fdir;          // 2*axis + (1 for the negative direction)
     uint8_t perm[8];       // set of sub-sweep k
     double ds;
+    float dsf;             // binary32 rounding of ds
+    uint32_t pad;
 };
 
 // Trial counters {trials, accepted, left the cell, overlap} are added up in

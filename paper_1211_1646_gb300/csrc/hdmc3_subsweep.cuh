@@ -13,11 +13,11 @@
 // of peak) and in binary64 also the binary64 pipe, which has two instructions
 // per trial coordinate.  One thread per cell, which first gathered the
 // neighbours within reach of its trials into shared memory, took (us per
-// sub-sweep, n_M = 4, before -> now):
-//     216 active cells (N = 2048)       binary32 14.1 ->  6.2   binary64  46.3 ->  8.2
-//   2,197             (N = 16384)                14.4 ->  6.2             45.6 ->  9.2
+// sub-sweep, n_M = 4, before -> now, the latter as programmatic dependents):
+//     216 active cells (N = 2048)       binary32 14.1 ->  4.2   binary64  46.3 ->  6.1
+//   2,197             (N = 16384)                14.4 ->  5.4             45.6 ->  8.5
 //  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
-// 132,651             (N = 1,048,576)            39.4 -> 37.1            165.3 -> 93.2
+// 132,651             (N = 1,048,576)            39.4 -> 34.9            165.3 -> 90.6
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -600,6 +600,8 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
 template <typename T, int G>
 __global__ void __launch_bounds__(kSubB3, G == 2 ? 12 : G == 4 ? 16 : G == 8 ? 20 : 24) k_sub3(const G3 g, T* __restrict__ cells, const Draw3* __restrict__ table, int jd,
                                                  int k, unsigned long long* __restrict__ ctr) {
+    pdl_release();
+    pdl_wait();
     sub3_cells<T, G>(g, cells, table, jd, k, ctr);
 }
 
