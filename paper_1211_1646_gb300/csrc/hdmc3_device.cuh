@@ -194,7 +194,7 @@ __device__ __forceinline__ size_t secondary3(const G3& g, unsigned s) { return (
 // half when slot 3 is occupied, else marks slots 4..7 empty.
 template <typename T>
 __device__ __forceinline__ void ld_rest3(const T* cells, const G3& g, unsigned s, T (&x)[8], T (&y)[8], T (&z)[8]) {
-    if (x[3] != (T)kEmpty) {
+    if (!is_empty(x[3])) {
         ld_half3<4>(cells + secondary3(g, s), x, y, z);
     } else {
 #pragma unroll

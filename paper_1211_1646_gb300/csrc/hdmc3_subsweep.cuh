@@ -14,10 +14,10 @@
 // per trial coordinate.  One thread per cell, which first gathered the
 // neighbours within reach of its trials into shared memory, took (us per
 // sub-sweep, n_M = 4, before -> now, the latter as programmatic dependents):
-//     216 active cells (N = 2048)       binary32 14.1 ->  4.2   binary64  46.3 ->  6.1
-//   2,197             (N = 16384)                14.4 ->  5.4             45.6 ->  8.5
+//     216 active cells (N = 2048)       binary32 14.1 ->  4.2   binary64  46.3 ->  5.8
+//   2,197             (N = 16384)                14.4 ->  5.4             45.6 ->  7.9
 //  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
-// 132,651             (N = 1,048,576)            39.4 -> 34.9            165.3 -> 90.6
+// 132,651             (N = 1,048,576)            39.4 -> 34.1            165.3 -> 80.8
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -40,19 +40,17 @@ __device__ __forceinline__ bool inside_ball(const uint32_t (&w)[6]) {
     return (u0 * u0 + u1 * u1) + u2 * u2 < 1.0;
 }
 
-constexpr float kFar3 = -1.0e18f;   // stands for no sphere: farther than any cell
-
 // Precision-specific parts of a cell update.
 //
 // Trial directions, uniform in the unit ball by rejection from (-1,1)^3:
 //   binary64: consecutive words of the trial stream, six per attempt, three
 //             sym52 variates u = m 2^-52 (m odd, |m| < 2^52); a lane takes
-//             three Philox blocks, two attempts.  A variate is kept as the
-//             binary64 with the sign of m and the magnitude 2^52 + |m|, put
-//             together from its bits, and d u is RN(d u) =
-//             fma(d 2^-52, 2^52 + |m|, -d), with the sign of m: the product
-//             is exactly d + d |m| 2^-52, so one instruction of the slow
-//             binary64 pipe gives the correctly rounded product.
+//             three Philox blocks, two attempts.  The words of a kept
+//             attempt are stored; the trial makes each variate the binary64
+//             with the sign of m and the magnitude 2^52 + |m| (sym52_offset),
+//             and d u is RN(d u) = fma(d 2^-52, 2^52 + |m|, -d), with the
+//             sign of m: the product is exactly d + d |m| 2^-52, so one
+//             instruction of the slow binary64 pipe rounds d u correctly.
 //   binary32: each Philox block of the trial stream cut into six 21-bit
 //             fields, two attempts of three sym21 variates per block, kept
 //             when fma(u, u, fma(v, v, s*s)) < 1; a lane takes one block.
@@ -97,11 +95,6 @@ template <> struct Sub3<double> {
         double u[2][3];
         bool keep[2];
     };
-    static __device__ __forceinline__ double variate(uint32_t hi, uint32_t lo) {
-        const long long m = (long long)(2 * ((((unsigned long long)hi << 32) | lo) >> 12) + 1) - (1ll << 52);
-        const unsigned long long a = (unsigned long long)(m < 0 ? -m : m);
-        return __longlong_as_double((long long)(a | 0x4330000000000000ull | ((unsigned long long)m & 0x8000000000000000ull)));
-    }
     static __device__ __forceinline__ uint32_t attempts(const G3& g, uint32_t sweep, uint32_t c, uint32_t dom,
                                                         uint32_t lane_block, Draw& d) {
         uint32_t w[12];
@@ -118,11 +111,12 @@ template <> struct Sub3<double> {
             const uint32_t v[6] = {w[6 * a], w[6 * a + 1], w[6 * a + 2], w[6 * a + 3], w[6 * a + 4], w[6 * a + 5]};
             d.keep[a] = inside_ball(v);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) d.u[a][q] = variate(v[2 * q], v[2 * q + 1]);
+            for (int q = 0; q < 3; ++q) d.u[a][q] = __hiloint2double((int)v[2 * q], (int)v[2 * q + 1]);
         }
         return w[0];
     }
-    static __device__ __forceinline__ double trial(const G3& g, double x, double v) {
+    static __device__ __forceinline__ double trial(const G3& g, double x, double words) {
+        const double v = sym52_offset((uint32_t)__double2hiint(words), (uint32_t)__double2loint(words));
         const double c = __longlong_as_double(__double_as_longlong(g.d) ^
                                               ((__double_as_longlong(v) & (1ll << 63)) ^ (1ll << 63)));   // -d with v's sign
         return __dadd_rn(x, __fma_rn(g.d52, v, c));
@@ -130,8 +124,8 @@ template <> struct Sub3<double> {
     static __device__ __forceinline__ bool inside(double p, double w) {
         return Prm<double>::ge0(p) && Prm<double>::lt(p, w);
     }
-    static __device__ __forceinline__ float est(double v) { return approx_f32(v); }
-    static __device__ __forceinline__ float est_or_far(double v) { return v == kEmpty ? kFar3 : approx_f32(v); }
+    static __device__ __forceinline__ float est(double v) { return approx_pos(v); }
+    static __device__ __forceinline__ float est_or_far(double v) { return pos_or_far(v); }
 };
 
 // Slots 0 and 1 of a cell, moved by (sx, sy, sz), as packed pairs, and
@@ -236,7 +230,7 @@ __device__ __forceinline__ bool slots_hit(const G3& g, const T* cells, unsigned 
     bool hit = false;
     for (int j = first; j <= last; ++j) {
         const T* q = slot3(cells, g, sn, j);
-        if (q[0] == (T)kEmpty) break;
+        if (is_empty(q[0])) break;
         hit |= A::hit(g, p[0] - (q[0] + sx), p[1] - (q[4] + sy), p[2] - (q[8] + sz));
     }
     return hit;
@@ -251,9 +245,10 @@ template <typename T, int G> struct Warp3 {
     // kept directions, a ring: fewer than kDir3 left over, 2 G more per round
     static constexpr int kRing = G <= 4 ? 16 : G <= 8 ? 32 : G <= 16 ? 64 : 128;
     static_assert(kRing >= kDir3 - 1 + 2 * G, "direction ring");
-    T dir[kCells][kRing][3];
-    T own[kCells][kSlots3][3];   // own spheres, slot order before the shuffle
-    T trial[kCells][4];          // the current trial position
+    // the cell last: the lanes of a warp read neighbouring banks
+    T dir[kRing][3][kCells];
+    T own[kSlots3][3][kCells];   // own spheres, slot order before the shuffle
+    T trial[3][kCells];          // the current trial position
 };
 
 // One sub-sweep: every cell of set Q = table[jd].perm[k] (Alg. 1, Alg. 2).
@@ -306,11 +301,11 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     auto neighbour = [&](int j, unsigned sn, float sx, float sy, float sz) {
         T x2;
         nb[j] = pair_at(cells + primary3(sn), sx, sy, sz, x2);
-        has2 |= x2 != (T)kEmpty ? 1u << j : 0u;
+        has2 |= !is_empty(x2) ? 1u << j : 0u;
     };
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-        nb[j].x = pk(kFar3, kFar3);
+        nb[j].x = pk(kFar, kFar);
         nb[j].y = nb[j].z = 0;
     }
     if (live) {
@@ -346,8 +341,8 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         const unsigned pos = have + __popc(b0 & below) + __popc(b1 & below);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            if (k0) sw.dir[grp][pos % W::kRing][q] = d.u[0][q];
-            if (k1) sw.dir[grp][(pos + k0) % W::kRing][q] = d.u[1][q];
+            if (k0) sw.dir[pos % W::kRing][q][grp] = d.u[0][q];
+            if (k1) sw.dir[(pos + k0) % W::kRing][q][grp] = d.u[1][q];
         }
         have += __popc(b0 & gm) + __popc(b1 & gm);
     };
@@ -380,10 +375,10 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     int n = 0;
 #pragma unroll
     for (int r = 0; r < NO; ++r) {
-        n += __popc(__ballot_sync(kFull, own[r][0] != (T)kEmpty) & gm);
+        n += __popc(__ballot_sync(kFull, !is_empty(own[r][0])) & gm);
         if (L + r * G < 4) {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) sw.own[grp][L + r * G][q] = own[r][q];
+            for (int q = 0; q < 3; ++q) sw.own[L + r * G][q][grp] = own[r][q];
         }
     }
     if (__any_sync(kFull, n == 4)) {
@@ -391,10 +386,10 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         if (n == 4)
             for (int j = L; j < 4; j += G) {
                 const T* p = cells + secondary3(g, sown) + j;
-                if (p[0] == (T)kEmpty) break;
-                sw.own[grp][4 + j][0] = p[0];
-                sw.own[grp][4 + j][1] = p[4];
-                sw.own[grp][4 + j][2] = p[8];
+                if (is_empty(p[0])) break;
+                sw.own[4 + j][0][grp] = p[0];
+                sw.own[4 + j][1][grp] = p[4];
+                sw.own[4 + j][2][grp] = p[8];
                 ++more4;
             }
 #pragma unroll
@@ -432,7 +427,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     // slots 2 and 3 of the first flagged neighbour cell; further flagged cells
     // and slots 4..7 (rare) are read in the trial loop
     Pair3 f23;
-    f23.x = pk(kFar3, kFar3);
+    f23.x = pk(kFar, kFar);
     f23.y = f23.z = 0;
     const bool any23 = __any_sync(kFull, has2 != 0);
     unsigned more = has2 & (has2 - 1u);   // bit 31: slots 4..7 of the first flagged cell may be occupied
@@ -440,7 +435,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         int dx, dy, dz;
         const T* p = cells + primary3(ax.at(g, number(__ffs(has2) - 1), dx, dy, dz));
         f23 = pair23_at(p, (float)dx * g.wf[0], (float)dy * g.wf[1], (float)dz * g.wf[2]);
-        more |= __ldg(p + 3) != (T)kEmpty ? 0x80000000u : 0u;
+        more |= !is_empty(__ldg(p + 3)) ? 0x80000000u : 0u;
     }
     const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots3 && __any_sync(kFull, n > G);
     __syncwarp();
@@ -457,17 +452,17 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     for (int t = 0; t < g.nsel; ++t) {
         if (t > 0 && t % kDir3 == 0) draw((unsigned)min(t + kDir3, g.nsel));
         const int cur = (int)((perm >> (4 * i)) & 7u);
-        T* const me = sw.own[grp][cur];
-        const T* const u = sw.dir[grp][(unsigned)t % W::kRing];
+        T(&me)[3][W::kCells] = sw.own[cur];
+        const T(&u)[3][W::kCells] = sw.dir[(unsigned)t % W::kRing];
         float px, py, pz;
         bool inside;
         if constexpr (S::kExact) {
-            px = S::trial(g, me[0], u[0]);
-            py = S::trial(g, me[1], u[1]);
-            pz = S::trial(g, me[2], u[2]);
+            px = S::trial(g, me[0][grp], u[0][grp]);
+            py = S::trial(g, me[1][grp], u[1][grp]);
+            pz = S::trial(g, me[2][grp], u[2][grp]);
             inside = S::inside(px, w0) && S::inside(py, w1) && S::inside(pz, w2);
         } else {
-            const T p = S::trial(g, me[a0], u[a0]);
+            const T p = S::trial(g, me[a0][grp], u[a0][grp]);
             bool in = S::inside(p, wa);
             const float pf = S::est(p);
             px = __shfl_sync(kFull, pf, gb);
@@ -475,14 +470,14 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
             if constexpr (G >= 4) {
                 pz = __shfl_sync(kFull, pf, gb + 2);
             } else {
-                const T pc = S::trial(g, me[2], u[2]);
+                const T pc = S::trial(g, me[2][grp], u[2][grp]);
                 in = in && S::inside(pc, w2);
                 pz = S::est(pc);
-                if (L == 0) sw.trial[grp][2] = pc;
+                if (L == 0) sw.trial[2][grp] = pc;
             }
             constexpr unsigned m3 = G >= 4 ? 7u : 3u;
             inside = ((__ballot_sync(kFull, in) >> gb) & m3) == m3;
-            if (L < 3) sw.trial[grp][L] = p;
+            if (L < 3) sw.trial[L][grp] = p;
             __syncwarp();
         }
         const f2x px2 = pk(px, px), py2 = pk(py, py), pz2 = pk(pz, pz);
@@ -508,15 +503,14 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         // own cell: the other spheres, one per lane
         if (crowd) {
             auto own_hit = [&](int j) {
-                const T* q = sw.own[grp][j];
+                const T q[3] = {sw.own[j][0][grp], sw.own[j][1][grp], sw.own[j][2][grp]};
                 if constexpr (S::kExact) {
                     return A::hit(g, px - q[0], py - q[1], pz - q[2]);
                 } else {
                     const float ex = px - S::est(q[0]), ey = py - S::est(q[1]), ez = pz - S::est(q[2]);
                     const float r2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
                     if (r2 < g.band_lo || r2 > g.band_hi) return r2 < g.band_lo;
-                    const T* tp = sw.trial[grp];
-                    return A::hit(g, tp[0] - q[0], tp[1] - q[1], tp[2] - q[2]);
+                    return A::hit(g, sw.trial[0][grp] - q[0], sw.trial[1][grp] - q[1], sw.trial[2][grp] - q[2]);
                 }
             };
             if (L < n && L != cur) hit |= own_hit(L);
@@ -534,13 +528,14 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
             }
             const f2x y = add2(ztriple(f23, px2, py2, pz2, lo2), band2);
             close |= ((lo32(y) >> 31) << 30) | (hi32(y) & 0x80000000u);
+            const T tp[3] = {sw.trial[0][grp], sw.trial[1][grp], sw.trial[2][grp]};
             while (close) {
                 const int b = __ffs(close) - 1;
                 close &= close - 1u;
                 const int j = b >= 30 ? __ffs(has2) - 1 : b >> 1, slot = b >= 30 ? b - 28 : b & 1;
                 int dx, dy, dz;
                 const unsigned sn = ax.at(g, number(j), dx, dy, dz);
-                hit |= slots_hit(g, cells, sn, dx, dy, dz, slot, slot, sw.trial[grp]);
+                hit |= slots_hit(g, cells, sn, dx, dy, dz, slot, slot, tp);
             }
         }
         if (more && !hit && inside) {   // rare: slots 2..7 of further flagged cells, slots 4..7 of the first
@@ -555,7 +550,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
                     tp[2] = pz;
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) tp[q] = sw.trial[grp][q];
+                    for (int q = 0; q < 3; ++q) tp[q] = sw.trial[q][grp];
                 }
                 hit |= slots_hit(g, cells, sn, dx, dy, dz, b == 31 ? 4 : 2, kSlots3 - 1, tp);
             }
@@ -564,12 +559,12 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         if (n > 0 && inside && !overlap) {
             if (L == 0) {
                 if constexpr (S::kExact) {
-                    me[0] = px;
-                    me[1] = py;
-                    me[2] = pz;
+                    me[0][grp] = px;
+                    me[1][grp] = py;
+                    me[2][grp] = pz;
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) me[q] = sw.trial[grp][q];
+                    for (int q = 0; q < 3; ++q) me[q][grp] = sw.trial[q][grp];
                 }
             }
             ++n_ac;
@@ -581,11 +576,11 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     // the shuffled slots back; unused slots keep their sentinels
 #pragma unroll 1
     for (int j = L; j < n; j += G) {
-        const T* q = sw.own[grp][(perm >> (4 * j)) & 7u];
+        const unsigned o = (perm >> (4 * j)) & 7u;
         T* p = cells + (j < 4 ? primary3(sown) + j : secondary3(g, sown) + (j - 4));
-        p[0] = q[0];
-        p[4] = q[1];
-        p[8] = q[2];
+        p[0] = sw.own[o][0][grp];
+        p[4] = sw.own[o][1][grp];
+        p[8] = sw.own[o][2][grp];
     }
     // counters: one lane per cell
     const bool count = L == 0 && n > 0;

@@ -210,6 +210,32 @@ __device__ __forceinline__ float approx_f32(double v) {
     return e < 897u ? __uint_as_float(hi & 0x80000000u) : __uint_as_float(f);
 }
 
+// The same for a stored coordinate or a trial position inside its cell
+// (non-negative): the nine low exponent bits and 23 of the significand,
+// rebiased.  pos_or_far: an empty slot is far from every cell.
+__device__ __forceinline__ float approx_pos(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t f = __funnelshift_l(lo, hi, 3) - 0xC0000000u;
+    return (hi << 1) < (897u << 21) ? 0.0f : __uint_as_float(f);
+}
+
+// The variate of sym52 (u = m 2^-52, m odd, |m| < 2^52) as the binary64 with
+// the sign of m and the magnitude 2^52 + |m|, put together from its bits.
+__device__ __forceinline__ double sym52_offset(uint32_t hi, uint32_t lo) {
+    const unsigned long long k = (((unsigned long long)hi << 32) | lo) >> 12;
+    const long long m = (long long)(2 * k + 1) - (1ll << 52);
+    const unsigned long long a = (unsigned long long)(m < 0 ? -m : m);
+    return __longlong_as_double((long long)(a | 0x4330000000000000ull | ((unsigned long long)m & 0x8000000000000000ull)));
+}
+
+// Is a stored coordinate that of an empty slot (kEmpty)?  Decided on the bit
+// pattern: binary64 comparisons run on the slow pipe.
+__device__ __forceinline__ bool is_empty(float v) { return v == (float)kEmpty; }
+__device__ __forceinline__ bool is_empty(double v) { return (uint32_t)__double2hiint(v) > 0x80000000u; }
+
+constexpr float kFar = -1.0e18f;   // stands for no disk or sphere: farther than any cell
+__device__ __forceinline__ float pos_or_far(double v) { return is_empty(v) ? kFar : approx_pos(v); }
+
 // Per-block trial counters bpart[{trials, accepted, left, overlap}] of the
 // block's own slot: each warp adds its sums with fire-and-forget atomic
 // adds (no value returned, so nothing waits on the round trip; integer sums
