@@ -2,9 +2,30 @@
 #include "hdmc_kernels.cuh"
 
 namespace hdmc {
+// Lanes per cell: few active cells leave the chip idle and the chain of one
+// cell update binds, so its work is spread over a group of lanes; with many
+// the instructions bind, of which one thread per cell needs fewest.  Crowded
+// cells (most directions have a third disk) keep two lanes, which hold all
+// slots in registers.  us per sub-sweep in-step at n_M = 4 with 8 / 4 / 2
+// lanes and one thread (before: 8.0, 12.8, 16.2, 17.3, 20.5, 47.9; crowded
+// 19.1, 43.1):
+//       270 active cells   3.7 / 4.3 / 5.7 / 6.7
+//     8,976                5.9 / 6.4 / 8.3 / 9.0
+//    18,270                8.4 / 6.6 / 8.9 / 10.8
+//    36,108               12.9 / 10.7 / 9.3 / 11.2
+//    73,332               22.5 / 17.8 / 15.8 / 16.0
+//   293,328               79.6 / 57.1 / 45.2 / 37.8
+//   crowded, 9,360         6.3 / 6.9 / 10.3 / 17.9
+//   crowded, 147,441      47.0 / 34.7 / 31.6 / 40.3
 void launch_subsweep_f64(const LaunchCtx& c, void* cells, const SweepDraw* draw, int k) {
-    launch_on(c, k_subsweep_f64, dim3((unsigned)((c.g.hx + 31) / 32), (unsigned)c.g.hy), dim3(32, 1), c.g,
-              reinterpret_cast<double*>(cells), draw, k, c.partial);
+    if (c.g.cq <= 12288) return launch_lanes<8>(c, cells, draw, k);
+    if (c.g.cq <= 24576) return launch_lanes<4>(c, cells, draw, k);
+    if (c.g.cq <= 65536 || c.g.dense) return launch_lanes<2>(c, cells, draw, k);
+    double* a = reinterpret_cast<double*>(cells);
+    const dim3 grid((unsigned)((c.g.hx + 31) / 32), (unsigned)((c.g.hy + 1) / 2)), block(32, 2);
+    if (c.g.nsel == 4) launch_on(c, k_subsweep_f64<2, 4>, grid, block, c.g, a, draw, k, c.partial);
+    else if (c.g.nsel == 8) launch_on(c, k_subsweep_f64<2, 8>, grid, block, c.g, a, draw, k, c.partial);
+    else launch_on(c, k_subsweep_f64<2, 0>, grid, block, c.g, a, draw, k, c.partial);
 }
 void launch_shift_f64(const LaunchCtx& c, const void* src, void* dst, const SweepDraw* draw) {
     launch_shift_t<double>(c, src, dst, draw);
@@ -18,7 +39,8 @@ void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long*
 }
 
 void launch_subsweep_f64_batch(const BatchCtx& c, void* arena, const SweepDraw* draws, int j, int k) {
-    k_subsweep_f64_batch<<<c.sub_blocks, dim3(32, 4), 0, c.stream>>>(c.reps, c.sub_map, reinterpret_cast<double*>(arena),
-                                                                      draws, c.R, j, k, c.partial);
+    constexpr int G = 2;
+    k_subsweep_f64_batch<G><<<c.sub_blocks, dim3(32, 4 * G), 0, c.stream>>>(c.reps, c.sub_map, reinterpret_cast<double*>(arena),
+                                                                            draws, c.R, j, k, c.partial);
 }
 }  // namespace hdmc

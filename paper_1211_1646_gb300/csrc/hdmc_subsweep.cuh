@@ -1,12 +1,10 @@
-// hdmc_subsweep.cuh -- the sub-sweep kernels (Alg. 2) in binary32 and
-// binary64.
+// hdmc_subsweep.cuh -- the binary32 sub-sweep (Alg. 2) with one thread per
+// active cell (hdmc_subsweep64.cuh has the form with several lanes per cell).
 //
 // Every floating-point operation that decides an acceptance is written with
 // an explicit round-to-nearest operation, so the result does not depend on
-// compiler contraction:
-//   binary64: trial coordinate p + d*u, overlap iff dx*dx + dy*dy < sigma^2;
-//   binary32: trial coordinate fma(d, u, p), overlap iff
-//             fma(dx, dx, fma(dy, dy, -sigma^2)) < 0.
+// compiler contraction: trial coordinate fma(d, u, p), overlap iff
+// fma(dx, dx, fma(dy, dy, -sigma^2)) < 0.
 #pragma once
 
 #include "hdmc_common.cuh"
@@ -342,231 +340,6 @@ k_subsweep_f32(const Geometry g, float* __restrict__ cells, const SweepDraw* __r
     // tile: atomic adds)
     const long long slot = (long long)(blockIdx.y * ROWS / kCounterRows) * gridDim.x + blockIdx.x;
     subsweep_f32<ROWS, NSEL, false, DENSE>(g, cells, draw, k, blockIdx.x, blockIdx.y, partial + 4 * slot, sdir);
-}
-
-// ---- binary64 sub-sweep ---------------------------------------------------------------
-// Same algorithm in binary64.  Draws: shuffle by one 32-bit Lemire draw in
-// [0, n!) from the cell's shuffle stream; trial t takes the t-th kept attempt
-// of the trial stream, attempt a = block a: u = sym52(w0,w1), v = sym52(w2,w3),
-// kept iff u*u + v*v < 1.
-//
-// Every decision is the exact binary64 expression, but binary64 arithmetic
-// is slow on this GPU, so binary32 estimates settle the clear cases first:
-//  - in-circle test: u, v truncated to 23 bits (|error| <= 2^-23); cases with
-//    the estimate of u^2 + v^2 within 2^-18 of 1 are decided in binary64;
-//  - overlap test: positions truncated to binary32 (relative error <= 2^-23),
-//    the squared distance estimated with binary32 pair arithmetic (error
-//    below 3e-6 where it matters, r^2 < 1.3); a candidate counts as certainly
-//    overlapping below sigma^2 - 2^-15 and certainly clear above sigma^2 + 2^-15;
-//    if any candidate falls in between, all candidates are tested in binary64.
-constexpr float kOverlapBand = 0x1p-15f;
-constexpr float kCircleBand = 0x1p-18f;
-
-// Exact binary64 overlap test of a trial position against every candidate
-// whose binary32 estimate (the prefilter's own expression, with the upper
-// band edge) says "possibly overlapping"; the others are certainly clear.
-// sigma^2 and r^2 are non-negative, so r^2 < sigma^2 compares bit patterns.
-__device__ __forceinline__ bool exact_trial_hit(const Geometry& g, const double* __restrict__ cells,
-                                                  const Neighbourhood& nbh, int hx, int hy, const Cell<double>& own,
-                                                  const float ofx[4], const float ofy[4], int i, double tx, double ty,
-                                                  float txf, float tyf) {
-    const long long s2 = __double_as_longlong(g.sig2);
-    const float nhi = -((float)g.sig2 + kOverlapBand);
-    bool hit = false;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float ex = __fsub_rn(txf, ofx[j]), ey = __fsub_rn(tyf, ofy[j]);
-        if (j != i && __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, nhi)) < 0.f) {
-            const double ddx = __dsub_rn(tx, own.x[j]), ddy = __dsub_rn(ty, own.y[j]);
-            hit |= __double_as_longlong(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy))) < s2;
-        }
-    }
-    const float wxf = (float)g.wx, wyf = (float)g.wy;
-    for (int c = 0; c < 8; ++c) {
-        Cell<double> a;
-        load_cell_ro(cell_at(cells, nbh.index(g, c, hx, hy)), a);
-        const double sx = (double)dir_dx(c) * g.wx, sy = (double)dir_dy(c) * g.wy;
-        const float sxf = (float)dir_dx(c) * wxf, syf = (float)dir_dy(c) * wyf;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float ex = __fsub_rn(txf, __fadd_rn(approx_f32(a.x[j]), sxf));
-            const float ey = __fsub_rn(tyf, __fadd_rn(approx_f32(a.y[j]), syf));
-            if (__fmaf_rn(ex, ex, __fmaf_rn(ey, ey, nhi)) < 0.f) {
-                const double ddx = __dsub_rn(tx, __dadd_rn(a.x[j], sx)), ddy = __dsub_rn(ty, __dadd_rn(a.y[j], sy));
-                hit |= __double_as_longlong(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy))) < s2;
-            }
-        }
-    }
-    return hit;
-}
-
-// 53-bit odd integer m of sym52 (u = m 2^-52) and its binary32 truncation m 2^-52.
-__device__ __forceinline__ long long sym52_int(uint32_t hi, uint32_t lo) {
-    const unsigned long long k = (((unsigned long long)hi << 32) | lo) >> 12;
-    return (long long)(2 * k + 1) - (1ll << 52);
-}
-__device__ __forceinline__ float sym52_est(long long m) { return (float)(int)(m >> 29) * 0x1p-23f; }
-
-template <int ROWS>
-__device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restrict__ cells,
-                                             const SweepDraw* __restrict__ draw, int k, int bx, int by,
-                                             unsigned long long* __restrict__ bpart) {
-    const int Q = draw->perm[k];
-    const uint32_t sweep = draw->sweep;
-    const int hx = bx * 32 + threadIdx.x;
-    const int hy = by * ROWS + threadIdx.y;
-    const int cx = 2 * hx + (Q & 1), cy = 2 * hy + (Q >> 1);
-    const bool live = hx < g.hx && hy < g.hy && cy >= g.ylo && cy <= g.yhi;
-    const Neighbourhood nbh(g, Q, hx, hy, live);
-
-    Cell<double> own;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = kEmpty;
-    double* ownp = cell_at(cells, nbh.own(g, hx, hy));
-    if (live) load_cell(ownp, own);
-    float4 n01[8];   // binary32 truncations of neighbour slots 0,1 (x0 x1 y0 y1)
-    float n2[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        n01[c] = make_float4((float)kEmpty, (float)kEmpty, (float)kEmpty, (float)kEmpty);
-        n2[c] = (float)kEmpty;
-        if (live) {
-            const double* p = cell_at(cells, nbh.index(g, c, hx, hy));
-            const double2 x01 = __ldg(reinterpret_cast<const double2*>(p));
-            const double2 y01 = __ldg(reinterpret_cast<const double2*>(p) + 2);
-            n01[c] = make_float4(approx_f32(x01.x), approx_f32(x01.y), approx_f32(y01.x), approx_f32(y01.y));
-            n2[c] = approx_f32(__ldg(p + 2));
-        }
-    }
-    const int n = Prm<double>::ge0(own.x[0]) + Prm<double>::ge0(own.x[1]) + Prm<double>::ge0(own.x[2]) +
-                  Prm<double>::ge0(own.x[3]);
-    uint32_t dir23 = 0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) dir23 |= __any_sync(0xffffffffu, n2[c] >= 0.f) ? (1u << c) : 0u;
-    const bool own23 = __any_sync(0xffffffffu, n >= 3);
-
-    unsigned int n_tr = 0, n_acc = 0, n_leave = 0;
-    if (n > 0) {
-        const uint32_t cell = (uint32_t)(cy + g.row0) * (uint32_t)g.mx + (uint32_t)cx;   // global cell number
-        const uint32_t setbits = (uint32_t)Q << 24;
-        if (n >= 2 && !(g.flags & kNoParticleShuffle)) {
-            WordStream s(g.key0, g.key1, sweep, cell, (kDomShuffle << 28) | setbits);
-            shuffle_slots(own.x, own.y, n, s.bounded(factorial(n)));
-        }
-        float ofx[4], ofy[4];   // binary32 truncations of the own slots
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            ofx[j] = approx_f32(own.x[j]);
-            ofy[j] = approx_f32(own.y[j]);
-        }
-        const float wxf = (float)g.wx, wyf = (float)g.wy;
-        f2x qx01[8], qy01[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float sx = (float)dir_dx(c) * wxf, sy = (float)dir_dy(c) * wyf;
-            qx01[c] = add2(pk(n01[c].x, n01[c].y), pk(sx, sx));
-            qy01[c] = add2(pk(n01[c].z, n01[c].w), pk(sy, sy));
-        }
-        f2x fx23 = 0, fy23 = 0;
-        const uint32_t more23 = dir23 & (dir23 - 1);
-        if (dir23) {
-            const int c = __ffs(dir23) - 1;
-            const double2* p = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-            const double2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
-            const float sx = (float)dir_dx(c) * wxf, sy = (float)dir_dy(c) * wyf;
-            fx23 = add2(pk(approx_f32(x23.x), approx_f32(x23.y)), pk(sx, sx));
-            fy23 = add2(pk(approx_f32(y23.x), approx_f32(y23.y)), pk(sy, sy));
-        }
-        const float s2f = (float)g.sig2;
-        const f2x nlo = pk(-(s2f - kOverlapBand), -(s2f - kOverlapBand));   // certainly overlapping below
-        const f2x nhi = pk(-(s2f + kOverlapBand), -(s2f + kOverlapBand));   // possibly overlapping below
-        const double dscaled = g.d * 0x1p-52;   // d*u = (d 2^-52) * m exactly as real numbers
-        const uint32_t c2 = (kDomTrial << 28) | setbits;
-        uint32_t blk = 0;
-        int i = 0;
-        for (int t = 0; t < g.nsel; ++t) {
-            long long mu, mv;
-            for (;;) {
-                const uint4 r = philox4x32_10(make_uint4(sweep, cell, c2, blk++), g.key0, g.key1);
-                mu = sym52_int(r.x, r.y);
-                mv = sym52_int(r.z, r.w);
-                const float uf = sym52_est(mu), vf = sym52_est(mv);
-                const float e = __fmaf_rn(uf, uf, __fmul_rn(vf, vf));
-                if (e < 1.0f - kCircleBand) break;
-                if (e >= 1.0f + kCircleBand) continue;
-                const double u = (double)mu * 0x1p-52, v = (double)mv * 0x1p-52;
-                if (__dadd_rn(__dmul_rn(u, u), __dmul_rn(v, v)) < 1.0) break;
-            }
-            const double tx = __dadd_rn(pick(own.x, i), __dmul_rn(dscaled, (double)mu));
-            const double ty = __dadd_rn(pick(own.y, i), __dmul_rn(dscaled, (double)mv));
-            const bool inside = Prm<double>::ge0(tx) && Prm<double>::lt(tx, g.wx) && Prm<double>::ge0(ty) &&
-                                Prm<double>::lt(ty, g.wy);
-            const float txf = approx_f32(tx), tyf = approx_f32(ty);
-            const f2x tx2 = pk(txf, txf), ty2 = pk(tyf, tyf);
-            uint32_t sure = 0, maybe = 0;   // sign bits: certainly / possibly overlapping
-            {
-                const f2x dx = sub2(tx2, pk(ofx[0], ofx[1])), dy = sub2(ty2, pk(ofy[0], ofy[1]));
-                const f2x zl = fma2(dx, dx, fma2(dy, dy, nlo)), zh = fma2(dx, dx, fma2(dy, dy, nhi));
-                sure |= (i == 0 ? 0u : lo32(zl)) | (i == 1 ? 0u : hi32(zl));
-                maybe |= (i == 0 ? 0u : lo32(zh)) | (i == 1 ? 0u : hi32(zh));
-            }
-            if (own23) {
-                const f2x dx = sub2(tx2, pk(ofx[2], ofx[3])), dy = sub2(ty2, pk(ofy[2], ofy[3]));
-                const f2x zl = fma2(dx, dx, fma2(dy, dy, nlo)), zh = fma2(dx, dx, fma2(dy, dy, nhi));
-                sure |= (i == 2 ? 0u : lo32(zl)) | (i == 3 ? 0u : hi32(zl));
-                maybe |= (i == 2 ? 0u : lo32(zh)) | (i == 3 ? 0u : hi32(zh));
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const f2x dx = sub2(tx2, qx01[c]), dy = sub2(ty2, qy01[c]);
-                const f2x zl = fma2(dx, dx, fma2(dy, dy, nlo)), zh = fma2(dx, dx, fma2(dy, dy, nhi));
-                sure |= lo32(zl) | hi32(zl);
-                maybe |= lo32(zh) | hi32(zh);
-            }
-            if (dir23) {
-                const f2x dx = sub2(tx2, fx23), dy = sub2(ty2, fy23);
-                const f2x zl = fma2(dx, dx, fma2(dy, dy, nlo)), zh = fma2(dx, dx, fma2(dy, dy, nhi));
-                sure |= lo32(zl) | hi32(zl);
-                maybe |= lo32(zh) | hi32(zh);
-            }
-            for (uint32_t m = more23; m; m &= m - 1) {
-                const int c = __ffs(m) - 1;
-                const double2* p = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-                const double2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
-                const float sx = (float)dir_dx(c) * wxf, sy = (float)dir_dy(c) * wyf;
-                const f2x dx = sub2(tx2, add2(pk(approx_f32(x23.x), approx_f32(x23.y)), pk(sx, sx)));
-                const f2x dy = sub2(ty2, add2(pk(approx_f32(y23.x), approx_f32(y23.y)), pk(sy, sy)));
-                const f2x zl = fma2(dx, dx, fma2(dy, dy, nlo)), zh = fma2(dx, dx, fma2(dy, dy, nhi));
-                sure |= lo32(zl) | hi32(zl);
-                maybe |= lo32(zh) | hi32(zh);
-            }
-            bool hit = (sure & 0x80000000u) != 0;
-            if (inside && !hit && (maybe & 0x80000000u))
-                hit = exact_trial_hit(g, cells, nbh, hx, hy, own, ofx, ofy, i, tx, ty, txf, tyf);
-            const bool ok = inside && !hit;
-            put_if(own.x, i, tx, ok);
-            put_if(own.y, i, ty, ok);
-            put_if(ofx, i, txf, ok);
-            put_if(ofy, i, tyf, ok);
-            ++n_tr;
-            n_acc += ok;
-            n_leave += !inside;
-            i = (i + 1 == n) ? 0 : i + 1;
-        }
-        store_cell(ownp, own);
-    }
-    add_block_counters<ROWS>(n_tr, n_acc, n_leave, bpart);
-}
-
-// One-warp blocks (one set row of 32 cells), 16 per SM (128 registers).
-static __global__ void __launch_bounds__(32, 16)
-k_subsweep_f64(const Geometry g, double* __restrict__ cells, const SweepDraw* __restrict__ draw, int k,
-               unsigned long long* __restrict__ partial) {
-    pdl_release();
-    pdl_wait();
-    // counters of the tile that holds this block (shared: atomic adds)
-    subsweep_f64<1>(g, cells, draw, k, blockIdx.x, blockIdx.y,
-                    partial + 4 * ((long long)(blockIdx.y / kCounterRows) * gridDim.x + blockIdx.x));
 }
 
 }  // namespace hdmc
