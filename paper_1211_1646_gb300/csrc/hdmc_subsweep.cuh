@@ -101,6 +101,7 @@ __device__ __forceinline__ void draw_directions_once(const PhiloxKeys& K, uint32
                                                      const uint32_t F0[6], float2 (*__restrict__ sdir)[32 * ROWS],
                                                      int tid) {
     static_assert(WANT <= kDirChunk && kDirRows >= kDirChunk + 2 && kDirRows >= 8, "sdir rows");
+    constexpr uint32_t kOnce = WANT == 1 ? 2 : 3;
     int have = 0;
     auto attempt = [&](uint32_t a, uint32_t b) {
         const float u = sym21(a), v = sym21(b);
@@ -112,20 +113,109 @@ __device__ __forceinline__ void draw_directions_once(const PhiloxKeys& K, uint32
     attempt(F0[2], F0[3]);
     attempt(F0[4], F0[5]);
 #pragma unroll
-    for (uint32_t blk = 1; blk < 3; ++blk) {   // every lane needs block 1, nearly every warp block 2
+    for (uint32_t blk = 1; blk < kOnce; ++blk) {   // every lane needs block 1, nearly every warp block 2
         uint32_t F[6];
         fields21(philox_rk<(WANT > 4)>(make_uint4(sweep, cell, c2, blk), K), F);
         attempt(F[0], F[1]);
         attempt(F[2], F[3]);
         attempt(F[4], F[5]);
     }
-    for (uint32_t blk = 3; have < WANT; ++blk) {
+    for (uint32_t blk = kOnce; have < WANT; ++blk) {
         uint32_t F[6];
         fields21(philox_rk<(WANT > 4)>(make_uint4(sweep, cell, c2, blk), K), F);
         attempt(F[0], F[1]);
         attempt(F[2], F[3]);
         attempt(F[4], F[5]);
     }
+}
+
+// Phases 3 and 4 for a warp whose cells hold at most two disks each: nearly
+// every warp with cells of about sigma (none of a 256^2-disk fluid at phi =
+// 0.716 held three).  Trial t moves slot t mod n, so even trials move slot 0
+// without a select, odd ones slot n - 1, and the shuffle is one conditional
+// exchange (bit 20 of field 0: the 21-bit Lemire draw in [0, 2)).  N = 1M, phi
+// = 0.70, in-step: 11.31 -> 10.60 us at n_M = 4, 17.88 -> 16.31 us at n_M = 8.  (Bounding the 16 neighbour slots
+// through |t|^2 + (|q|^2 - sigma^2) - 2 t.q first, two packed multiply-adds
+// and a three-input minimum per pair with a band that falls back on the
+// method's expression, was slower: 11.77 us.)
+template <int ROWS, int NSEL>
+__device__ __forceinline__ void trials_of_two(const Geometry& g, const float* __restrict__ cells, const Neighbourhood& nbh,
+                                              int hx, int hy, Cell<float>& own, int n, uint32_t f0, const float4 (&n01)[8],
+                                              uint32_t dir23, const float2 (*__restrict__ sdir)[32 * ROWS], int tid,
+                                              unsigned int& n_acc, unsigned int& n_leave) {
+    const bool two = n == 2;
+    float x0 = own.x[0], y0 = own.y[0], x1 = own.x[1], y1 = own.y[1];
+    if (two && !(f0 >> 20) && !(g.flags & kNoParticleShuffle)) {
+        x0 = own.x[1];
+        y0 = own.y[1];
+        x1 = own.x[0];
+        y1 = own.y[0];
+    }
+    const f2x ns2 = pk(-g.sig2f, -g.sig2f);
+    f2x qx[8], qy[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
+        qx[c] = add2(pk(n01[c].x, n01[c].y), pk(sx, sx));
+        qy[c] = add2(pk(n01[c].z, n01[c].w), pk(sy, sy));
+    }
+    // slot pair (2,3) of flagged direction c, translated
+    auto pair23 = [&](int c, f2x& x, f2x& y) {
+        const float2* p = reinterpret_cast<const float2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
+        const float2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
+        const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
+        x = add2(pk(x23.x, x23.y), pk(sx, sx));
+        y = add2(pk(y23.x, y23.y), pk(sy, sy));
+    };
+    f2x fx23 = 0, fy23 = 0;
+    const uint32_t more23 = dir23 & (dir23 - 1);
+    if (dir23) pair23(__ffs(dir23) - 1, fx23, fy23);
+    const float df = g.df;
+#pragma unroll
+    for (int t = 0; t < NSEL; ++t) {
+        const bool second = (t & 1) && two;   // moves slot 1
+        const float2 uv = sdir[t][tid];
+        const float tx = __fmaf_rn(df, uv.x, second ? x1 : x0);
+        const float ty = __fmaf_rn(df, uv.y, second ? y1 : y0);
+        // 0 <= t < w as one unsigned compare of the bit patterns (w > 0; fma(d, u, p) with d*u != 0 is never -0)
+        const bool inside = __float_as_uint(tx) < __float_as_uint(g.wxf) && __float_as_uint(ty) < __float_as_uint(g.wyf);
+        const f2x tx2 = pk(tx, tx), ty2 = pk(ty, ty);
+        // the other own slot (empty unless two), by the method's expression
+        const float ex = __fsub_rn(tx, second ? x0 : x1), ey = __fsub_rn(ty, second ? y0 : y1);
+        uint32_t acc = __float_as_uint(__fmaf_rn(ex, ex, __fmaf_rn(ey, ey, -g.sig2f)));
+        if (dir23) {
+            const f2x z = zpair(tx2, ty2, fx23, fy23, ns2);
+            acc |= lo32(z) | hi32(z);
+        }
+        for (uint32_t m = more23; m; m &= m - 1) {   // warp-uniform, rarely taken
+            f2x x, y;
+            pair23(__ffs(m) - 1, x, y);
+            const f2x z = zpair(tx2, ty2, x, y, ns2);
+            acc |= lo32(z) | hi32(z);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const f2x z = zpair(tx2, ty2, qx[c], qy[c], ns2);
+            acc |= lo32(z) | hi32(z);
+        }
+        const bool ok = inside && !(acc >> 31);
+        if (t & 1) {
+            const bool ok1 = ok && two, ok0 = ok && !two;
+            x1 = ok1 ? tx : x1;
+            y1 = ok1 ? ty : y1;
+            x0 = ok0 ? tx : x0;
+            y0 = ok0 ? ty : y0;
+        } else {
+            x0 = ok ? tx : x0;
+            y0 = ok ? ty : y0;
+        }
+        n_acc += ok;
+        n_leave += !inside;
+    }
+    own.x[0] = x0;
+    own.y[0] = y0;
+    own.x[1] = x1;
+    own.y[1] = y1;
 }
 
 // DENSE (cells that often hold three or four disks, as with the paper's
@@ -202,6 +292,17 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
 
     unsigned int n_tr = 0, n_acc = 0, n_leave = 0;
     float net2 = 0.f;
+    if constexpr (!DENSE && !TRACK && NSEL > 0 && NSEL <= kDirChunk) {
+        if (!own23) {   // warp-uniform
+            if (n > 0) {
+                trials_of_two<ROWS, NSEL>(g, cells, nbh, hx, hy, own, n, f0, n01, dir23, sdir, tid, n_acc, n_leave);
+                n_tr = (unsigned)NSEL;
+                store_cell(ownp, own);
+            }
+            add_block_counters<ROWS>(n_tr, n_acc, n_leave, bpart);
+            return;
+        }
+    }
     if (n > 0) {
         // shuffle of the cell's disks (Alg. 1): one draw in [0, n!) by 21-bit Lemire on field 0
         if (n >= 2 && !(g.flags & kNoParticleShuffle)) {
