@@ -25,11 +25,15 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
+#include <new>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
 #include "hdmc.h"
 #include "hdmc3_subsweep.cuh"
+#include "hdmc_export.cuh"
 
 namespace hdmc {
 
@@ -388,6 +392,45 @@ __global__ void __launch_bounds__(kHistB3, 4) k_hist3(G3 g, const T* __restrict_
         if (sh[b]) atomicAdd(&hist[b], (unsigned long long)sh[b]);
 }
 
+// Export of the coordinates (hdmc_export.cuh): canonical cell c of the
+// thread, its storage index and its number of spheres.
+template <typename T>
+__device__ __forceinline__ unsigned export_cell3(const G3& g, const T* __restrict__ cells, unsigned c, int (&at)[3], unsigned& s) {
+    if (c >= g.C) return 0u;
+    const unsigned r = c / (unsigned)g.m[0];
+    at[0] = (int)(c - r * (unsigned)g.m[0]);
+    at[1] = (int)(r % (unsigned)g.m[1]);
+    at[2] = (int)(r / (unsigned)g.m[1]);
+    s = sidx3(g, at[0], at[1], at[2]);
+    unsigned n = 0;
+    while (n < kSlots3 && !is_empty(__ldg(slot3(cells, g, s, (int)n)))) ++n;   // slots fill from 0
+    return n;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kExportB) k_export_count3(const G3 g, const T* __restrict__ cells, unsigned* __restrict__ counts) {
+    int at[3];
+    unsigned s, total;
+    block_prefix(export_cell3(g, cells, blockIdx.x * kExportB + threadIdx.x, at, s), total);
+    if (threadIdx.x == 0) counts[blockIdx.x] = total;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kExportB) k_export3(const G3 g, const T* __restrict__ cells, const unsigned* __restrict__ counts,
+                                                      double w0, double w1, double w2, double L0, double L1, double L2,
+                                                      const Dev3* __restrict__ st, unsigned limit, double* __restrict__ xyz) {
+    int at[3];
+    unsigned s, total;
+    const unsigned n = export_cell3(g, cells, blockIdx.x * kExportB + threadIdx.x, at, s);
+    unsigned p = counts[blockIdx.x] + block_prefix(n, total);
+    for (unsigned j = 0; j < n && p < limit; ++j, ++p) {
+        const T* q = slot3(cells, g, s, (int)j);
+        xyz[3 * (size_t)p] = global_coordinate(st->origin[0], at[0], w0, (double)__ldg(q), L0);
+        xyz[3 * (size_t)p + 1] = global_coordinate(st->origin[1], at[1], w1, (double)__ldg(q + 4), L1);
+        xyz[3 * (size_t)p + 2] = global_coordinate(st->origin[2], at[2], w2, (double)__ldg(q + 8), L2);
+    }
+}
+
 // Check of a cell image (snapshot load): occupied slots form a prefix of
 // each cell (slot 3 occupied before the secondary half is read), occupied
 // coordinates lie in [0, w) on every axis, empty slots hold kEmpty in all
@@ -614,41 +657,34 @@ void pack3(const hdmc3_t* h, const std::vector<double>& loc, const std::vector<u
             }
 }
 
-void unpack3(const hdmc3_t* h, const std::vector<char>& raw, std::vector<double>& loc, std::vector<uint8_t>& cnt) {
-    const G3& g = h->g;
-    loc.assign((size_t)g.C * kCell3, kEmpty);
-    cnt.assign((size_t)g.C, 0);
+// The raw cells in the canonical layout, written once.
+template <typename T>
+void unpack3(const G3& g, const T* raw, double* loc, uint8_t* cnt) {
     for (int cz = 0; cz < g.m[2]; ++cz)
         for (int cy = 0; cy < g.m[1]; ++cy)
             for (int cx = 0; cx < g.m[0]; ++cx) {
                 const size_t c = ((size_t)cz * g.m[1] + cy) * g.m[0] + cx;
                 const size_t s = sidx3(g, cx, cy, cz);
                 int n = 0;
-                for (int j = 0; j < kSlots3; ++j) {
-                    double v[3];
-                    for (int a = 0; a < 3; ++a) {
-                        const char* src = raw.data() + host_slot3(g, s, j, a) * h->el;
-                        if (h->prec == HDMC_FP64) std::memcpy(&v[a], src, 8);
-                        else {
-                            float f;
-                            std::memcpy(&f, src, 4);
-                            v[a] = f;
-                        }
-                    }
-                    if (v[0] == kEmpty) break;   // slots fill from 0; a secondary half is valid only after a full primary
-                    n = j + 1;
-                    for (int a = 0; a < 3; ++a) loc[(8 * c + j) * 3 + a] = v[a];
+                for (; n < kSlots3; ++n) {
+                    const size_t q = host_slot3(g, s, n, 0);
+                    if ((double)raw[q] == kEmpty) break;   // slots fill from 0; a secondary half is valid only after a full primary
+                    for (int a = 0; a < 3; ++a) loc[(8 * c + n) * 3 + a] = (double)raw[q + 4 * (size_t)a];
                 }
+                for (int i = 3 * n; i < kCell3; ++i) loc[8 * 3 * c + i] = kEmpty;
                 cnt[c] = (uint8_t)n;
             }
 }
 
-int download3(hdmc3_t* h, std::vector<double>& loc, std::vector<uint8_t>& cnt) {
-    int e = finish3(h);
-    std::vector<char> raw((size_t)h->g.C * kCell3 * h->el);
-    const cudaError_t ce = cudaMemcpy(raw.data(), h->cells[h->cur], raw.size(), cudaMemcpyDeviceToHost);
+int download3(hdmc3_t* h, double* loc, uint8_t* cnt) {
+    const int e = finish3(h);
+    const size_t bytes = (size_t)h->g.C * kCell3 * h->el;
+    std::unique_ptr<char[]> raw(new (std::nothrow) char[bytes]);
+    if (!raw) return HDMC_ENOMEM;
+    const cudaError_t ce = cudaMemcpy(raw.get(), h->cells[h->cur], bytes, cudaMemcpyDeviceToHost);
     if (ce != cudaSuccess) return cuda_code(ce);
-    unpack3(h, raw, loc, cnt);
+    if (h->prec == HDMC_FP64) unpack3(h->g, reinterpret_cast<const double*>(raw.get()), loc, cnt);
+    else unpack3(h->g, reinterpret_cast<const float*>(raw.get()), loc, cnt);
     return e;
 }
 
@@ -1215,46 +1251,43 @@ int hdmc3_pressure(hdmc3_t* h, double* betaP_over_rho, double* g_contact, uint64
 
 int hdmc3_get_state(hdmc3_t* h, double* local, uint8_t* counts) {
     if (!h || !local || !counts) return HDMC_EINVAL;
-    std::vector<double> loc;
-    std::vector<uint8_t> cnt;
-    const int e = download3(h, loc, cnt);
-    if (e && e != HDMC_EOVERFLOW) return e;
-    std::memcpy(local, loc.data(), loc.size() * sizeof(double));
-    std::memcpy(counts, cnt.data(), cnt.size());
-    return e;
+    return download3(h, local, counts);
 }
 
 int hdmc3_positions(hdmc3_t* h, double* xyz) {
     if (!h || !xyz) return HDMC_EINVAL;
-    std::vector<double> loc;
-    std::vector<uint8_t> cnt;
-    int e = download3(h, loc, cnt);
+    int e = finish3(h);
     if (e && e != HDMC_EOVERFLOW) return e;
-    Dev3 st;
-    const cudaError_t ce = cudaMemcpy(&st, h->st, sizeof(st), cudaMemcpyDeviceToHost);
-    if (ce != cudaSuccess) return cuda_code(ce);
+    // scratch between sweeps: the idle half of the double buffer (a legal
+    // state has fewer than 2.2 spheres per cell, 53 of its 96 bytes or more)
     const G3& g = h->g;
+    const unsigned nb = (g.C + kExportB - 1) / kExportB;
+    const size_t head = export_counts_bytes(nb), bytes = sizeof(double) * 3 * (size_t)h->N;
+    if (head + bytes > (size_t)g.C * kCell3 * h->el) return HDMC_ENOMEM;
+    unsigned* counts = static_cast<unsigned*>(h->cells[1 - h->cur]);
+    double* out = reinterpret_cast<double*>(static_cast<char*>(h->cells[1 - h->cur]) + head);
     double w[3], L[3];
     for (int a = 0; a < 3; ++a) {
         w[a] = h->prec == HDMC_FP64 ? g.w[a] : (double)g.wf[a];
         L[a] = h->prec == HDMC_FP64 ? h->L[a] : (double)g.m[a] * w[a];
     }
-    int64_t p = 0;
-    for (int cz = 0; cz < g.m[2]; ++cz)
-        for (int cy = 0; cy < g.m[1]; ++cy)
-            for (int cx = 0; cx < g.m[0]; ++cx) {
-                const size_t c = ((size_t)cz * g.m[1] + cy) * g.m[0] + cx;
-                const int cc[3] = {cx, cy, cz};
-                for (int j = 0; j < cnt[c]; ++j) {
-                    if (p >= h->N) return HDMC_EOVERFLOW;
-                    for (int a = 0; a < 3; ++a) {
-                        const double gl = st.origin[a] + ((double)cc[a] * w[a] + loc[(8 * c + j) * 3 + a]);
-                        xyz[3 * p + a] = gl - L[a] * std::floor(gl / L[a]);
-                    }
-                    ++p;
-                }
-            }
-    return e;
+    auto run = [&](auto* cells) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(cells)>>;
+        k_export_count3<T><<<nb, kExportB, 0, h->stream>>>(g, cells, counts);
+        k_export_scan<<<1, kExportB, 0, h->stream>>>(counts, nb);
+        k_export3<T><<<nb, kExportB, 0, h->stream>>>(g, cells, counts, w[0], w[1], w[2], L[0], L[1], L[2], h->st, (unsigned)h->N, out);
+    };
+    if (h->prec == HDMC_FP64) run((const double*)h->cells[h->cur]);
+    else run((const float*)h->cells[h->cur]);
+    unsigned total = 0;
+    int e2 = cuda_code(cudaGetLastError());
+    if (!e2) e2 = cuda_code(cudaMemcpyAsync(&total, counts + nb, sizeof(total), cudaMemcpyDeviceToHost, h->stream));
+    if (!e2) e2 = cuda_code(cudaStreamSynchronize(h->stream));
+    const size_t got = sizeof(double) * 3 * (size_t)std::min<int64_t>(total, h->N);
+    if (!e2) e2 = cuda_code(cudaMemcpyAsync(xyz, out, got, cudaMemcpyDeviceToHost, h->stream));
+    if (!e2) e2 = cuda_code(cudaStreamSynchronize(h->stream));
+    if (e2) return e2;
+    return (int64_t)total > h->N ? HDMC_EOVERFLOW : e;
 }
 
 int hdmc3_counters(hdmc3_t* h, uint64_t out[4]) {

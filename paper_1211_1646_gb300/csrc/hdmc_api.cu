@@ -12,6 +12,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <new>
 #include <utility>
 #include <vector>
@@ -115,13 +116,15 @@ int upload(hdmc_t* h, const HostState& hs) {
     return cuda_code(cudaMemcpy(h->cells[h->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice));
 }
 
-int download(hdmc_t* h, HostState& hs) {
+int download(hdmc_t* h, double* loc, uint8_t* cnt) {
     int e = cuda_code(cudaStreamSynchronize(h->stream));
     if (e) return e;
-    std::vector<char> raw(h->lay.cells);
-    e = cuda_code(cudaMemcpy(raw.data(), h->cells[h->cur], raw.size(), cudaMemcpyDeviceToHost));
+    const size_t bytes = h->desc().cells_bytes();
+    std::unique_ptr<char[]> raw(new (std::nothrow) char[bytes]);
+    if (!raw) return HDMC_ENOMEM;
+    e = cuda_code(cudaMemcpy(raw.get(), h->cells[h->cur], bytes, cudaMemcpyDeviceToHost));
     if (e) return e;
-    unpack(h->desc(), raw, hs);
+    unpack(h->desc(), raw.get(), loc, cnt);
     return HDMC_OK;
 }
 
@@ -522,42 +525,45 @@ int hdmc_psi6(hdmc_t* h, double r_cut, double out[4], double* psi) {
 int hdmc_positions(hdmc_t* h, double* xy, int32_t* cell) {
     if (!h || !xy) return HDMC_EINVAL;
     if (h->nstrips) return HDMC_EINVAL;   // strips sweep in two phases (hdmc_strip_*)
-    HostState hs;
-    int e = download(h, hs);
-    DevState ds;
-    if (!e) e = read_devstate(h, ds);
-    if (e) return e;
+    // scratch between sweeps: the idle half of the double buffer, or where the
+    // coordinates of a crowded binary32 state do not fit it, a buffer of this call
     const Geometry& g = h->g;
-    const double wx = h->prec == HDMC_FP64 ? g.wx : (double)g.wxf;
-    const double wy = h->prec == HDMC_FP64 ? g.wy : (double)g.wyf;
-    const double Lx = h->prec == HDMC_FP64 ? h->Lx : (double)g.mx * wx;
-    const double Ly = h->prec == HDMC_FP64 ? h->Ly : (double)g.my * wy;
-    int64_t p = 0;
-    for (int cy = 0; cy < g.my; ++cy)
-        for (int cx = 0; cx < g.mx; ++cx) {
-            const int64_t c = (int64_t)cy * g.mx + cx;
-            for (int j = 0; j < hs.cnt[c]; ++j) {
-                if (p >= h->N) return HDMC_EOVERFLOW;
-                double gx = ds.origin[0] + ((double)cx * wx + hs.loc[2 * (4 * c + j)]);
-                double gy = ds.origin[1] + ((double)cy * wy + hs.loc[2 * (4 * c + j) + 1]);
-                gx = gx - Lx * std::floor(gx / Lx);
-                gy = gy - Ly * std::floor(gy / Ly);
-                xy[2 * p] = gx;
-                xy[2 * p + 1] = gy;
-                if (cell) cell[p] = (int32_t)c;
-                ++p;
-            }
-        }
-    return p == h->N ? HDMC_OK : HDMC_EOVERFLOW;
+    const unsigned nb = export_blocks(g);
+    const size_t head = export_counts_bytes(nb), xy_bytes = sizeof(double) * 2 * (size_t)h->N;
+    const size_t need = head + xy_bytes + sizeof(int32_t) * (size_t)h->N;
+    char* buf = static_cast<char*>(h->cells[h->cur ^ 1]);
+    int e = HDMC_OK;
+    if (need > h->lay.cells) e = cuda_code(cudaMalloc((void**)&buf, need));
+    if (e) return e;
+    unsigned* counts = reinterpret_cast<unsigned*>(buf);
+    double* out = reinterpret_cast<double*>(buf + head);
+    int32_t* out_cell = reinterpret_cast<int32_t*>(buf + head + xy_bytes);
+    ExportCtx x;
+    x.wx = h->prec == HDMC_FP64 ? g.wx : (double)g.wxf;
+    x.wy = h->prec == HDMC_FP64 ? g.wy : (double)g.wyf;
+    x.Lx = h->prec == HDMC_FP64 ? h->Lx : (double)g.mx * x.wx;
+    x.Ly = h->prec == HDMC_FP64 ? h->Ly : (double)g.my * x.wy;
+    x.limit = (unsigned)h->N;
+    const LaunchCtx c = h->ctx(h->stream);
+    if (h->prec == HDMC_FP64) launch_export_f64(c, h->cells[h->cur], x, counts, out, out_cell);
+    else launch_export_f32(c, h->cells[h->cur], x, counts, out, out_cell);
+    unsigned total = 0;
+    e = cuda_code(cudaGetLastError());
+    if (!e) e = cuda_code(cudaMemcpyAsync(&total, counts + nb, sizeof(total), cudaMemcpyDeviceToHost, h->stream));
+    if (!e) e = cuda_code(cudaStreamSynchronize(h->stream));
+    const size_t got = (size_t)std::min<int64_t>(total, h->N);
+    if (!e) e = cuda_code(cudaMemcpyAsync(xy, out, sizeof(double) * 2 * got, cudaMemcpyDeviceToHost, h->stream));
+    if (!e && cell) e = cuda_code(cudaMemcpyAsync(cell, out_cell, sizeof(int32_t) * got, cudaMemcpyDeviceToHost, h->stream));
+    if (!e) e = cuda_code(cudaStreamSynchronize(h->stream));
+    if (need > h->lay.cells) cudaFree(buf);
+    if (e) return e;
+    return (int64_t)total == h->N ? HDMC_OK : HDMC_EOVERFLOW;
 }
 
 int hdmc_get_state(hdmc_t* h, double* local, uint8_t* counts) {
     if (!h) return HDMC_EINVAL;
-    HostState hs;
-    int e = download(h, hs);
+    const int e = download(h, local, counts);
     if (e) return e;
-    if (local) std::memcpy(local, hs.loc.data(), sizeof(double) * hs.loc.size());
-    if (counts) std::memcpy(counts, hs.cnt.data(), hs.cnt.size());
     return check_device(h);
 }
 

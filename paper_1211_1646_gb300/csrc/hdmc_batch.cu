@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <new>
 #include <tuple>
 #include <vector>
@@ -414,14 +415,12 @@ int hdmc_batch_get_state(hdmc_batch_t* b, int r, double* local, uint8_t* counts)
     int e = check_batch(b);
     if (e) return e;
     const SysDesc& d = b->sys[r];
-    std::vector<char> raw(d.cells_bytes());
-    e = cuda_code(cudaMemcpy(raw.data(), (const char*)b->arena[b->cur] + (size_t)b->cell_off[r] * 8 * d.coord_bytes(),
-                             raw.size(), cudaMemcpyDeviceToHost));
+    std::unique_ptr<char[]> raw(new (std::nothrow) char[d.cells_bytes()]);
+    if (!raw) return HDMC_ENOMEM;
+    e = cuda_code(cudaMemcpy(raw.get(), (const char*)b->arena[b->cur] + (size_t)b->cell_off[r] * 8 * d.coord_bytes(),
+                             d.cells_bytes(), cudaMemcpyDeviceToHost));
     if (e) return e;
-    HostState hs;
-    unpack(d, raw, hs);
-    if (local) std::memcpy(local, hs.loc.data(), sizeof(double) * hs.loc.size());
-    if (counts) std::memcpy(counts, hs.cnt.data(), hs.cnt.size());
+    unpack(d, raw.get(), local, counts);
     return HDMC_OK;
 }
 

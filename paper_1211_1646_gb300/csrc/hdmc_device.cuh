@@ -270,6 +270,17 @@ void launch_hist_f64(const LaunchCtx& c, const void* cells);
 void launch_psi6_f64(const LaunchCtx& c, const void* cells, double rc2, double* psi, double* partial, double* out);
 void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long* out);
 
+// Export of the global coordinates (hdmc_export.cuh).
+struct ExportCtx {
+    double wx, wy, Lx, Ly;   // cell widths and box of the coordinate type
+    unsigned limit;          // disks written at most
+};
+constexpr int kExportB = 256;              // canonical cells per block
+unsigned export_blocks(const Geometry& g);
+inline size_t export_counts_bytes(unsigned nb) { return (sizeof(unsigned) * ((size_t)nb + 1) + 255) / 256 * 256; }
+void launch_export_f64(const LaunchCtx& c, const void* cells, const ExportCtx& x, unsigned* counts, double* xy, int32_t* cell);
+void launch_export_f32(const LaunchCtx& c, const void* cells, const ExportCtx& x, unsigned* counts, double* xy, int32_t* cell);
+
 void launch_subsweep_f32(const LaunchCtx& c, void* cells, const SweepDraw* draw, int k);
 
 // Batched stages (one launch over all R replicas).

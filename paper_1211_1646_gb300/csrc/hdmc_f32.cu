@@ -1,4 +1,5 @@
 // Binary32 cell-local coordinates (HDMC_FP32_LOCAL).
+#include "hdmc_export.cuh"
 #include "hdmc_kernels.cuh"
 
 namespace hdmc {
@@ -42,6 +43,10 @@ void launch_psi6_f32(const LaunchCtx& c, const void* cells, double rc2, double* 
 unsigned psi6_blocks(const Geometry& g) {
     const dim3 grid = set_grid(g, dim3(kPsiBX, kPsiBY));
     return grid.x * grid.y * grid.z;
+}
+unsigned export_blocks(const Geometry& g) { return (unsigned)((g.C + kExportB - 1) / kExportB); }
+void launch_export_f32(const LaunchCtx& c, const void* cells, const ExportCtx& x, unsigned* counts, double* xy, int32_t* cell) {
+    launch_export_t<float>(c, cells, x, counts, xy, cell);
 }
 void launch_check_f32(const LaunchCtx& c, const void* cells, unsigned long long* out) {
     launch_check_t<float>(c, cells, out);

@@ -1,4 +1,5 @@
 // Binary64 cell-local coordinates (HDMC_FP64).
+#include "hdmc_export.cuh"
 #include "hdmc_kernels.cuh"
 
 namespace hdmc {
@@ -33,6 +34,9 @@ void launch_shift_f64(const LaunchCtx& c, const void* src, void* dst, const Swee
 void launch_hist_f64(const LaunchCtx& c, const void* cells) { launch_hist_t<double>(c, cells); }
 void launch_psi6_f64(const LaunchCtx& c, const void* cells, double rc2, double* psi, double* partial, double* out) {
     launch_psi6_t<double>(c, cells, rc2, psi, partial, out);
+}
+void launch_export_f64(const LaunchCtx& c, const void* cells, const ExportCtx& x, unsigned* counts, double* xy, int32_t* cell) {
+    launch_export_t<double>(c, cells, x, counts, xy, cell);
 }
 void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long* out) {
     launch_check_t<double>(c, cells, out);

@@ -277,34 +277,32 @@ void pack(const SysDesc& h, const HostState& hs, std::vector<char>& raw) {
         }
 }
 
-void unpack(const SysDesc& h, const std::vector<char>& raw, HostState& hs) {
-    const Geometry& g = h.g;
-    const size_t el = h.prec == HDMC_FP64 ? sizeof(double) : sizeof(float);
-    hs.loc.assign(8 * (size_t)g.C, kEmpty);
-    hs.cnt.assign((size_t)g.C, 0);
+// One pass over the raw cells in the order of the canonical arrays; a half
+// row of a set is contiguous.
+template <typename T>
+static void unpack_cells(const Geometry& g, const T* raw, double* loc, uint8_t* cnt) {
     for (int cy = 0; cy < g.my; ++cy)
-        for (int cx = 0; cx < g.mx; ++cx) {
-            const int64_t c = (int64_t)cy * g.mx + cx;
-            const long long s = storage_index(g, cx, cy);
-            int n = 0;
-            for (int j = 0; j < kSlots; ++j) {
-                double x, y;
-                if (h.prec == HDMC_FP64) {
-                    std::memcpy(&x, raw.data() + (8 * s + j) * el, el);
-                    std::memcpy(&y, raw.data() + (8 * s + 4 + j) * el, el);
-                } else {
-                    float fx, fy;
-                    std::memcpy(&fx, raw.data() + (8 * s + j) * el, el);
-                    std::memcpy(&fy, raw.data() + (8 * s + 4 + j) * el, el);
-                    x = fx;
-                    y = fy;
+        for (int p = 0; p < 2; ++p) {
+            const T* q = raw + 8 * storage_index(g, p, cy);
+            for (int hx = 0; hx < g.hx; ++hx, q += 8) {
+                const int64_t c = (int64_t)cy * g.mx + 2 * hx + p;
+                int n = 0;
+                for (int j = 0; j < kSlots; ++j) {
+                    const bool used = q[j] >= T(0);
+                    if (used) n = j + 1;
+                    if (loc) {
+                        loc[8 * c + 2 * j] = used ? (double)q[j] : kEmpty;
+                        loc[8 * c + 2 * j + 1] = used ? (double)q[4 + j] : kEmpty;
+                    }
                 }
-                if (x >= 0.0) n = j + 1;
-                hs.loc[2 * (4 * c + j)] = x >= 0.0 ? x : kEmpty;
-                hs.loc[2 * (4 * c + j) + 1] = x >= 0.0 ? y : kEmpty;
+                if (cnt) cnt[c] = (uint8_t)n;
             }
-            hs.cnt[c] = (uint8_t)n;
         }
+}
+
+void unpack(const SysDesc& h, const void* raw, double* loc, uint8_t* cnt) {
+    if (h.prec == HDMC_FP64) unpack_cells(h.g, static_cast<const double*>(raw), loc, cnt);
+    else unpack_cells(h.g, static_cast<const float*>(raw), loc, cnt);
 }
 
 // ---- Sec. 4 pressure fit -------------------------------------------------------

@@ -40,7 +40,8 @@ bool any_overlap(const SysDesc& d, const HostState& hs);
 int start_state(const SysDesc& d, HostState& hs);   // hexagonal start, binned and checked
 int state_from_local(const SysDesc& d, const double* local, const uint8_t* counts, HostState& hs);
 void pack(const SysDesc& d, const HostState& hs, std::vector<char>& raw);
-void unpack(const SysDesc& d, const std::vector<char>& raw, HostState& hs);
+// device layout -> canonical arrays (loc: 8 doubles per cell, cnt: one byte; each nullable)
+void unpack(const SysDesc& d, const void* raw, double* loc, uint8_t* cnt);
 void squared_edges(double sigma, double* E);          // kHistBins + 1 values
 double poly_intercept(const std::vector<double>& t, const std::vector<double>& y, int deg);
 double pressure_from_hist(const SysDesc& d, const unsigned long long* hist, int64_t n_samples, double* g_contact);
