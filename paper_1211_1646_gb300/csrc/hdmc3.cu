@@ -180,23 +180,25 @@ __global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* __rest
     const bool live = r < g.cq;
     const int Q = (int)blockIdx.y;
     const unsigned s = (unsigned)Q * g.cq + r;
-    const Draw3& dr = table[jd];
+    const int fdir = table[jd].fdir;
+    const double ds = table[jd].ds;
+    const float dsf = table[jd].dsf;
     Shift3<T> P;
-    P.ax = dr.fdir >> 1;
-    const int sgn = (dr.fdir & 1) ? -1 : 1;
+    P.ax = fdir >> 1;
+    const int sgn = (fdir & 1) ? -1 : 1;
     if (sizeof(T) == 8) {
         P.w = (T)sel3(P.ax, g.w[0], g.w[1], g.w[2]);
-        P.sd = sgn > 0 ? (T)dr.ds : (T)-dr.ds;
+        P.sd = sgn > 0 ? (T)ds : (T)-ds;
         P.wprev = (T)sel3(P.ax, g.wprev[0], g.wprev[1], g.wprev[2]);
     } else {
         P.w = (T)sel3(P.ax, g.wf[0], g.wf[1], g.wf[2]);
-        P.sd = sgn > 0 ? (T)dr.dsf : (T)-dr.dsf;
+        P.sd = sgn > 0 ? (T)dsf : (T)-dsf;
         P.wprev = (T)sel3(P.ax, g.wprevf[0], g.wprevf[1], g.wprevf[2]);
     }
     P.sw = sgn > 0 ? P.w : -P.w;
     if (s == 0) {
-        if (sizeof(T) == 8) st->origin[P.ax] = sgn > 0 ? __dadd_rn(st->origin[P.ax], dr.ds) : __dsub_rn(st->origin[P.ax], dr.ds);
-        else st->origin[P.ax] += (double)(sgn > 0 ? dr.dsf : -dr.dsf);
+        if (sizeof(T) == 8) st->origin[P.ax] = sgn > 0 ? __dadd_rn(st->origin[P.ax], ds) : __dsub_rn(st->origin[P.ax], ds);
+        else st->origin[P.ax] += (double)(sgn > 0 ? dsf : -dsf);
     }
     // old cell c + f
     const unsigned r1 = g.div0(r), iz = g.div1(r1);

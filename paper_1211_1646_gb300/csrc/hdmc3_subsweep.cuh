@@ -14,10 +14,10 @@
 // per trial coordinate.  One thread per cell, which first gathered the
 // neighbours within reach of its trials into shared memory, took (us per
 // sub-sweep, n_M = 4, before -> now, the latter as programmatic dependents):
-//     216 active cells (N = 2048)       binary32 14.1 ->  4.2   binary64  46.3 ->  5.8
-//   2,197             (N = 16384)                14.4 ->  5.4             45.6 ->  7.9
+//     216 active cells (N = 2048)       binary32 14.1 ->  4.1   binary64  46.3 ->  5.4
+//   2,197             (N = 16384)                14.4 ->  4.7             45.6 ->  7.6
 //  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
-// 132,651             (N = 1,048,576)            39.4 -> 34.1            165.3 -> 80.8
+// 132,651             (N = 1,048,576)            39.4 -> 33.0            165.3 -> 79.8
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -136,12 +136,12 @@ struct Pair3 {
 template <typename T>
 __device__ __forceinline__ void ld2(const T* p, T& a, T& b);
 template <> __device__ __forceinline__ void ld2(const float* p, float& a, float& b) {
-    const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+    const float2 v = *reinterpret_cast<const float2*>(p);
     a = v.x;
     b = v.y;
 }
 template <> __device__ __forceinline__ void ld2(const double* p, double& a, double& b) {
-    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 v = *reinterpret_cast<const double2*>(p);
     a = v.x;
     b = v.y;
 }
@@ -149,13 +149,13 @@ template <typename T>
 __device__ __forceinline__ Pair3 pair_at(const T* p, float sx, float sy, float sz, T& x2) {
     T x0, x1, y0, y1, z0, z1;
     if constexpr (sizeof(T) == 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 v = *reinterpret_cast<const float4*>(p);
         x0 = v.x;
         x1 = v.y;
         x2 = v.z;
     } else {
         ld2(p, x0, x1);
-        x2 = __ldg(p + 2);
+        x2 = p[2];
     }
     ld2(p + 4, y0, y1);
     ld2(p + 8, z0, z1);
@@ -266,9 +266,10 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     const int lane = threadIdx.x & 31, grp = lane / G, L = lane % G, gb = grp * G;
     const unsigned gm = (G == 32 ? kFull : ((1u << G) - 1u) << gb);   // lanes of my group
     const unsigned below = gm & ((1u << lane) - 1u);                    // those before me
-    const Draw3& dr = table[jd];
-    const int Q = dr.perm[k];
-    const uint32_t sweep = dr.sweep;
+    // the draw table, read through L2 ahead of pdl_wait
+    const Draw3* dr = table + jd;
+    const uint32_t sweep = __ldcg(&dr->sweep);
+    const int Q = (int)((__ldcg(reinterpret_cast<const uint32_t*>(dr->perm) + (k >> 2)) >> (8 * (k & 3))) & 0xFFu);
     const unsigned s = (blockIdx.x * (kSubB3 / 32) + threadIdx.x / 32) * W::kCells + grp;
     const bool live = s < g.cq;
     const unsigned r1 = g.div0(s), ix = s - r1 * (unsigned)g.h[0];
@@ -277,6 +278,46 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     const int cx = 2 * (int)ix + (Q & 1), cy = 2 * (int)iy + ((Q >> 1) & 1), cz = 2 * (int)iz + (Q >> 2);
     const uint32_t c = ((uint32_t)cz * (uint32_t)g.m[1] + (uint32_t)cy) * (uint32_t)g.m[0] + (uint32_t)cx;
     const unsigned sown = (unsigned)checked_cell(g.check, live ? ax.x[1] + ax.y[1] + ax.z[1] : 0u, g.C);
+
+    // the first trial directions, while the previous kernel's last blocks run
+    const uint32_t setbits = (uint32_t)Q << 24;
+    unsigned have = 0, used = 0;   // directions kept so far, lane blocks used
+    auto keep = [&](bool need, const typename S::Draw& d) {
+        const bool k0 = need && d.keep[0], k1 = need && d.keep[1];
+        const unsigned b0 = __ballot_sync(kFull, k0), b1 = __ballot_sync(kFull, k1);
+        const unsigned pos = have + __popc(b0 & below) + __popc(b1 & below);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            if (k0) sw.dir[pos % W::kRing][q][grp] = d.u[0][q];
+            if (k1) sw.dir[(pos + k0) % W::kRing][q][grp] = d.u[1][q];
+        }
+        have += __popc(b0 & gm) + __popc(b1 & gm);
+    };
+    auto draw = [&](unsigned upto) {
+#pragma unroll 1
+        for (;;) {
+            const bool need = live && have < upto;
+            if (!__any_sync(kFull, need)) break;
+            typename S::Draw d;
+            S::attempts(g, sweep, c, (kDomTrial << 28) | setbits, used + L, d);
+            keep(need, d);
+            used += need ? G : 0;
+        }
+        __syncwarp();
+    };
+    // first round: the group's last lane draws the first word of the shuffle
+    // stream instead, the others the first G - 1 lane blocks
+    uint32_t word;
+    {
+        typename S::Draw d;
+        const bool last = L == G - 1;
+        word = S::attempts(g, sweep, c, ((last ? kDomShuffle : kDomTrial) << 28) | setbits, last ? 0u : (uint32_t)L, d);
+        keep(live && !last, d);
+        used = G - 1;
+        word = __shfl_sync(kFull, word, gb + G - 1);
+    }
+    draw((unsigned)min(kDir3, g.nsel));
+    pdl_wait();   // what comes before depends on the draw table alone
 
     // own spheres: the primary half's slots L, L + G
     constexpr int NO = G < 4 ? 4 / G : 1;
@@ -331,45 +372,6 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
             neighbour(0, sn, (float)dx * g.wf[0], (float)dy * g.wf[1], (float)dz * g.wf[2]);
         }
     }
-
-    // the first trial directions, while the loads are under way
-    const uint32_t setbits = (uint32_t)Q << 24;
-    unsigned have = 0, used = 0;   // directions kept so far, lane blocks used
-    auto keep = [&](bool need, const typename S::Draw& d) {
-        const bool k0 = need && d.keep[0], k1 = need && d.keep[1];
-        const unsigned b0 = __ballot_sync(kFull, k0), b1 = __ballot_sync(kFull, k1);
-        const unsigned pos = have + __popc(b0 & below) + __popc(b1 & below);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (k0) sw.dir[pos % W::kRing][q][grp] = d.u[0][q];
-            if (k1) sw.dir[(pos + k0) % W::kRing][q][grp] = d.u[1][q];
-        }
-        have += __popc(b0 & gm) + __popc(b1 & gm);
-    };
-    auto draw = [&](unsigned upto) {
-#pragma unroll 1
-        for (;;) {
-            const bool need = live && have < upto;
-            if (!__any_sync(kFull, need)) break;
-            typename S::Draw d;
-            S::attempts(g, sweep, c, (kDomTrial << 28) | setbits, used + L, d);
-            keep(need, d);
-            used += need ? G : 0;
-        }
-        __syncwarp();
-    };
-    // first round: the group's last lane draws the first word of the shuffle
-    // stream instead, the others the first G - 1 lane blocks
-    uint32_t word;
-    {
-        typename S::Draw d;
-        const bool last = L == G - 1;
-        word = S::attempts(g, sweep, c, ((last ? kDomShuffle : kDomTrial) << 28) | setbits, last ? 0u : (uint32_t)L, d);
-        keep(live && !last, d);
-        used = G - 1;
-        word = __shfl_sync(kFull, word, gb + G - 1);
-    }
-    draw((unsigned)min(kDir3, g.nsel));
 
     // own cell: number of spheres, slots 4..7 when slot 3 is occupied
     int n = 0;
@@ -435,7 +437,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         int dx, dy, dz;
         const T* p = cells + primary3(ax.at(g, number(__ffs(has2) - 1), dx, dy, dz));
         f23 = pair23_at(p, (float)dx * g.wf[0], (float)dy * g.wf[1], (float)dz * g.wf[2]);
-        more |= !is_empty(__ldg(p + 3)) ? 0x80000000u : 0u;
+        more |= !is_empty(p[3]) ? 0x80000000u : 0u;
     }
     const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots3 && __any_sync(kFull, n > G);
     __syncwarp();
@@ -596,7 +598,6 @@ template <typename T, int G>
 __global__ void __launch_bounds__(kSubB3, G == 2 ? 12 : G == 4 ? 16 : G == 8 ? 20 : 24) k_sub3(const G3 g, T* __restrict__ cells, const Draw3* __restrict__ table, int jd,
                                                  int k, unsigned long long* __restrict__ ctr) {
     pdl_release();
-    pdl_wait();
     sub3_cells<T, G>(g, cells, table, jd, k, ctr);
 }
 

@@ -213,12 +213,13 @@ int set_rows(hdmc_batch_t* b, int rows) {
 }
 
 void enqueue_batch_sweeps(hdmc_batch_t* b, cudaStream_t s, int K, int parity, bool track) {
-    const BatchCtx c = b->ctx(s);
+    BatchCtx c = b->ctx(s);   // launches as in a single system: programmatic dependents after the first sub-sweep
     launch_draws_batch(s, b->reps, b->sts, b->table, b->R, K);
     for (int j = 0; j < K; ++j) {
         void* a = b->arena[parity ^ (j & 1)];
         void* o = b->arena[parity ^ (j & 1) ^ 1];
         for (int k = 0; k < 4; ++k) {
+            c.pdl = j > 0 || k > 0;
             if (b->prec == HDMC_FP64) launch_subsweep_f64_batch(c, a, b->table, j, k);
             else launch_subsweep_f32_batch(c, a, b->table, j, k, track);
         }

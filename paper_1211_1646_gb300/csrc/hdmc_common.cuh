@@ -22,6 +22,17 @@ namespace hdmc {
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The set and the sweep number of sub-sweep k of a sweep.  Read through L2:
+// a programmatic dependent reads them before pdl_wait (the draws kernel
+// completed before the first kernel of the run started).  One read a warp: the
+// shift, with four times the warps and four reads each, took 31 instead of 12
+// us this way, queueing at one L2 slice, and waits first.
+__device__ __forceinline__ void set_and_sweep(const SweepDraw* draw, int k, int& Q, uint32_t& sweep) {
+    const uint4 w = __ldcg(reinterpret_cast<const uint4*>(draw));   // sweep, fdir, perm, dsf
+    sweep = w.x;
+    Q = (int)((w.z >> (8 * k)) & 0xFFu);
+}
+
 constexpr int kDirChunk = 8;   // trial directions drawn ahead per thread (binary32 sub-sweep)
 constexpr int kDirRows = kDirChunk + 2;   // rows of its buffer: a one-pass draw keeps up to two more
 
@@ -87,8 +98,10 @@ template <typename T> struct Cell { T x[4], y[4]; };
 // later); cells are 32-byte aligned (256-byte aligned buffers, 32-byte
 // cells).  Binary64 cells use four 128-bit accesses, which measured faster
 // in the binary64 kernels.
-// The _ro loads take the read-only path: only for cells the kernel does
-// not write.  The loads are volatile: each stays where it is written.
+// The _ro loads take the read-only path: only for cells that nothing writes
+// from the kernel's start on -- not after a pdl_wait that is not the kernel's
+// first statement, since the assembler may move read-only loads ahead of it.
+// The loads are volatile: each stays where it is written.
 __device__ __forceinline__ void load_cell(const float* p, Cell<float>& c) {
     asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=f"(c.x[0]), "=f"(c.x[1]), "=f"(c.x[2]), "=f"(c.x[3]), "=f"(c.y[0]), "=f"(c.y[1]), "=f"(c.y[2]),

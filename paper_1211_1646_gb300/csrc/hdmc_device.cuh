@@ -235,10 +235,10 @@ struct LaunchCtx {
 
 // Launches kernel<<<grid, block>>>(args) on c.stream; with c.pdl, as a
 // programmatic dependent launch: its blocks may be scheduled while the
-// previous kernel of the stream finishes, and wait (griddepcontrol.wait, at
-// the top of every such kernel) for its completion before reading anything.
-template <typename... P, typename... A>
-inline void launch_on(const LaunchCtx& c, void (*kernel)(P...), dim3 grid, dim3 block, A... args) {
+// previous kernel of the stream finishes, and wait (griddepcontrol.wait) for
+// its completion before reading anything but the draw table.
+template <typename C, typename... P, typename... A>
+inline void launch_on(const C& c, void (*kernel)(P...), dim3 grid, dim3 block, A... args) {
     if (!c.pdl) {
         kernel<<<grid, block, 0, c.stream>>>(args...);
         return;
@@ -286,6 +286,7 @@ void launch_subsweep_f32(const LaunchCtx& c, void* cells, const SweepDraw* draw,
 // Batched stages (one launch over all R replicas).
 struct BatchCtx {
     cudaStream_t stream;
+    bool pdl = false;              // launch as a programmatic dependent of the previous kernel
     const ReplicaDesc* reps;
     const unsigned short* sub_map;
     const unsigned short* sh_map;

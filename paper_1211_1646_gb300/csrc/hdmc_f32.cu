@@ -3,25 +3,30 @@
 #include "hdmc_kernels.cuh"
 
 namespace hdmc {
+// A binary32 state of up to 64 MB stays in L2 (129 MB, with its other half)
+// from one sub-sweep to the next.
+constexpr long long kAheadCells = 2000000;
+
 void launch_subsweep_f32(const LaunchCtx& c, void* cells, const SweepDraw* draw, int k) {
     float* a = reinterpret_cast<float*>(cells);
     // blocks of two set rows of 32 cells: in-step faster than one-row blocks
     // (fewer blocks to schedule) and as fast as four-row blocks
     const dim3 grid((unsigned)((c.g.hx + 31) / 32), (unsigned)((c.g.hy + 1) / 2));
+    auto run = [&](auto kernel) { launch_on(c, kernel, grid, dim3(32, 2), c.g, a, draw, k, c.partial); };
+    const int nsel = c.g.nsel;
+    const bool ahead = c.g.C <= kAheadCells;   // see subsweep_f32, phase 1
     if (c.g.dense) {   // cells that often hold three or four disks
-        if (c.g.nsel == 4)
-            launch_on(c, k_subsweep_f32<2, 4, true>, grid, dim3(32, 2), c.g, a, draw, k, c.partial);
-        else if (c.g.nsel == 8)
-            launch_on(c, k_subsweep_f32<2, 8, true>, grid, dim3(32, 2), c.g, a, draw, k, c.partial);
-        else
-            launch_on(c, k_subsweep_f32<2, 0, true>, grid, dim3(32, 2), c.g, a, draw, k, c.partial);
-        return;
+        if (ahead) return nsel == 4 ? run(k_subsweep_f32<2, 4, true>) : nsel == 8 ? run(k_subsweep_f32<2, 8, true>)
+                                                                                  : run(k_subsweep_f32<2, 0, true>);
+        return nsel == 4 ? run(k_subsweep_f32<2, 4, true, false>)
+                         : nsel == 8 ? run(k_subsweep_f32<2, 8, true, false>) : run(k_subsweep_f32<2, 0, true, false>);
     }
+    if (!ahead && nsel == 4) return run(k_subsweep_f32<2, 4, false, false>);
+    if (!ahead && nsel == 8) return run(k_subsweep_f32<2, 8, false, false>);
     // n_M fixed at compile time (directions drawn in one pass, trials
     // unrolled) up to kDirChunk; 100 sweeps of 2,585 active cells at n_M = 7 and
     // their pressure: 2.21 -> 1.70 ms
-    auto run = [&](auto kernel) { launch_on(c, kernel, grid, dim3(32, 2), c.g, a, draw, k, c.partial); };
-    switch (c.g.nsel) {
+    switch (nsel) {
         case 1: return run(k_subsweep_f32<2, 1>);
         case 2: return run(k_subsweep_f32<2, 2>);
         case 3: return run(k_subsweep_f32<2, 3>);
@@ -55,8 +60,8 @@ void launch_check_f32(const LaunchCtx& c, const void* cells, unsigned long long*
 void launch_subsweep_f32_batch(const BatchCtx& c, void* arena, const SweepDraw* draws, int j, int k, bool track) {
     float* a = reinterpret_cast<float*>(arena);
 #define HDMC_SUB_BATCH(ROWS, TRACK, DENSE, NSEL)                                                           \
-    k_subsweep_f32_batch<ROWS, TRACK, DENSE, NSEL><<<c.sub_blocks, dim3(32, ROWS), 0, c.stream>>>(        \
-        c.reps, c.sub_map, a, draws, c.R, j, k, c.partial, c.msd)
+    launch_on(c, k_subsweep_f32_batch<ROWS, TRACK, DENSE, NSEL>, dim3(c.sub_blocks), dim3(32, ROWS),      \
+              c.reps, c.sub_map, a, draws, c.R, j, k, c.partial, c.msd)
     // crowded cells in every replica: the dense kernel; one n_M shared by
     // every replica (4 or 8): the kernel with n_M fixed (the autotuner's
     // tracking launches keep the general one)
@@ -82,13 +87,13 @@ void launch_subsweep_f32_batch(const BatchCtx& c, void* arena, const SweepDraw* 
 }
 
 void launch_shift_batch(const BatchCtx& c, int prec, const void* src, void* dst, const SweepDraw* draws, int j) {
+    const dim3 grid(c.sh_blocks), block(kShiftBX, kShiftBY);
     if (prec == 1)
-        k_shift_batch<float><<<c.sh_blocks, dim3(kShiftBX, kShiftBY), 0, c.stream>>>(
-            c.reps, c.sh_map, reinterpret_cast<const float*>(src), reinterpret_cast<float*>(dst), draws, c.R, j, c.sts);
+        launch_on(c, k_shift_batch<float>, grid, block, c.reps, c.sh_map, reinterpret_cast<const float*>(src),
+                  reinterpret_cast<float*>(dst), draws, c.R, j, c.sts);
     else
-        k_shift_batch<double><<<c.sh_blocks, dim3(kShiftBX, kShiftBY), 0, c.stream>>>(
-            c.reps, c.sh_map, reinterpret_cast<const double*>(src), reinterpret_cast<double*>(dst), draws, c.R, j,
-            c.sts);
+        launch_on(c, k_shift_batch<double>, grid, block, c.reps, c.sh_map, reinterpret_cast<const double*>(src),
+                  reinterpret_cast<double*>(dst), draws, c.R, j, c.sts);
 }
 
 void launch_hist_batch(const BatchCtx& c, int prec, const void* arena) {

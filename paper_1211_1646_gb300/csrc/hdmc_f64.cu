@@ -9,7 +9,8 @@ namespace hdmc {
 // cells (most directions have a third disk) keep two lanes, which hold all
 // slots in registers.  us per sub-sweep in-step at n_M = 4 with 8 / 4 / 2
 // lanes and one thread (before: 8.0, 12.8, 16.2, 17.3, 20.5, 47.9; crowded
-// 19.1, 43.1):
+// 19.1, 43.1), the loads ahead of the draws; with the draws ahead (pdl_wait)
+// the chosen forms take 3.2, 5.2, 5.3, 7.3, 14.6, 36.0; crowded 5.7, 30.3:
 //       270 active cells   3.7 / 4.3 / 5.7 / 6.7
 //     8,976                5.9 / 6.4 / 8.3 / 9.0
 //    18,270                8.4 / 6.6 / 8.9 / 10.8
@@ -44,7 +45,7 @@ void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long*
 
 void launch_subsweep_f64_batch(const BatchCtx& c, void* arena, const SweepDraw* draws, int j, int k) {
     constexpr int G = 2;
-    k_subsweep_f64_batch<G><<<c.sub_blocks, dim3(32, 4 * G), 0, c.stream>>>(c.reps, c.sub_map, reinterpret_cast<double*>(arena),
-                                                                            draws, c.R, j, k, c.partial);
+    launch_on(c, k_subsweep_f64_batch<G>, dim3(c.sub_blocks), dim3(32, 4 * G), c.reps, c.sub_map,
+              reinterpret_cast<double*>(arena), draws, c.R, j, k, c.partial);
 }
 }  // namespace hdmc

@@ -644,17 +644,22 @@ static __global__ void __launch_bounds__(256) k_psi6_sum(const double* __restric
 // counters and histogram.  Replica r's cells start at cell rd.cell_off of
 // the arena; its sweep draws of chunk position j sit at draws[j*R + r].
 // NSEL > 0: every replica makes NSEL trial moves per cell update.
+// Launched as programmatic dependents like the single system's kernels, the
+// directions drawn ahead: 64 sweeps of the 64-replica workload at n_M = 8 28.6
+// -> 25.9 ms (27.1 with the loads first), of 16 replicas of 1024 to 8192 disks
+// 1.37 -> 1.08 ms.
 template <int ROWS, bool TRACK, bool DENSE = false, int NSEL = 0>
 static __global__ void __launch_bounds__(32 * ROWS, DENSE ? (16 / ROWS > 0 ? 16 / ROWS : 1) : 20 / ROWS)
 k_subsweep_f32_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
                      float* __restrict__ arena, const SweepDraw* __restrict__ draws, int R, int j, int k,
                      unsigned long long* __restrict__ partial, double* __restrict__ msd) {
+    pdl_release();
     __shared__ float2 sdir[kDirRows][32 * ROWS];
     const int r = map[blockIdx.x];
     const ReplicaDesc* rd = reps + r;
     const int local = (int)blockIdx.x - rd->sub_block0;
     const int by = local / rd->sub_gx, bx = local - by * rd->sub_gx;
-    subsweep_f32<ROWS, NSEL, TRACK, DENSE>(rd->g, arena + 8 * rd->cell_off, draws + (size_t)j * R + r, k, bx, by,
+    subsweep_f32<ROWS, NSEL, TRACK, DENSE, true>(rd->g, arena + 8 * rd->cell_off, draws + (size_t)j * R + r, k, bx, by,
                                      partial + 4 * (rd->part_off + local), sdir, msd + r);
 }
 
@@ -664,6 +669,7 @@ static __global__ void __launch_bounds__(128 * G)
 k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
                      double* __restrict__ arena, const SweepDraw* __restrict__ draws, int R, int j, int k,
                      unsigned long long* __restrict__ partial) {
+    pdl_release();
     __shared__ Warp2<G> sw[4 * G];
     const int r = map[blockIdx.x];
     const ReplicaDesc* rd = reps + r;
@@ -679,6 +685,8 @@ __global__ void __launch_bounds__(kShiftBX * kShiftBY)
 k_shift_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
               const T* __restrict__ src, T* __restrict__ dst, const SweepDraw* __restrict__ draws, int R, int j,
               DevState* __restrict__ sts) {
+    pdl_release();
+    pdl_wait();
     const int r = map[blockIdx.x];
     const ReplicaDesc* rd = reps + r;
     const int local = (int)blockIdx.x - rd->sh_block0;

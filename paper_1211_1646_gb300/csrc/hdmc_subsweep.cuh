@@ -13,12 +13,19 @@ namespace hdmc {
 
 // ---- binary32 sub-sweep: the cell updates of Alg. 1 / Alg. 2 ---------------------------
 // One thread per active cell of set Q = draw->perm[k]; block 32 x ROWS over
-// the set's half-resolution grid.  Phases, ordered so that the latency of the
-// cell loads is covered by work that does not need them:
-//   1. issue the loads of the own cell and of the 8 neighbouring cells (they
-//      belong to other sets and are not written by this launch);
-//   2. draw the trial directions of the cell's stream (kept attempts staged
-//      in shared memory, kDirChunk at a time);
+// the set's half-resolution grid.  Phases:
+//   1. draw the trial directions of the cell's stream (kept attempts staged
+//      in shared memory, kDirChunk at a time).  They depend on the draw table
+//      alone, so with AHEAD they come before pdl_wait: as a programmatic
+//      dependent the kernel draws them while the previous kernel's last blocks
+//      run.  Where the state does not fit L2 the loads go first and the draws
+//      cover their latency.  us per sub-sweep in-step at n_M = 4, loads first
+//      -> draws first: 270 active cells 1.84 -> 1.69, 9k 3.6 -> 2.6, 73k 4.05 ->
+//      3.2, 293k 10.6 either way (n_M = 8 16.4 -> 15.8), 1.15M (147 MB) 37.3 ->
+//      38.9; crowded 9k 4.0 -> 2.7.  Draws first only in the blocks of the
+//      first wave: 11.0 at 293k;
+//   2. load the own cell and the 8 neighbouring cells (they belong to other
+//      sets and are not written by this launch);
 //   3. shuffle the disks with the draw in field 0 of the stream's first block,
 //      translate neighbour slot pair (0,1) into this cell's frame as packed
 //      binary32 pairs, flag (warp-uniformly) the directions where some lane
@@ -96,38 +103,40 @@ __device__ __forceinline__ uint4 philox_rk(uint4 c, const PhiloxKeys& K) {
 // while the lane has fewer than WANT kept attempts.  A lane may keep more
 // than WANT (at most max(8, WANT + 2) <= kDirRows), in rows of sdir that no
 // trial reads; the stream is not continued.
-template <int ROWS, int WANT>
-__device__ __forceinline__ void draw_directions_once(const PhiloxKeys& K, uint32_t sweep, uint32_t cell, uint32_t c2,
-                                                     const uint32_t F0[6], float2 (*__restrict__ sdir)[32 * ROWS],
-                                                     int tid) {
+template <int ROWS, int WANT> struct DrawOnce {
     static_assert(WANT <= kDirChunk && kDirRows >= kDirChunk + 2 && kDirRows >= 8, "sdir rows");
-    constexpr uint32_t kOnce = WANT == 1 ? 2 : 3;
-    int have = 0;
-    auto attempt = [&](uint32_t a, uint32_t b) {
+    static constexpr uint32_t kOnce = WANT == 1 ? 2 : 3;   // blocks without a loop
+    const PhiloxKeys K;
+    uint32_t sweep, cell, c2;
+    float2 (*sdir)[32 * ROWS];
+    int tid, have;
+    __device__ __forceinline__ DrawOnce(const Geometry& g, uint32_t sweep_, uint32_t cell_, uint32_t c2_,
+                                        float2 (*sdir_)[32 * ROWS], int tid_)
+        : K(g.key0, g.key1), sweep(sweep_), cell(cell_), c2(c2_), sdir(sdir_), tid(tid_), have(0) {}
+    __device__ __forceinline__ void attempt(uint32_t a, uint32_t b) {
         const float u = sym21(a), v = sym21(b);
         if (__fmaf_rn(u, u, __fmul_rn(v, v)) < 1.0f) {
             sdir[have][tid] = make_float2(u, v);
             ++have;
         }
-    };
-    attempt(F0[2], F0[3]);
-    attempt(F0[4], F0[5]);
+    }
+    // The attempts of one block; returns its field 0 (block 0: the shuffle draw).
+    __device__ __forceinline__ uint32_t block(uint32_t blk) {
+        uint32_t F[6];
+        fields21(philox_rk<(WANT > 4)>(make_uint4(sweep, cell, c2, blk), K), F);
+        if (blk != 0u) attempt(F[0], F[1]);
+        attempt(F[2], F[3]);
+        attempt(F[4], F[5]);
+        return F[0];
+    }
+    __device__ __forceinline__ uint32_t all() {   // returns field 0 of block 0
+        const uint32_t f0 = block(0u);
 #pragma unroll
-    for (uint32_t blk = 1; blk < kOnce; ++blk) {   // every lane needs block 1, nearly every warp block 2
-        uint32_t F[6];
-        fields21(philox_rk<(WANT > 4)>(make_uint4(sweep, cell, c2, blk), K), F);
-        attempt(F[0], F[1]);
-        attempt(F[2], F[3]);
-        attempt(F[4], F[5]);
+        for (uint32_t blk = 1; blk < kOnce; ++blk) block(blk);
+        for (uint32_t blk = kOnce; have < WANT; ++blk) block(blk);
+        return f0;
     }
-    for (uint32_t blk = kOnce; have < WANT; ++blk) {
-        uint32_t F[6];
-        fields21(philox_rk<(WANT > 4)>(make_uint4(sweep, cell, c2, blk), K), F);
-        attempt(F[0], F[1]);
-        attempt(F[2], F[3]);
-        attempt(F[4], F[5]);
-    }
-}
+};
 
 // Phases 3 and 4 for a warp whose cells hold at most two disks each: nearly
 // every warp with cells of about sigma (none of a 256^2-disk fluid at phi =
@@ -162,7 +171,7 @@ __device__ __forceinline__ void trials_of_two(const Geometry& g, const float* __
     // slot pair (2,3) of flagged direction c, translated
     auto pair23 = [&](int c, f2x& x, f2x& y) {
         const float2* p = reinterpret_cast<const float2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-        const float2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
+        const float2 x23 = p[1], y23 = p[3];
         const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
         x = add2(pk(x23.x, x23.y), pk(sx, sx));
         y = add2(pk(y23.x, y23.y), pk(sy, sy));
@@ -222,22 +231,42 @@ __device__ __forceinline__ void trials_of_two(const Geometry& g, const float* __
 // cells just below sqrt(2) sigma): slot pairs (2,3) of all 8 neighbours stay
 // in registers and every trial tests all of them, instead of the flagged
 // directions' pairs being read again in every trial.
-template <int ROWS, int NSEL, bool TRACK = false, bool DENSE = false>
+template <int ROWS, int NSEL, bool TRACK, bool DENSE, bool AHEAD>
 __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restrict__ cells,
                                              const SweepDraw* __restrict__ draw, int k, int bx, int by,
                                              unsigned long long* __restrict__ bpart,
                                              float2 (*__restrict__ sdir)[32 * ROWS], double* msd = nullptr) {
     const int nsel = NSEL > 0 ? NSEL : g.nsel;
     const int tid = threadIdx.y * 32 + threadIdx.x;
-    const int Q = draw->perm[k];
-    const uint32_t sweep = draw->sweep;
+    int Q;
+    uint32_t sweep;
+    set_and_sweep(draw, k, Q, sweep);
     const int hx = bx * 32 + threadIdx.x;
     const int hy = by * ROWS + threadIdx.y;
     const int cx = 2 * hx + (Q & 1), cy = 2 * hy + (Q >> 1);
     const bool live = hx < g.hx && hy < g.hy && cy >= g.ylo && cy <= g.yhi;
     const Neighbourhood nbh(g, Q, hx, hy, live);
+    const uint32_t cell = (uint32_t)(cy + g.row0) * (uint32_t)g.mx + (uint32_t)cx;   // global cell number
+    const uint32_t c2 = (kDomTrial << 28) | ((uint32_t)Q << 24);
+    uint32_t f0;   // shuffle draw: field 0 of block 0
+    constexpr bool kFixed = NSEL > 0 && NSEL <= kDirChunk;
+    DrawOnce<ROWS, kFixed ? NSEL : 1> D(g, sweep, cell, c2, sdir, tid);
+    uint32_t F[6];
+    uint32_t blk = 0;
+    int pnext = 1;               // next attempt: field pair 1 of block 0 (fields 2,3)
+    auto draw_first = [&] {
+        if constexpr (kFixed) {
+            f0 = D.all();
+        } else {
+            fields21(philox4x32_10(make_uint4(sweep, cell, c2, 0u), g.key0, g.key1), F);
+            f0 = F[0];
+            draw_directions<ROWS>(g, sweep, cell, c2, F, blk, pnext, min(kDirChunk, nsel), sdir, tid);   // refills F
+        }
+    };
+    if (AHEAD) draw_first();
+    pdl_wait();
 
-    // 1. loads
+    // 2. loads
     Cell<float> own;
 #pragma unroll
     for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = (float)kEmpty;
@@ -254,30 +283,14 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
         if (live) {
             const float* p = cell_at(cells, nbh.index(g, c, hx, hy));
             Cell<float> a;
-            load_cell_ro(p, a);   // one 256-bit load; slots 0, 1 and x2 are used
+            load_cell(p, a);   // one 256-bit load; slots 0, 1 and x2 are used
             n01[c] = make_float4(a.x[0], a.x[1], a.y[0], a.y[1]);
             n2[c] = a.x[2];
             if (DENSE) n23[c] = make_float4(a.x[2], a.x[3], a.y[2], a.y[3]);
         }
     }
 
-    // 2. directions of the first chunk (the cell's trial stream)
-    const uint32_t cell = (uint32_t)(cy + g.row0) * (uint32_t)g.mx + (uint32_t)cx;   // global cell number
-    const uint32_t c2 = (kDomTrial << 28) | ((uint32_t)Q << 24);
-    uint32_t F[6];
-    uint32_t f0;                 // shuffle draw: field 0 of block 0
-    uint32_t blk = 0;
-    int pnext = 1;               // next attempt: field pair 1 of block 0 (fields 2,3)
-    if constexpr (NSEL > 0 && NSEL <= kDirChunk) {
-        const PhiloxKeys K(g.key0, g.key1);
-        fields21(philox_rk<(NSEL > 4)>(make_uint4(sweep, cell, c2, 0u), K), F);
-        f0 = F[0];
-        draw_directions_once<ROWS, NSEL>(K, sweep, cell, c2, F, sdir, tid);
-    } else {
-        fields21(philox4x32_10(make_uint4(sweep, cell, c2, 0u), g.key0, g.key1), F);
-        f0 = F[0];
-        draw_directions<ROWS>(g, sweep, cell, c2, F, blk, pnext, min(kDirChunk, nsel), sdir, tid);   // refills F
-    }
+    if (!AHEAD) draw_first();   // covers the latency of the loads
 
     // 3. cell contents
     const int n = (own.x[0] >= 0.f) + (own.x[1] >= 0.f) + (own.x[2] >= 0.f) + (own.x[3] >= 0.f);
@@ -343,7 +356,7 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
         if (!DENSE && dir23) {
             const int c = __ffs(dir23) - 1;
             const float2* p = reinterpret_cast<const float2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-            const float2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
+            const float2 x23 = p[1], y23 = p[3];
             const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
             fx23 = add2(pk(x23.x, x23.y), pk(sx, sx));
             fy23 = add2(pk(y23.x, y23.y), pk(sy, sy));
@@ -389,7 +402,7 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
                 for (uint32_t m = more23; m; m &= m - 1) {   // warp-uniform, rarely taken
                     const int c = __ffs(m) - 1;
                     const float2* p = reinterpret_cast<const float2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-                    const float2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
+                    const float2 x23 = p[1], y23 = p[3];
                     const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
                     z = zpair(tx2, ty2, add2(pk(x23.x, x23.y), pk(sx, sx)), add2(pk(y23.x, y23.y), pk(sy, sy)), ns2);
                     acc |= lo32(z) | hi32(z);
@@ -430,17 +443,16 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
     add_block_counters<ROWS>(n_tr, n_acc, n_leave, bpart);
 }
 
-template <int ROWS, int NSEL, bool DENSE = false>
+template <int ROWS, int NSEL, bool DENSE = false, bool AHEAD = true>
 static __global__ void __launch_bounds__(32 * ROWS, DENSE ? 16 / ROWS : 20 / ROWS)
 k_subsweep_f32(const Geometry g, float* __restrict__ cells, const SweepDraw* __restrict__ draw, int k,
                unsigned long long* __restrict__ partial) {
     pdl_release();
-    pdl_wait();
     __shared__ float2 sdir[kDirRows][32 * ROWS];
     // counters of the tile that holds this block (shared by the blocks of a
     // tile: atomic adds)
     const long long slot = (long long)(blockIdx.y * ROWS / kCounterRows) * gridDim.x + blockIdx.x;
-    subsweep_f32<ROWS, NSEL, false, DENSE>(g, cells, draw, k, blockIdx.x, blockIdx.y, partial + 4 * slot, sdir);
+    subsweep_f32<ROWS, NSEL, false, DENSE, AHEAD>(g, cells, draw, k, blockIdx.x, blockIdx.y, partial + 4 * slot, sdir);
 }
 
 }  // namespace hdmc

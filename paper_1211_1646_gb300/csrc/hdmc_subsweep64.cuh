@@ -72,37 +72,13 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
     static_assert(NSEL <= kDirChunk && kDirRows64 >= kDirChunk && kDirRows64 >= straight_blocks(kDirChunk), "sdir rows");
     const int nsel = NSEL > 0 ? NSEL : g.nsel;
     const int tid = threadIdx.y * 32 + threadIdx.x;
-    const int Q = draw->perm[k];
-    const uint32_t sweep = draw->sweep;
+    int Q;
+    uint32_t sweep;
+    set_and_sweep(draw, k, Q, sweep);
     const int hx = bx * 32 + threadIdx.x, hy = by * ROWS + threadIdx.y;
     const int cx = 2 * hx + (Q & 1), cy = 2 * hy + (Q >> 1);
     const bool live = hx < g.hx && hy < g.hy && cy >= g.ylo && cy <= g.yhi;
     const Neighbourhood nbh(g, Q, hx, hy, live);
-
-    Cell<double> own;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = kEmpty;
-    double* ownp = cell_at(cells, nbh.own(g, hx, hy));
-    if (live) load_cell(ownp, own);
-    // slots 0, 1 of the neighbours as packed binary32 pairs in this cell's
-    // frame; directions with a third disk flagged (all 24 loads ahead of the
-    // first use need registers that spill: 37.8 -> 40.0 us)
-    f2x qx[8], qy[8];
-    uint32_t mine = 0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        qx[c] = pk(kFar, kFar);
-        qy[c] = 0;
-        if (live) {
-            const double2* p = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-            const double2 x01 = __ldg(p), y01 = __ldg(p + 2);
-            const double x2 = __ldg(reinterpret_cast<const double*>(p + 1));
-            const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
-            qx[c] = add2(pk(pos_or_far(x01.x), pos_or_far(x01.y)), pk(sx, sx));
-            qy[c] = add2(pk(approx_pos(y01.x), approx_pos(y01.y)), pk(sy, sy));
-            mine |= is_empty(x2) ? 0u : 1u << c;
-        }
-    }
 
     // trial directions: the words of kept attempts (attempt a = block a)
     const uint32_t cell = (uint32_t)(cy + g.row0) * (uint32_t)g.mx + (uint32_t)cx;   // global cell number
@@ -120,6 +96,32 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
         for (uint32_t b = straight_blocks(NSEL); have < NSEL; ++b) attempt(b);
     } else {
         for (const int want = min(kDirChunk, nsel); have < want; ++blk) attempt(blk);
+    }
+    pdl_wait();   // what comes before depends on the draw table alone
+
+    Cell<double> own;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = kEmpty;
+    double* ownp = cell_at(cells, nbh.own(g, hx, hy));
+    if (live) load_cell(ownp, own);
+    // slots 0, 1 of the neighbours as packed binary32 pairs in this cell's
+    // frame; directions with a third disk flagged (all 24 loads ahead of the
+    // first use need registers that spill: 37.8 -> 40.0 us)
+    f2x qx[8], qy[8];
+    uint32_t mine = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        qx[c] = pk(kFar, kFar);
+        qy[c] = 0;
+        if (live) {
+            const double2* p = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
+            const double2 x01 = p[0], y01 = p[2];
+            const double x2 = reinterpret_cast<const double*>(p + 1)[0];
+            const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
+            qx[c] = add2(pk(pos_or_far(x01.x), pos_or_far(x01.y)), pk(sx, sx));
+            qy[c] = add2(pk(approx_pos(y01.x), approx_pos(y01.y)), pk(sy, sy));
+            mine |= is_empty(x2) ? 0u : 1u << c;
+        }
     }
 
     const int n = !is_empty(own.x[0]) + !is_empty(own.x[1]) + !is_empty(own.x[2]) + !is_empty(own.x[3]);
@@ -143,7 +145,7 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
         const uint32_t more23 = dir23 & (dir23 - 1);
         auto pair23 = [&](int c, f2x& x, f2x& y) {
             const double2* p = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-            const double2 x23 = __ldg(p + 1), y23 = __ldg(p + 3);
+            const double2 x23 = p[1], y23 = p[3];
             const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
             x = add2(pk(pos_or_far(x23.x), pos_or_far(x23.y)), pk(sx, sx));
             y = add2(pk(approx_pos(y23.x), approx_pos(y23.y)), pk(sy, sy));
@@ -194,9 +196,9 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
                 }
                 auto slot_hit = [&](int c, int j) {
                     const double* q = cell_at(cells, nbh.index(g, c, hx, hy)) + j;
-                    return !is_empty(__ldg(q)) &&
-                           hit64(g, __dsub_rn(tx, __dadd_rn(__ldg(q), (double)dir_dx(c) * g.wx)),
-                                 __dsub_rn(ty, __dadd_rn(__ldg(q + 4), (double)dir_dy(c) * g.wy)));
+                    return !is_empty(q[0]) &&
+                           hit64(g, __dsub_rn(tx, __dadd_rn(q[0], (double)dir_dx(c) * g.wx)),
+                                 __dsub_rn(ty, __dadd_rn(q[4], (double)dir_dy(c) * g.wy)));
                 };
                 for (; close; close &= close - 1) {
                     const int b = __ffs(close) - 1;
@@ -241,7 +243,6 @@ static __global__ void __launch_bounds__(32 * ROWS, 16 / ROWS)
 k_subsweep_f64(const Geometry g, double* __restrict__ cells, const SweepDraw* __restrict__ draw, int k,
                unsigned long long* __restrict__ partial) {
     pdl_release();
-    pdl_wait();
     __shared__ uint4 sdir[kDirRows64][32 * ROWS];
     // counters of the tile that holds this block (shared: atomic adds)
     subsweep_f64<ROWS, NSEL>(g, cells, draw, k, blockIdx.x, blockIdx.y,
@@ -277,45 +278,13 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
     const int lane = threadIdx.x, grp = lane / G, L = lane % G, gb = grp * G;
     const unsigned gm = ((1u << G) - 1u) << gb;          // lanes of my group
     const unsigned below = gm & ((1u << lane) - 1u);      // those before me
-    const int Q = draw->perm[k];
-    const uint32_t sweep = draw->sweep;
+    int Q;
+    uint32_t sweep;
+    set_and_sweep(draw, k, Q, sweep);
     const int hx = hx0 + grp;
     const int cx = 2 * hx + (Q & 1), cy = 2 * hy + (Q >> 1);
     const bool live = hx < g.hx && hy < g.hy && cy >= g.ylo && cy <= g.yhi;
     const Neighbourhood nbh(g, Q, hx, hy, live);
-
-    // own slots L, L + G and my neighbour cells (slots 2, 3 where used)
-    double* const ownp = cell_at(cells, nbh.own(g, hx, hy));
-    double own[NO][2];
-#pragma unroll
-    for (int r = 0; r < NO; ++r) {
-        own[r][0] = own[r][1] = kEmpty;
-        if (live && L + r * G < 4) {
-            own[r][0] = ownp[L + r * G];
-            own[r][1] = ownp[4 + L + r * G];
-        }
-    }
-    f2x qx[NC][2], qy[NC][2];
-    uint32_t has2 = 0;   // bit j: my j-th neighbour has a third disk
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        const int c = j * G + L;
-        qx[j][0] = qx[j][1] = pk(kFar, kFar);
-        qy[j][0] = qy[j][1] = 0;
-        if (live) {
-            const double2* q = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
-            const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
-            const double2 x01 = __ldg(q), x23 = __ldg(q + 1), y01 = __ldg(q + 2);
-            qx[j][0] = add2(pk(pos_or_far(x01.x), pos_or_far(x01.y)), pk(sx, sx));
-            qy[j][0] = add2(pk(approx_pos(y01.x), approx_pos(y01.y)), pk(sy, sy));
-            if (!is_empty(x23.x)) {
-                const double2 y23 = __ldg(q + 3);
-                qx[j][1] = add2(pk(approx_pos(x23.x), pos_or_far(x23.y)), pk(sx, sx));
-                qy[j][1] = add2(pk(approx_pos(y23.x), approx_pos(y23.y)), pk(sy, sy));
-                has2 |= 1u << j;
-            }
-        }
-    }
 
     // Trial directions: attempt a = block a of the trial stream, u = sym52(w0,
     // w1), v = sym52(w2, w3), kept iff u*u + v*v < 1; trial t takes the t-th
@@ -358,6 +327,41 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
     uint32_t word = attempt(live && !shuf, ((shuf ? kDomShuffle : kDomTrial) << 28) | setbits, shuf ? 0u : (uint32_t)L);
     used = G - 1;
     word = __shfl_sync(kFull, word, gb + G - 1);
+    fill(0, min(kDir2, g.nsel));
+    pdl_wait();   // what comes before depends on the draw table alone
+
+    // own slots L, L + G and my neighbour cells (slots 2, 3 where used)
+    double* const ownp = cell_at(cells, nbh.own(g, hx, hy));
+    double own[NO][2];
+#pragma unroll
+    for (int r = 0; r < NO; ++r) {
+        own[r][0] = own[r][1] = kEmpty;
+        if (live && L + r * G < 4) {
+            own[r][0] = ownp[L + r * G];
+            own[r][1] = ownp[4 + L + r * G];
+        }
+    }
+    f2x qx[NC][2], qy[NC][2];
+    uint32_t has2 = 0;   // bit j: my j-th neighbour has a third disk
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        const int c = j * G + L;
+        qx[j][0] = qx[j][1] = pk(kFar, kFar);
+        qy[j][0] = qy[j][1] = 0;
+        if (live) {
+            const double2* q = reinterpret_cast<const double2*>(cell_at(cells, nbh.index(g, c, hx, hy)));
+            const float sx = (float)dir_dx(c) * g.wxf, sy = (float)dir_dy(c) * g.wyf;
+            const double2 x01 = q[0], x23 = q[1], y01 = q[2];
+            qx[j][0] = add2(pk(pos_or_far(x01.x), pos_or_far(x01.y)), pk(sx, sx));
+            qy[j][0] = add2(pk(approx_pos(y01.x), approx_pos(y01.y)), pk(sy, sy));
+            if (!is_empty(x23.x)) {
+                const double2 y23 = q[3];
+                qx[j][1] = add2(pk(approx_pos(x23.x), pos_or_far(x23.y)), pk(sx, sx));
+                qy[j][1] = add2(pk(approx_pos(y23.x), approx_pos(y23.y)), pk(sy, sy));
+                has2 |= 1u << j;
+            }
+        }
+    }
 
     // own cell
     int n = 0;
@@ -369,7 +373,7 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
             sw.own[L + r * G][1][grp] = own[r][1];
         }
     }
-    fill(0, min(kDir2, g.nsel));
+    __syncwarp();
     // shuffle (Alg. 1): slot j of the shuffled cell is old slot (perm >> 4j) & 3
     unsigned perm = 0x3210u;
     if (n >= 2 && !(g.flags & kNoParticleShuffle)) {
@@ -457,8 +461,8 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
                 close &= close - 1u;
                 const int c = (b >> 2) * G + L;
                 const double* q = cell_at(cells, nbh.index(g, c, hx, hy)) + (b & 3);
-                hit |= hit64(g, __dsub_rn(tx, __dadd_rn(__ldg(q), (double)dir_dx(c) * g.wx)),
-                             __dsub_rn(ty, __dadd_rn(__ldg(q + 4), (double)dir_dy(c) * g.wy)));
+                hit |= hit64(g, __dsub_rn(tx, __dadd_rn(q[0], (double)dir_dx(c) * g.wx)),
+                             __dsub_rn(ty, __dadd_rn(q[4], (double)dir_dy(c) * g.wy)));
             }
         }
         const bool overlap = (__ballot_sync(kFull, hit) & gm) != 0;
@@ -495,7 +499,6 @@ static __global__ void __launch_bounds__(32 * kCounterRows, 5)
 k_subsweep_lanes(const Geometry g, double* __restrict__ cells, const SweepDraw* __restrict__ draw, int k, int tiles,
                  unsigned long long* __restrict__ partial) {
     pdl_release();
-    pdl_wait();
     __shared__ Warp2<G> sw[kCounterRows];
     const int hx0 = (int)blockIdx.x * (32 / G), hy = (int)blockIdx.y * kCounterRows + (int)threadIdx.y;
     // counters of the tile (32 columns x kCounterRows rows, `tiles` in a row) that holds these cells
