@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(kDrawChunk3) k_draws3(const G3 g, Draw3* table
 // Cell shift (Alg. 4) along one of three axes: new cell c keeps the spheres
 // of old c that stay inside it (slot order), then takes those of old c+f
 // that leave c+f, re-expressed in c's frame and clamped into [0, w).  One
-// thread per new cell, grid (cells of a set, set).
+// thread per new cell, grid (cells of a set, set); plain loads, as in two
+// dimensions.
 //
 // The new cell is put together in registers; a slot is looked at only if some
 // lane of the warp has a sphere in it, since nine cells in ten hold at most
@@ -150,7 +151,7 @@ template <typename T> struct Shift3 {
     }
     // The same for all slots, from memory to memory.
     template <bool MIGRANTS>
-    __device__ __forceinline__ void copy(const G3& g, const T* __restrict__ src, unsigned from, T* __restrict__ dst, unsigned to,
+    __device__ __forceinline__ void copy(const G3& g, const T* src, unsigned from, T* dst, unsigned to,
                                          int& k) const {
 #pragma unroll 1
         for (int j = 0; j < kSlots3; ++j) {
@@ -172,7 +173,7 @@ template <typename T> struct Shift3 {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* __restrict__ src, T* __restrict__ dst,
+__global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* src, T* dst,
                                                      const Draw3* __restrict__ table, int jd, Dev3* st) {
     pdl_release();
     pdl_wait();

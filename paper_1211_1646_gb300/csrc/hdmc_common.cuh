@@ -99,8 +99,8 @@ template <typename T> struct Cell { T x[4], y[4]; };
 // cells).  Binary64 cells use four 128-bit accesses, which measured faster
 // in the binary64 kernels.
 // The _ro loads take the read-only path: only for cells that nothing writes
-// from the kernel's start on -- not after a pdl_wait that is not the kernel's
-// first statement, since the assembler may move read-only loads ahead of it.
+// from the kernel's start on -- not for what a pdl_wait waits for, since the
+// assembler may move read-only loads ahead of it.
 // The loads are volatile: each stays where it is written.
 __device__ __forceinline__ void load_cell(const float* p, Cell<float>& c) {
     asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"

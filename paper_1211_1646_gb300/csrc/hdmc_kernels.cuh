@@ -21,6 +21,9 @@ namespace hdmc {
 // lands in exactly one cell (Sec. 3.2).  A re-expressed value that rounds
 // onto the upper edge is clamped below it.
 //
+// The cells are read with plain loads (src is not __restrict__): the assembler
+// may move read-only loads ahead of pdl_wait.
+//
 // Grid origin O += f*ds (one thread per shift), binary64: ds added or
 // subtracted (the same rounding as adding -ds).  Kept out of line so that
 // the binary64 instruction stays in that one thread.
@@ -158,7 +161,7 @@ template <> struct ShiftParams<float> {
 };
 
 template <typename T>
-__device__ __forceinline__ void shift_cells(const Geometry& g, const T* __restrict__ src, T* __restrict__ dst,
+__device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* dst,
                                             const SweepDraw* __restrict__ draw, DevState* __restrict__ st, int bx,
                                             int by, int q) {
     const int hx = bx * kShiftBX + threadIdx.x;
@@ -175,8 +178,8 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* __restri
     const int ncy = ax ? wrap(cy + sgn, g.my) : cy;
     const long long idx = (long long)q * g.cq + (long long)hy * g.hx + hx;
     Cell<T> o, b, r;
-    load_cell_ro(src + 8 * idx, o);
-    load_cell_ro(src + 8 * storage_index(g, ncx, ncy), b);
+    load_cell(src + 8 * idx, o);
+    load_cell(src + 8 * storage_index(g, ncx, ncy), b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) r.x[j] = r.y[j] = T(kEmpty);
     int kept = 0;
@@ -216,7 +219,7 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* __restri
 
 template <typename T>
 __global__ void __launch_bounds__(kShiftBX * kShiftBY)
-k_shift(const Geometry g, const T* __restrict__ src, T* __restrict__ dst, const SweepDraw* __restrict__ draw,
+k_shift(const Geometry g, const T* src, T* dst, const SweepDraw* __restrict__ draw,
         DevState* __restrict__ st) {
     pdl_release();
     pdl_wait();
@@ -683,7 +686,7 @@ k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short*
 template <typename T>
 __global__ void __launch_bounds__(kShiftBX * kShiftBY)
 k_shift_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
-              const T* __restrict__ src, T* __restrict__ dst, const SweepDraw* __restrict__ draws, int R, int j,
+              const T* src, T* dst, const SweepDraw* __restrict__ draws, int R, int j,
               DevState* __restrict__ sts) {
     pdl_release();
     pdl_wait();
