@@ -181,6 +181,15 @@ __global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* src, T
     const bool live = r < g.cq;
     const int Q = (int)blockIdx.y;
     const unsigned s = (unsigned)Q * g.cq + r;
+    T ox[4], oy[4], oz[4], bx[4], by[4], bz[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ox[j] = bx[j] = (T)kEmpty;
+    if (live) {   // before the draw is known
+        const T* p = src + primary3(s);
+        ld4(p, ox);
+        ld4(p + 4, oy);
+        ld4(p + 8, oz);
+    }
     const int fdir = table[jd].fdir;
     const double ds = table[jd].ds;
     const float dsf = table[jd].dsf;
@@ -209,17 +218,10 @@ __global__ void __launch_bounds__(kShiftB3) k_shift3(const G3 g, const T* src, T
     else if (P.ax == 1) ny = wrap3(ny + sgn, g.m[1]);
     else nz = wrap3(nz + sgn, g.m[2]);
     const unsigned sb = live ? sidx3(g, nx, ny, nz) : 0u;
-    T ox[4], oy[4], oz[4], bx[4], by[4], bz[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) ox[j] = bx[j] = (T)kEmpty;
     if (live) {
-        const T* p = src + primary3(s);
         const T* q = src + primary3(sb);
-        ld4(p, ox);
         ld4(q, bx);
-        ld4(p + 4, oy);
         ld4(q + 4, by);
-        ld4(p + 8, oz);
         ld4(q + 8, bz);
     }
     T rx[4], ry[4], rz[4];

@@ -14,10 +14,10 @@
 // per trial coordinate.  One thread per cell, which first gathered the
 // neighbours within reach of its trials into shared memory, took (us per
 // sub-sweep, n_M = 4, before -> now, the latter as programmatic dependents):
-//     216 active cells (N = 2048)       binary32 14.1 ->  4.1   binary64  46.3 ->  5.4
-//   2,197             (N = 16384)                14.4 ->  4.7             45.6 ->  7.6
+//     216 active cells (N = 2048)       binary32 14.1 ->  4.1   binary64  46.3 ->  5.1
+//   2,197             (N = 16384)                14.4 ->  4.7             45.6 ->  7.0
 //  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
-// 132,651             (N = 1,048,576)            39.4 -> 33.0            165.3 -> 79.8
+// 132,651             (N = 1,048,576)            39.4 -> 32.9            165.3 -> 77.0
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -46,8 +46,8 @@ __device__ __forceinline__ bool inside_ball(const uint32_t (&w)[6]) {
 //   binary64: consecutive words of the trial stream, six per attempt, three
 //             sym52 variates u = m 2^-52 (m odd, |m| < 2^52); a lane takes
 //             three Philox blocks, two attempts.  The words of a kept
-//             attempt are stored; the trial makes each variate the binary64
-//             with the sign of m and the magnitude 2^52 + |m| (sym52_offset),
+//             attempt are stored, then made into displacements: each variate is
+//             the binary64 with m's sign and magnitude 2^52 + |m| (sym52_offset),
 //             and d u is RN(d u) = fma(d 2^-52, 2^52 + |m|, -d), with the
 //             sign of m: the product is exactly d + d |m| 2^-52, so one
 //             instruction of the slow binary64 pipe rounds d u correctly.
@@ -115,12 +115,13 @@ template <> struct Sub3<double> {
         }
         return w[0];
     }
-    static __device__ __forceinline__ double trial(const G3& g, double x, double words) {
+    static __device__ __forceinline__ double displacement(const G3& g, double words) {
         const double v = sym52_offset((uint32_t)__double2hiint(words), (uint32_t)__double2loint(words));
         const double c = __longlong_as_double(__double_as_longlong(g.d) ^
                                               ((__double_as_longlong(v) & (1ll << 63)) ^ (1ll << 63)));   // -d with v's sign
-        return __dadd_rn(x, __fma_rn(g.d52, v, c));
+        return __fma_rn(g.d52, v, c);
     }
+    static __device__ __forceinline__ double trial(const G3&, double x, double du) { return __dadd_rn(x, du); }
     static __device__ __forceinline__ bool inside(double p, double w) {
         return Prm<double>::ge0(p) && Prm<double>::lt(p, w);
     }
@@ -293,10 +294,11 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         }
         have += __popc(b0 & gm) + __popc(b1 & gm);
     };
-    auto draw = [&](unsigned upto) {
+    // directions t0 .. t0 + want - 1 (binary64: as displacements d u)
+    auto draw = [&](int t0, int want) {
 #pragma unroll 1
         for (;;) {
-            const bool need = live && have < upto;
+            const bool need = live && have < (unsigned)(t0 + want);
             if (!__any_sync(kFull, need)) break;
             typename S::Draw d;
             S::attempts(g, sweep, c, (kDomTrial << 28) | setbits, used + L, d);
@@ -304,6 +306,14 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
             used += need ? G : 0;
         }
         __syncwarp();
+        if constexpr (!S::kExact) {
+#pragma unroll 1
+            for (int i = L; i < 3 * want; i += G) {
+                T& w = sw.dir[(unsigned)(t0 + i / 3) % W::kRing][i % 3][grp];
+                w = S::displacement(g, w);
+            }
+            __syncwarp();
+        }
     };
     // first round: the group's last lane draws the first word of the shuffle
     // stream instead, the others the first G - 1 lane blocks
@@ -316,7 +326,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         used = G - 1;
         word = __shfl_sync(kFull, word, gb + G - 1);
     }
-    draw((unsigned)min(kDir3, g.nsel));
+    draw(0, min(kDir3, g.nsel));
     pdl_wait();   // what comes before depends on the draw table alone
 
     // own spheres: the primary half's slots L, L + G
@@ -442,7 +452,11 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots3 && __any_sync(kFull, n > G);
     __syncwarp();
 
-    // binary64: lane L computes trial coordinate L (two lanes: the first also coordinate 2)
+    // Binary32: every lane computes the trial position.  Binary64, where the
+    // slow pipe's instructions count: lane L computes coordinate L (all three
+    // in every lane: 8.4 instead of 7.0 us at 2,197 active cells).
+    constexpr bool kAll = S::kExact;
+    static_assert(kAll || G >= 4, "one lane per coordinate");
     const int a0 = L < 3 ? L : 0;
     const T w0 = A::w(g, 0), w1 = A::w(g, 1), w2 = A::w(g, 2);
     const T wa = a0 == 0 ? w0 : a0 == 1 ? w1 : w2;
@@ -452,36 +466,31 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
     int i = 0;
 #pragma unroll 1
     for (int t = 0; t < g.nsel; ++t) {
-        if (t > 0 && t % kDir3 == 0) draw((unsigned)min(t + kDir3, g.nsel));
+        if (t > 0 && t % kDir3 == 0) draw(t, min(kDir3, g.nsel - t));
         const int cur = (int)((perm >> (4 * i)) & 7u);
         T(&me)[3][W::kCells] = sw.own[cur];
         const T(&u)[3][W::kCells] = sw.dir[(unsigned)t % W::kRing];
-        float px, py, pz;
+        float px, py, pz;   // estimates of the trial position (binary32: the position)
         bool inside;
-        if constexpr (S::kExact) {
-            px = S::trial(g, me[0][grp], u[0][grp]);
-            py = S::trial(g, me[1][grp], u[1][grp]);
-            pz = S::trial(g, me[2][grp], u[2][grp]);
-            inside = S::inside(px, w0) && S::inside(py, w1) && S::inside(pz, w2);
+        T tp[3];
+        if constexpr (kAll) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) tp[q] = S::trial(g, me[q][grp], u[q][grp]);
+            inside = S::inside(tp[0], w0) && S::inside(tp[1], w1) && S::inside(tp[2], w2);
+            px = S::est(tp[0]);
+            py = S::est(tp[1]);
+            pz = S::est(tp[2]);
         } else {
             const T p = S::trial(g, me[a0][grp], u[a0][grp]);
-            bool in = S::inside(p, wa);
             const float pf = S::est(p);
             px = __shfl_sync(kFull, pf, gb);
             py = __shfl_sync(kFull, pf, gb + 1);
-            if constexpr (G >= 4) {
-                pz = __shfl_sync(kFull, pf, gb + 2);
-            } else {
-                const T pc = S::trial(g, me[2][grp], u[2][grp]);
-                in = in && S::inside(pc, w2);
-                pz = S::est(pc);
-                if (L == 0) sw.trial[2][grp] = pc;
-            }
-            constexpr unsigned m3 = G >= 4 ? 7u : 3u;
-            inside = ((__ballot_sync(kFull, in) >> gb) & m3) == m3;
+            pz = __shfl_sync(kFull, pf, gb + 2);
+            inside = ((__ballot_sync(kFull, S::inside(p, wa)) >> gb) & 7u) == 7u;
             if (L < 3) sw.trial[L][grp] = p;
             __syncwarp();
         }
+        auto position = [&](int q) { return kAll ? tp[q] : sw.trial[q][grp]; };   // the exact one
         const f2x px2 = pk(px, px), py2 = pk(py, py), pz2 = pk(pz, pz);
         uint32_t sure = 0, maybe = 0;   // sign bits: certainly / possibly overlapping
 #pragma unroll
@@ -512,7 +521,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
                     const float ex = px - S::est(q[0]), ey = py - S::est(q[1]), ez = pz - S::est(q[2]);
                     const float r2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
                     if (r2 < g.band_lo || r2 > g.band_hi) return r2 < g.band_lo;
-                    return A::hit(g, sw.trial[0][grp] - q[0], sw.trial[1][grp] - q[1], sw.trial[2][grp] - q[2]);
+                    return A::hit(g, position(0) - q[0], position(1) - q[1], position(2) - q[2]);
                 }
             };
             if (L < n && L != cur) hit |= own_hit(L);
@@ -530,14 +539,14 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
             }
             const f2x y = add2(ztriple(f23, px2, py2, pz2, lo2), band2);
             close |= ((lo32(y) >> 31) << 30) | (hi32(y) & 0x80000000u);
-            const T tp[3] = {sw.trial[0][grp], sw.trial[1][grp], sw.trial[2][grp]};
+            const T at[3] = {position(0), position(1), position(2)};
             while (close) {
                 const int b = __ffs(close) - 1;
                 close &= close - 1u;
                 const int j = b >= 30 ? __ffs(has2) - 1 : b >> 1, slot = b >= 30 ? b - 28 : b & 1;
                 int dx, dy, dz;
                 const unsigned sn = ax.at(g, number(j), dx, dy, dz);
-                hit |= slots_hit(g, cells, sn, dx, dy, dz, slot, slot, tp);
+                hit |= slots_hit(g, cells, sn, dx, dy, dz, slot, slot, at);
             }
         }
         if (more && !hit && inside) {   // rare: slots 2..7 of further flagged cells, slots 4..7 of the first
@@ -545,29 +554,15 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
                 const int b = __ffs(m) - 1;
                 int dx, dy, dz;
                 const unsigned sn = ax.at(g, number(b == 31 ? __ffs(has2) - 1 : b), dx, dy, dz);
-                T tp[3];
-                if constexpr (S::kExact) {
-                    tp[0] = px;
-                    tp[1] = py;
-                    tp[2] = pz;
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) tp[q] = sw.trial[q][grp];
-                }
-                hit |= slots_hit(g, cells, sn, dx, dy, dz, b == 31 ? 4 : 2, kSlots3 - 1, tp);
+                const T at[3] = {position(0), position(1), position(2)};
+                hit |= slots_hit(g, cells, sn, dx, dy, dz, b == 31 ? 4 : 2, kSlots3 - 1, at);
             }
         }
         const bool overlap = (__ballot_sync(kFull, hit) & gm) != 0;
         if (n > 0 && inside && !overlap) {
             if (L == 0) {
-                if constexpr (S::kExact) {
-                    me[0][grp] = px;
-                    me[1][grp] = py;
-                    me[2][grp] = pz;
-                } else {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) me[q][grp] = sw.trial[q][grp];
-                }
+                for (int q = 0; q < 3; ++q) me[q][grp] = position(q);
             }
             ++n_ac;
         }

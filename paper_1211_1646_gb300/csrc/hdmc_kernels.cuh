@@ -166,19 +166,19 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* 
                                             int by, int q) {
     const int hx = bx * kShiftBX + threadIdx.x;
     const int hy = by * kShiftBY + threadIdx.y;
+    const int cx = 2 * hx + (q & 1), cy = 2 * hy + (q >> 1);
+    const bool live = hx < g.hx && hy < g.hy && cy >= g.slo && cy <= g.shi;   // a strip's halo rows are not its own
+    const long long idx = (long long)q * g.cq + (long long)hy * g.hx + hx;
+    Cell<T> o, b, r;
+    if (live) load_cell(src + 8 * idx, o);   // before the draw is known
     const int fdir = draw->fdir;
     const int ax = fdir >> 1;
     const int sgn = (fdir & 1) ? -1 : 1;
     const ShiftParams<T> P(g, *draw, ax, sgn);
     if (hx == 0 && hy == 0 && q == 0) add_origin(st, ax, sgn, P.origin_ds());
-    if (hx >= g.hx || hy >= g.hy) return;
-    const int cx = 2 * hx + (q & 1), cy = 2 * hy + (q >> 1);
-    if (cy < g.slo || cy > g.shi) return;   // a strip's halo rows are not its own
+    if (!live) return;
     const int ncx = ax ? cx : wrap(cx + sgn, g.mx);
     const int ncy = ax ? wrap(cy + sgn, g.my) : cy;
-    const long long idx = (long long)q * g.cq + (long long)hy * g.hx + hx;
-    Cell<T> o, b, r;
-    load_cell(src + 8 * idx, o);
     load_cell(src + 8 * storage_index(g, ncx, ncy), b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) r.x[j] = r.y[j] = T(kEmpty);
