@@ -240,153 +240,211 @@ k_shift(const Geometry g, const T* src, T* dst, const SweepDraw* __restrict__ dr
 // binary64 distance and bin of 32 queued pairs at a time, so the (slow)
 // binary64 instructions run with every lane busy.  Non-negative doubles
 // order like their bit patterns read as signed integers, so the bin search
-// compares integers.  One thread per cell, grid (set row, set column, set);
-// per-block shared histogram.
+// compares integers.
+//
+// The estimates bind the kernel, so each is made once for the two orders of a
+// pair: a cell looks at itself and at the 12 cells ahead of it (dy > 0, or dy
+// = 0 and dx > 0), and a candidate is queued in both orders, each evaluated
+// with its own roundings.  A cell two steps away is looked at only if some
+// lane has a disk within reach of it (a band of 0.02 sigma with cells of
+// sigma, nowhere with the paper's cells), its corners never.  What is left on
+// the binary64 pipe is seven instructions per queued pair.  A block does four
+// tiles of 32 x 8 cells before it adds its bins to the global ones.  One
+// histogram with its launch, N = 1M: binary32 120 -> 71 us, binary64 241 -> 111
+// us; the paper's cells (N = 1520^2) 196 -> 88 us.
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(double v) { return approx_f32(v); }
 
-constexpr int kHistQueue = 64;   // per-warp candidate queue (< 32 pending + 32 appended)
+// Exact binary32 -> binary64 on the integer pipe (conversions run on the
+// binary64 pipe); subnormal binary32 values, not met in earnest, convert.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
+    if (m < 0x00800000u && m != 0u) return (double)v;
+    const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
 
-// Candidate entry: source lane (5 bits), own slot i (2), neighbour slot j (2),
-// dx + 2 (3), dy + 2 (3).
-__device__ __forceinline__ uint32_t hist_entry(int lane, int b, int dx, int dy) {
+constexpr int kHistQueue = 96;   // per-warp candidate queue (< 32 pending + 64 appended)
+constexpr int kHistTiles = 4;    // tiles of kHistBY set rows of a block
+
+struct HistShared {
+    unsigned int bins[kHistBins];
+    long long edge[kHistBins + 1];   // bit patterns of the squared edges
+    uint32_t queue[kHistBY][kHistQueue];
+    double sx[5], sy[5];             // cell offsets (k - 2) wx, (k - 2) wy
+};
+
+template <typename T>
+__device__ __forceinline__ void hist_begin(const Geometry& g, const double* __restrict__ edges2, HistShared& S) {
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    for (int b = tid; b < kHistBins; b += blockDim.x * blockDim.y) S.bins[b] = 0u;
+    for (int b = tid; b <= kHistBins; b += blockDim.x * blockDim.y) S.edge[b] = __double_as_longlong(edges2[b]);
+    if (tid < 10) {
+        const int k = tid % 5;
+        (tid < 5 ? S.sx : S.sy)[k] = (double)(k - 2) * (tid < 5 ? (double)Prm<T>::wx(g) : (double)Prm<T>::wy(g));
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ void hist_end(HistShared& S, unsigned long long* __restrict__ hist) {
+    __syncthreads();
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    for (int b = tid; b < kHistBins; b += blockDim.x * blockDim.y)
+        if (S.bins[b]) atomicAdd(&hist[b], (unsigned long long)S.bins[b]);
+}
+
+// Candidate entry: source lane (5 bits), its slot i (2), the neighbour's slot
+// j (2), dx + 2 (3), dy (2), 1 if the neighbour's disk comes first (1).
+__device__ __forceinline__ uint32_t hist_entry(int lane, int b, int dx, int dy, int back) {
     return (uint32_t)lane | ((uint32_t)(b >> 2) << 5) | ((uint32_t)(b & 3) << 7) | ((uint32_t)(dx + 2) << 9) |
-           ((uint32_t)(dy + 2) << 12);
+           ((uint32_t)dy << 12) | ((uint32_t)back << 14);
 }
 
 // Bins the first `count` queued pairs, one per lane (warp-uniform call).
 template <typename T>
-__device__ __forceinline__ void hist_flush(const Geometry& g, const T* __restrict__ cells, const uint32_t* sq,
-                                           int count, int q, int bx, int hy, const long long* sEi,
-                                           unsigned int* sh, double wxd, double wyd, float sigf, float inv_drf) {
+__device__ __forceinline__ void hist_flush(const Geometry& g, const T* __restrict__ cells, HistShared& S, const uint32_t* sq,
+                                           int count, int q, int bx, int hy, float sigf, float inv_drf) {
     const int lane = threadIdx.x;
     if (lane >= count) return;
     const uint32_t e = sq[lane];
     const int src = e & 31, i = (e >> 5) & 3, j = (e >> 7) & 3;
-    const int dx = (int)((e >> 9) & 7) - 2, dy = (int)((e >> 12) & 7) - 2;
+    const int dx = (int)((e >> 9) & 7) - 2, dy = (int)((e >> 12) & 3), back = (int)((e >> 14) & 1);
     const int hx = bx * kHistBX + src;
     const int cx = 2 * hx + (q & 1), cy = 2 * hy + (q >> 1);
-    const T* own = cells + 8 * ((long long)q * g.cq + (long long)hy * g.hx + hx);
-    const T* nb = cells + 8 * storage_index(g, wrap(cx + dx, g.mx), wrap(cy + dy, g.my));
-    const double px = (double)__ldg(own + i), py = (double)__ldg(own + 4 + i);
-    const double ex = __dadd_rn((double)__ldg(nb + j), (double)dx * wxd);
-    const double ey = __dadd_rn((double)__ldg(nb + 4 + j), (double)dy * wyd);
-    const double ddx = __dsub_rn(px, ex), ddy = __dsub_rn(py, ey);
+    const T* own = cells + 8 * ((long long)q * g.cq + (long long)hy * g.hx + hx) + i;
+    const T* nb = cells + 8 * storage_index(g, wrap(cx + dx, g.mx), wrap(cy + dy, g.my)) + j;
+    const T* p = back ? nb : own;
+    const T* r = back ? own : nb;
+    const double ex = __dadd_rn(widen(__ldg(r)), S.sx[(back ? -dx : dx) + 2]);
+    const double ey = __dadd_rn(widen(__ldg(r + 4)), S.sy[(back ? -dy : dy) + 2]);
+    const double ddx = __dsub_rn(widen(__ldg(p)), ex), ddy = __dsub_rn(widen(__ldg(p + 4)), ey);
     const double r2 = __dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy));
     const long long r2i = __double_as_longlong(r2);   // r2 >= +0
-    if (r2i >= sEi[0] && r2i < sEi[kHistBins]) {
-        // bin b: sE[b] <= r2 < sE[b+1]; start from a binary32 estimate
+    if (r2i >= S.edge[0] && r2i < S.edge[kHistBins]) {
+        // bin b: edge[b] <= r2 < edge[b+1]; start from a binary32 estimate
         const float r2f = approx_f32(r2);
         int bb = (int)((r2f * rsqrtf(r2f) - sigf) * inv_drf);
         bb = bb < 0 ? 0 : (bb > kHistBins - 1 ? kHistBins - 1 : bb);
-        while (bb > 0 && r2i < sEi[bb]) --bb;
-        while (bb < kHistBins - 1 && r2i >= sEi[bb + 1]) ++bb;
-        atomicAdd(&sh[bb], 1u);
+        while (bb > 0 && r2i < S.edge[bb]) --bb;
+        while (bb < kHistBins - 1 && r2i >= S.edge[bb + 1]) ++bb;
+        atomicAdd(&S.bins[bb], 1u);
     }
 }
 
+// The pairs of one tile of kHistBX x kHistBY cells of set q.
 template <typename T>
-__device__ __forceinline__ void hist_cells(const Geometry& g, const T* __restrict__ cells,
-                                           const double* __restrict__ edges2, unsigned long long* __restrict__ hist,
-                                           int bx, int by, int q) {
-    __shared__ unsigned int sh[kHistBins];
-    __shared__ long long sEi[kHistBins + 1];   // bit patterns of the squared edges
-    __shared__ uint32_t squeue[kHistBY][kHistQueue];
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    for (int b = tid; b < kHistBins; b += blockDim.x * blockDim.y) sh[b] = 0u;
-    for (int b = tid; b <= kHistBins; b += blockDim.x * blockDim.y) sEi[b] = __double_as_longlong(edges2[b]);
-    __syncthreads();
+__device__ __forceinline__ void hist_tile(const Geometry& g, const T* __restrict__ cells, HistShared& S, int bx, int by, int q) {
     const int lane = threadIdx.x;
     const int hx = bx * kHistBX + threadIdx.x;
     const int hy = by * kHistBY + threadIdx.y;
     const int cx = 2 * hx + (q & 1), cy = 2 * hy + (q >> 1);
-    const bool live = hx < g.hx && hy < g.hy && cy >= g.slo && cy <= g.shi;   // own rows only
-    uint32_t* sq = squeue[threadIdx.y];
+    // first disks lie in rows slo..shi; a strip's two halo rows below its own
+    // are looked at for the pairs whose first disk is the one ahead
+    const bool live = hx < g.hx && hy < g.hy && cy >= max(g.slo - 2, 0) && cy <= g.shi;
+    const bool mine = live && cy >= g.slo;
+    uint32_t* sq = S.queue[threadIdx.y];
     Cell<T> own;
 #pragma unroll
     for (int j = 0; j < 4; ++j) own.x[j] = own.y[j] = T(kEmpty);
     if (live) load_cell_ro(cells + 8 * ((long long)q * g.cq + (long long)hy * g.hx + hx), own);
-    const bool any = __any_sync(0xffffffffu, Prm<T>::ge0(own.x[0]));
+    if (!__any_sync(0xffffffffu, Prm<T>::ge0(own.x[0]))) return;
     const bool own23 = __any_sync(0xffffffffu, Prm<T>::ge0(own.x[2]));
-    if (any) {
-        const double wxd = (double)Prm<T>::wx(g), wyd = (double)Prm<T>::wy(g);
-        const float wxf = (float)Prm<T>::wx(g), wyf = (float)Prm<T>::wy(g);
-        const float sigf = (float)g.sigma, inv_drf = (float)(1.0 / (kHistDr * g.sigma));
-        const float rmax = (float)(g.sigma + kHistBins * kHistDr * g.sigma);
-        const float thr = rmax * rmax * 1.001f;   // binary32 estimate margin (estimate error < 1e-6)
-        float ox[4], oy[4];
-        uint32_t occupied = 0;   // bits 4i..4i+3 set when own slot i holds a disk
+    const float wxf = g.wxf, wyf = g.wyf;
+    const float sigf = (float)g.sigma, inv_drf = 1.0f / ((float)kHistDr * sigf);
+    const float rmax = sigf * (1.0f + kHistBins * (float)kHistDr) * (1.0f + 1.0e-6f);
+    const float thr = rmax * rmax * 1.001f;   // binary32 estimate margin (estimate error < 1e-6)
+    const f2x nt = pk(-thr, -thr);
+    float ox[4], oy[4];
+    float minx = 3.0e38f, maxx = -3.0e38f, maxy = -3.0e38f;
+    uint32_t occupied = 0;   // bits 4i..4i+3 set when own slot i holds a disk
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            ox[i] = to_f32(own.x[i]);
-            oy[i] = to_f32(own.y[i]);
-            occupied |= Prm<T>::ge0(own.x[i]) ? (0xFu << (4 * i)) : 0u;
+    for (int i = 0; i < 4; ++i) {
+        ox[i] = to_f32(own.x[i]);
+        oy[i] = to_f32(own.y[i]);
+        if (Prm<T>::ge0(own.x[i])) {
+            occupied |= 0xFu << (4 * i);
+            minx = fminf(minx, ox[i]);
+            maxx = fmaxf(maxx, ox[i]);
+            maxy = fmaxf(maxy, oy[i]);
         }
-        int qn = 0;   // queued candidates of this warp (warp-uniform)
-        for (int dy = -2; dy <= 2; ++dy) {
-            for (int dx = -2; dx <= 2; ++dx) {
-                Cell<T> c;
+    }
+    // is a cell two steps away within reach of some lane's disks (margin far above the binary32 roundings)
+    const float reach = rmax * (1.0f + 1.0e-4f);
+    const bool left2 = __any_sync(0xffffffffu, minx + wxf < reach);
+    const bool right2 = __any_sync(0xffffffffu, 2.0f * wxf - maxx < reach);
+    const bool up2 = __any_sync(0xffffffffu, 2.0f * wyf - maxy < reach);
+    int qn = 0;   // queued candidates of this warp (warp-uniform)
+    for (int dy = 0; dy <= (up2 ? 2 : 1); ++dy) {
+        const int ny = wrap(cy + dy, g.my);
+        const bool theirs = ny >= g.slo && ny <= g.shi;
+        // corner cells begin sqrt(wx^2 + wy^2) >= 1.41 sigma away
+        const int dx0 = dy == 0 ? 0 : (left2 && dy < 2 ? -2 : -1), dx1 = right2 && dy < 2 ? 2 : 1;
+        for (int dx = dx0; dx <= dx1; ++dx) {
+            Cell<T> c;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) c.x[j] = c.y[j] = T(kEmpty);
-                if (live) load_cell_ro(cells + 8 * storage_index(g, wrap(cx + dx, g.mx), wrap(cy + dy, g.my)), c);
-                const float sxf = (float)dx * wxf, syf = (float)dy * wyf;
-                const f2x qx01 = add2(pk(to_f32(c.x[0]), to_f32(c.x[1])), pk(sxf, sxf));
-                const f2x qx23 = add2(pk(to_f32(c.x[2]), to_f32(c.x[3])), pk(sxf, sxf));
-                const f2x qy01 = add2(pk(to_f32(c.y[0]), to_f32(c.y[1])), pk(syf, syf));
-                const f2x qy23 = add2(pk(to_f32(c.y[2]), to_f32(c.y[3])), pk(syf, syf));
-                const f2x nt = pk(-thr, -thr);
-                const bool c23 = __any_sync(0xffffffffu, Prm<T>::ge0(c.x[2]));
-                uint32_t cand = 0;   // bit 4i+j: pair (own i, neighbour slot j) passes the estimate
+            for (int j = 0; j < 4; ++j) c.x[j] = c.y[j] = T(kEmpty);
+            if (live) load_cell_ro(cells + 8 * storage_index(g, wrap(cx + dx, g.mx), ny), c);
+            const float sxf = (float)dx * wxf, syf = (float)dy * wyf;
+            const f2x qx01 = add2(pk(to_f32(c.x[0]), to_f32(c.x[1])), pk(sxf, sxf));
+            const f2x qx23 = add2(pk(to_f32(c.x[2]), to_f32(c.x[3])), pk(sxf, sxf));
+            const f2x qy01 = add2(pk(to_f32(c.y[0]), to_f32(c.y[1])), pk(syf, syf));
+            const f2x qy23 = add2(pk(to_f32(c.y[2]), to_f32(c.y[3])), pk(syf, syf));
+            const bool c23 = __any_sync(0xffffffffu, Prm<T>::ge0(c.x[2]));
+            uint32_t cand = 0;   // bit 4i+j: pair (own i, neighbour slot j) passes the estimate
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (i >= 2 && !own23) continue;
-                    const f2x tx2 = pk(ox[i], ox[i]), ty2 = pk(oy[i], oy[i]);
-                    f2x z = zpair(tx2, ty2, qx01, qy01, nt);
-                    cand |= ((lo32(z) >> 31) << (4 * i)) | ((hi32(z) >> 31) << (4 * i + 1));
-                    if (c23) {
-                        z = zpair(tx2, ty2, qx23, qy23, nt);
-                        cand |= ((lo32(z) >> 31) << (4 * i + 2)) | ((hi32(z) >> 31) << (4 * i + 3));
-                    }
+            for (int i = 0; i < 4; ++i) {
+                if (i >= 2 && !own23) continue;
+                const f2x tx2 = pk(ox[i], ox[i]), ty2 = pk(oy[i], oy[i]);
+                f2x z = zpair(tx2, ty2, qx01, qy01, nt);
+                cand |= ((lo32(z) >> 31) << (4 * i)) | ((hi32(z) >> 31) << (4 * i + 1));
+                if (c23) {
+                    z = zpair(tx2, ty2, qx23, qy23, nt);
+                    cand |= ((lo32(z) >> 31) << (4 * i + 2)) | ((hi32(z) >> 31) << (4 * i + 3));
                 }
-                // empty own slots are excluded (two empty slots sit one cell offset
-                // apart), and no disk is paired with itself
-                cand &= occupied;
-                if (dx == 0 && dy == 0) cand &= ~0x8421u;
-                for (;;) {   // queue the candidates, one per lane and round
-                    const unsigned act = __ballot_sync(0xffffffffu, cand != 0);
-                    if (!act) break;
-                    if (cand) {
-                        const int b = __ffs(cand) - 1;
-                        cand &= cand - 1;
-                        sq[qn + __popc(act & ((1u << lane) - 1u))] = hist_entry(lane, b, dx, dy);
-                    }
-                    qn += __popc(act);
-                    if (qn >= 32) {
-                        __syncwarp();
-                        hist_flush<T>(g, cells, sq, 32, q, bx, hy, sEi, sh, wxd, wyd, sigf, inv_drf);
-                        __syncwarp();
-                        const uint32_t v = lane < qn - 32 ? sq[32 + lane] : 0u;
-                        __syncwarp();
-                        if (lane < qn - 32) sq[lane] = v;
-                        __syncwarp();
-                        qn -= 32;
-                    }
+            }
+            // empty own slots are excluded (two empty slots sit one cell offset
+            // apart), and no disk is paired with itself; pairs inside the cell
+            // appear in both orders already
+            cand &= occupied;
+            const bool self = dx == 0 && dy == 0;
+            if (self) cand &= ~0x8421u;
+            for (;;) {   // queue the candidates, one per lane and round
+                const bool more = cand != 0;
+                if (!__any_sync(0xffffffffu, more)) break;
+                const unsigned fwd = __ballot_sync(0xffffffffu, more && mine);
+                const unsigned rev = __ballot_sync(0xffffffffu, more && theirs && !self);
+                if (more) {
+                    const int b = __ffs(cand) - 1;
+                    cand &= cand - 1;
+                    const unsigned below = (1u << lane) - 1u;
+                    if (mine) sq[qn + __popc(fwd & below)] = hist_entry(lane, b, dx, dy, 0);
+                    if (theirs && !self) sq[qn + __popc(fwd) + __popc(rev & below)] = hist_entry(lane, b, dx, dy, 1);
+                }
+                qn += __popc(fwd) + __popc(rev);
+                while (qn >= 32) {
+                    __syncwarp();
+                    hist_flush<T>(g, cells, S, sq + (qn - 32), 32, q, bx, hy, sigf, inv_drf);
+                    qn -= 32;
+                    __syncwarp();
                 }
             }
         }
-        __syncwarp();
-        hist_flush<T>(g, cells, sq, qn, q, bx, hy, sEi, sh, wxd, wyd, sigf, inv_drf);
     }
-    __syncthreads();
-    for (int b = tid; b < kHistBins; b += blockDim.x * blockDim.y)
-        if (sh[b]) atomicAdd(&hist[b], (unsigned long long)sh[b]);
+    __syncwarp();
+    hist_flush<T>(g, cells, S, sq, qn, q, bx, hy, sigf, inv_drf);
+    __syncwarp();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kHistBX * kHistBY)
 k_hist(const Geometry g, const T* __restrict__ cells, const double* __restrict__ edges2,
        unsigned long long* __restrict__ hist) {
-    hist_cells<T>(g, cells, edges2, hist, blockIdx.x, blockIdx.y, blockIdx.z);
+    __shared__ HistShared S;
+    hist_begin<T>(g, edges2, S);
+#pragma unroll 1
+    for (int t = 0; t < kHistTiles; ++t) hist_tile<T>(g, cells, S, blockIdx.x, blockIdx.y * kHistTiles + t, blockIdx.z);
+    hist_end(S, hist);
 }
 
 // ---- bond-orientational order psi_6 (Sec. 3.3's order parameter) -------------------------
@@ -404,7 +462,7 @@ k_hist(const Geometry g, const T* __restrict__ cells, const double* __restrict__
 // and evaluated 32 at a time, and each lane then adds its own terms up in
 // list order, which is the order dy, dx, slot.  Coordinates are widened to
 // binary64 on the integer pipe.  N = 1M, phi = 0.716, r_cut = 1.4 sigma,
-// binary32, one histogram, pressure and psi_6: 3.25 -> 0.96 ms (the pair loop
+// binary32, psi_6 alone: 3.21 -> 0.80 ms (the pair loop
 // in binary64 over every disk of the 25 cells had 18.7 of 32 lanes active).
 // One thread per cell, one warp per 32 cells of a set row; block sums of
 // {re, im, |psi_6|, n} in a fixed order to partial[4 * block]; k_psi6_sum adds
@@ -412,16 +470,6 @@ k_hist(const Geometry g, const T* __restrict__ cells, const double* __restrict__
 constexpr int kPsiBX = 32, kPsiBY = 4;
 constexpr int kPsiList = 32;    // candidates a lane holds; a cell adds at most 16
 constexpr int kPsiFlat = 256;   // terms evaluated between two rounds of sums
-
-// Exact binary32 -> binary64 on the integer pipe (conversions run on the
-// binary64 pipe); subnormal binary32 values, not met in earnest, convert.
-__device__ __forceinline__ double widen(float v) {
-    const uint32_t u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
-    if (m < 0x00800000u && m != 0u) return (double)v;
-    const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double v) { return v; }
 
 // 2 v exactly as __dmul_rn(2.0, v) gives it, on the integer pipe (v finite
 // and far below overflow; a subnormal v, not met in earnest, is multiplied).
@@ -583,24 +631,53 @@ k_psi6(const Geometry g, const T* __restrict__ cells, double rc2, double* __rest
         }
         psi6_flush<T>(g, cells, s, count, own0, cx - 2 * lane, cy, rc2, shx, shy, are, aim, nb);
     }
-    double t[3] = {0, 0, 0};   // re, im, |psi_6| of this thread's disks
-    int tn = 0;                // their neighbours
-    const long long cc = (long long)cy * g.mx + cx;
+    // psi_6 of the warp's disks, laid end to end so that the divisions and
+    // square roots run with full warps too
+    double t[3] = {0, 0, 0};   // re, im, |psi_6|
+    int tn = 0;                // neighbours
+    {
+        PsiShared& s = sh[threadIdx.y];
+        int total = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (!live || !Prm<T>::ge0(own.x[i])) continue;
-        double pr = 0.0, pi = 0.0;
-        if (nb[i] > 0) {
-            pr = __ddiv_rn(are[i], (double)nb[i]);
-            pi = __ddiv_rn(aim[i], (double)nb[i]);
-            t[0] = __dadd_rn(t[0], pr);
-            t[1] = __dadd_rn(t[1], pi);
-            t[2] = __dadd_rn(t[2], __dsqrt_rn(__dadd_rn(__dmul_rn(pr, pr), __dmul_rn(pi, pi))));
+        for (int i = 0; i < 4; ++i) {
+            const bool used = Prm<T>::ge0(own.x[i]);
+            const unsigned m = __ballot_sync(0xffffffffu, used);
+            if (used) {
+                const int k = total + __popc(m & ((1u << lane) - 1u));
+                s.term[k] = make_double2(are[i], aim[i]);
+                s.flat[k] = (uint32_t)lane | ((uint32_t)i << 5) | ((uint32_t)nb[i] << 8);
+                tn += nb[i];
+            }
+            total += __popc(m);
         }
-        tn += nb[i];
-        if (psi) {
-            psi[(4 * cc + i) * 2] = pr;
-            psi[(4 * cc + i) * 2 + 1] = pi;
+        __syncwarp();
+        for (int k = lane; k < total; k += 32) {
+            const uint32_t e = s.flat[k];
+            const double2 a = s.term[k];
+            const int n = (int)(e >> 8);
+            double pr = 0.0, pi = 0.0;
+            if (n > 0) {
+                pr = __ddiv_rn(a.x, (double)n);
+                pi = __ddiv_rn(a.y, (double)n);
+                t[0] = __dadd_rn(t[0], pr);
+                t[1] = __dadd_rn(t[1], pi);
+                t[2] = __dadd_rn(t[2], __dsqrt_rn(__dadd_rn(__dmul_rn(pr, pr), __dmul_rn(pi, pi))));
+            }
+            if (psi) {
+                const long long cc = (long long)cy * g.mx + (cx - 2 * lane + 2 * (int)(e & 31));
+                const int i = (int)((e >> 5) & 3);
+                psi[(4 * cc + i) * 2] = pr;
+                psi[(4 * cc + i) * 2 + 1] = pi;
+            }
+        }
+        if (psi && live) {   // unused slots
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (!Prm<T>::ge0(own.x[i])) {
+                    const long long cc = (long long)cy * g.mx + cx;
+                    psi[(4 * cc + i) * 2] = 0.0;
+                    psi[(4 * cc + i) * 2 + 1] = 0.0;
+                }
         }
     }
 #pragma unroll
@@ -709,7 +786,10 @@ k_hist_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restr
     const int per_set = rd->hi_gx * rd->hi_gy;
     const int q = local / per_set, rem = local - q * per_set;
     const int by = rem / rd->hi_gx, bx = rem - by * rd->hi_gx;
-    hist_cells<T>(rd->g, arena + 8 * rd->cell_off, edges2, hist + (size_t)r * kHistBins, bx, by, q);
+    __shared__ HistShared S;
+    hist_begin<T>(rd->g, edges2, S);
+    hist_tile<T>(rd->g, arena + 8 * rd->cell_off, S, bx, by, q);
+    hist_end(S, hist + (size_t)r * kHistBins);
 }
 
 // ---- launchers ---------------------------------------------------------------------
@@ -737,7 +817,8 @@ void launch_psi6_t(const LaunchCtx& c, const void* cells, double rc2, double* ps
 template <typename T>
 void launch_hist_t(const LaunchCtx& c, const void* cells) {
     const dim3 block(kHistBX, kHistBY);
-    k_hist<T><<<set_grid(c.g, block), block, 0, c.stream>>>(c.g, reinterpret_cast<const T*>(cells), c.edges2,
+    const dim3 sg = set_grid(c.g, block);
+    k_hist<T><<<dim3(sg.x, (sg.y + kHistTiles - 1) / kHistTiles, sg.z), block, 0, c.stream>>>(c.g, reinterpret_cast<const T*>(cells), c.edges2,
                                                               c.hist);
 }
 
