@@ -18,7 +18,8 @@ namespace hdmc {
 // next kernel of the stream launch once every block of this grid has called
 // it; pdl_wait returns when the previous kernel has completed and its writes
 // are visible (at once for a normal launch).  Kernels launched this way call
-// both before their first memory access.
+// pdl_release first and pdl_wait before their first access to anything that a
+// kernel of the run writes; only the draw table is read ahead of it.
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -252,14 +253,19 @@ __device__ __forceinline__ float pos_or_far(double v) { return is_empty(v) ? kFa
 // Per-block trial counters bpart[{trials, accepted, left, overlap}] of the
 // block's own slot: each warp adds its sums with fire-and-forget atomic
 // adds (no value returned, so nothing waits on the round trip; integer sums
-// do not depend on their order).
+// do not depend on their order).  Lanes that the binary64 decisions of their
+// trials kept apart may arrive separately (measured with n_M = 8 in binary64:
+// a full-mask reduction then summed each part by itself, and only the part
+// with lane 0 was counted), so the sums are over the lanes that are here and
+// the first of them adds.
 template <int ROWS>
 __device__ __forceinline__ void add_block_counters(unsigned int n_tr, unsigned int n_acc, unsigned int n_leave,
                                                    unsigned long long* __restrict__ bpart) {
-    const unsigned a = __reduce_add_sync(0xffffffffu, n_tr);
-    const unsigned b = __reduce_add_sync(0xffffffffu, n_acc);
-    const unsigned c = __reduce_add_sync(0xffffffffu, n_leave);
-    if (threadIdx.x == 0 && a != 0) {
+    const unsigned here = __activemask();
+    const unsigned a = __reduce_add_sync(here, n_tr);
+    const unsigned b = __reduce_add_sync(here, n_acc);
+    const unsigned c = __reduce_add_sync(here, n_leave);
+    if ((int)threadIdx.x == __ffs((int)here) - 1 && a != 0) {
         atomicAdd(bpart + 0, (unsigned long long)a);
         atomicAdd(bpart + 1, (unsigned long long)b);
         atomicAdd(bpart + 2, (unsigned long long)c);
