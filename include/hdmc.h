@@ -153,7 +153,9 @@ int hdmc_psi6(hdmc_t *h, double r_cut, double out[4], double *psi);
  * slot) order: x = O_x + cx*wx + local_x wrapped into [0, mx*wx) (likewise
  * y), O the accumulated grid origin; cells use the binary32 widths in
  * HDMC_FP32_LOCAL mode.  cell (nullable, host int32[N]) receives each disk's
- * canonical cell index.  Synchronises. */
+ * canonical cell index.  The coordinates are put together on the device in the
+ * idle half of the state; where they do not fit it (crowded binary32 cells)
+ * 20 bytes per disk are allocated for the duration of the call.  Synchronises. */
 int hdmc_positions(hdmc_t *h, double *xy, int32_t *cell);
 
 /* Raw state in the canonical layout described above: local[(4c+j)*2 + k]
@@ -518,8 +520,10 @@ typedef struct hdmc3_handle hdmc3_t;
 int hdmc3_create(hdmc3_t **out, int64_t N, double Lx, double Ly, double Lz, double sigma, double d,
                  int nselect, uint64_t seed, int precision, const double *xyz, void *stream);
 
-/* Enqueues n sweeps: one launch of the sweep draws per 64 sweeps, then per
- * sweep eight sub-sweep launches and one cell-shift launch. */
+/* Enqueues n sweeps: per sweep eight sub-sweeps and one cell shift, recorded
+ * once into CUDA graphs of up to 32 sweeps (with the launch of their draws) and
+ * replayed.  On a stream that is being captured the launches themselves are
+ * enqueued. */
 int hdmc3_sweep(hdmc3_t *h, int64_t n);
 
 /* Enqueues one extra cell shift drawn from the stream of explicit shifts. */
