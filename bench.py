@@ -36,6 +36,7 @@ METRIC = "trial moves/sec at N=1M phi=0.716 (1 GB300), FP32-local vs FP64; % HBM
 KERNELS_PER_SWEEP = 5          # 4 sub-sweeps + 1 cell shift
 SPHERE_KERNELS_PER_SWEEP = 9   # 8 sub-sweeps + 1 cell shift (three dimensions)
 GRAPH_CHUNK = 64               # sweeps per recorded graph (one draws kernel each)
+SPHERE_GRAPH_CHUNK = 32        # the same for spheres
 
 
 def parse():
@@ -493,7 +494,7 @@ def run_hdmc(args, rank, world, dist):
                    "step": "%d sweeps (8 sub-sweeps + 1 shift each) + contact histogram + pressure fit"
                            % SWEEPS_PER_STEP,
                    "launches_per_step": SPHERE_KERNELS_PER_SWEEP * SWEEPS_PER_STEP
-                                        + math.ceil(SWEEPS_PER_STEP / GRAPH_CHUNK) + 1}
+                                        + math.ceil(SWEEPS_PER_STEP / SPHERE_GRAPH_CHUNK) + 1}
         for prec, nsteps in (("fp32", args.steps), ("fp64", max(1, args.fp64_steps - 1))):
             s3 = hdmc.System3(w3.N, w3.L, 1.0, w3.d, w3.nselect, seed, prec)
             t3, ms3, p3 = timed_steps(s3, nsteps, 1)
