@@ -47,6 +47,7 @@ struct Geometry {
     float wxf, wyf;        // binary32 cell widths (FP32 path)
     double sigma, sig2;    // sigma, sigma*sigma
     float sig2f;           // binary32 rounding of sigma*sigma
+    float band_lo, band_hi;   // binary32 estimates of r^2 outside decide an overlap (binary64 mode, pair_bands)
     double d;              // maximum trial displacement
     float df;              // its binary32 rounding
     int nsel;              // trial moves per cell and sub-sweep (n_M)
@@ -60,6 +61,18 @@ struct Geometry {
     int slo, shi;          // rows the shift writes and the contact histogram counts
     int dense;             // cells hold 1.3 disks or more on average (binary32 sub-sweep variant)
 };
+
+// Binary64 pair tests are settled by a binary32 estimate of r^2 where it lies
+// outside sigma^2 -+ 2^-15 sigma^2.  Its error is below 3e-6 sigma^2 (coordinates
+// truncated to 24 bits, below 2.9 sigma in the own cell's frame, where r^2 <
+// 1.3 sigma^2), a tenth of the band.  Below sigma = 2^-40 the band no longer
+// shrinks, so that estimates which near the binary32 underflow range decide
+// nothing.
+inline void pair_bands(Geometry& g) {
+    const double band = 0x1p-15 * (g.sig2 > 0x1p-80 ? g.sig2 : 0x1p-80);
+    g.band_lo = (float)(g.sig2 - band);
+    g.band_hi = (float)(g.sig2 + band);
+}
 
 // Device error word bits: a cell received more than its slots (bit 0); a
 // computed cell index fell outside the grid (bit 1, builds with -DHDMC_CHECK

@@ -84,6 +84,7 @@ int make_system(SysDesc& d, int64_t N, double Lx, double Ly, double sigma, doubl
     g.sigma = sigma;
     g.sig2 = sigma * sigma;
     g.sig2f = (float)(sigma * sigma);
+    pair_bands(g);
     g.d = dmove;
     g.df = (float)dmove;
     g.nsel = nselect;

@@ -10,9 +10,10 @@
 //    the estimate of u^2 + v^2 within 2^-18 of 1 are decided in binary64;
 //  - overlap test: positions truncated to binary32 (relative error <= 2^-23),
 //    the squared distance estimated with binary32 pair arithmetic (error
-//    below 3e-6 where it matters, r^2 < 1.3); a candidate counts as certainly
-//    overlapping below sigma^2 - 2^-15 and certainly clear above sigma^2 + 2^-15;
-//    those in between are decided in binary64, slot by slot.
+//    below 3e-6 sigma^2 where it matters, r^2 < 1.3 sigma^2); a candidate counts
+//    as certainly overlapping below sigma^2 (1 - 2^-15) and certainly clear above
+//    sigma^2 (1 + 2^-15) (pair_bands); those in between are decided in binary64,
+//    slot by slot.
 // What is left on the binary64 pipe is one fused multiply-add per variate and
 // one addition per trial coordinate.
 #pragma once
@@ -22,7 +23,6 @@
 
 namespace hdmc {
 
-constexpr float kOverlapBand = 0x1p-15f;
 constexpr float kCircleBand = 0x1p-18f;
 constexpr int kDir2 = 8;   // trial directions drawn ahead per cell
 
@@ -154,8 +154,8 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
         };
         if (dir23) pair23(__ffs(dir23) - 1, fx23, fy23);
         const double d = g.d, d52 = times_2m52(d);
-        const float lim = -(g.sig2f - kOverlapBand);   // certainly overlapping below
-        const f2x lo2 = pk(lim, lim), band2 = pk(-2.0f * kOverlapBand, -2.0f * kOverlapBand);   // possibly: 2 bands above
+        const float lim = -g.band_lo, bands = g.band_hi - g.band_lo;   // certainly overlapping below band_lo
+        const f2x lo2 = pk(lim, lim), band2 = pk(-bands, -bands);      // possibly: up to band_hi
 
         int i = 0;
         auto trial = [&](int tt, auto slots) {
@@ -405,8 +405,8 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
     else any23 = __reduce_or_sync(kFull, has2);
     const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots && __any_sync(kFull, n > G);
 
-    const float lim = -(g.sig2f - kOverlapBand);   // certainly overlapping below
-    const f2x lo2 = pk(lim, lim), band2 = pk(-2.0f * kOverlapBand, -2.0f * kOverlapBand);   // possibly: 2 bands above
+    const float lim = -g.band_lo, bands = g.band_hi - g.band_lo;   // certainly overlapping below band_lo
+    const f2x lo2 = pk(lim, lim), band2 = pk(-bands, -bands);      // possibly: up to band_hi
     unsigned n_ac = 0, n_lf = 0;
     int i = 0, cur = (int)(perm & 3u);
     double px = sw.own[cur][0][grp], py = sw.own[cur][1][grp];   // disk `cur` before its trial
@@ -440,7 +440,7 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
                 const double ox = sw.own[j][0][grp], oy = sw.own[j][1][grp];
                 const float ex = __fsub_rn(txf, approx_pos(ox)), ey = __fsub_rn(tyf, approx_pos(oy));
                 const float z = __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, lim));
-                if (z < 0.f || z >= 2.0f * kOverlapBand) return z < 0.f;
+                if (z < 0.f || z >= bands) return z < 0.f;
                 return hit64(g, __dsub_rn(tx, ox), __dsub_rn(ty, oy));
             };
             if (L < n && L != cur) hit |= own_hit(L);
