@@ -269,7 +269,7 @@ size_t hdmc_batch_workspace_bytes(int R, const int64_t* N, const double* Lx, con
     if ((precision & 0xFF) != HDMC_FP64 && (precision & 0xFF) != HDMC_FP32_LOCAL) return 0;
     std::vector<SysDesc> sys(R);
     for (int r = 0; r < R; ++r)
-        if (make_system(sys[r], N[r], Lx[r], Ly[r], sigma, 0.25, 4, 0, precision)) return 0;
+        if (make_system(sys[r], N[r], Lx[r], Ly[r], sigma, 0.25 * sigma, 4, 0, precision)) return 0;
     return batch_layout(sys, precision & 0xFF).total;
 }
 

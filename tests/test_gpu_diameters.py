@@ -53,6 +53,22 @@ def test_disks(prec, nx, ny, phi, cells, nsel, sweeps, sigma):
     assert np.array_equal(g.pressure()[2], r.histogram(200, 1e-4))
 
 
+@pytest.mark.parametrize("sigma", [0.05, 300.0])
+def test_batch_of_binary64_replicas(sigma):
+    from paper_1211_1646_gb300 import hdmc
+    reps = []
+    for k, (nx, ny, phi) in enumerate([(40, 38, 0.70), (94, 110, 0.68)]):
+        Lx, Ly = W.hex_box(nx, ny, phi)
+        reps.append(W.Workload("r%d" % k, nx * ny, Lx * sigma, Ly * sigma, 0.11 * sigma, 4, 7 + k, 0))
+    b = hdmc.Batch(reps, sigma=sigma, precision="fp64")
+    b.sweep(60)
+    for k, w in enumerate(reps):
+        r = O.System(w.N, w.Lx, w.Ly, sigma, w.d, 4, w.seed, O.FP64)
+        r.sweep(60)
+        assert np.array_equal(b.state(k)[0], r.state()[0])
+        assert np.array_equal(b.counters()[k], r.counters())
+
+
 @pytest.mark.parametrize("sigma", [1e-6, 0.05, 300.0, 3000.0])
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("q,sweeps", [(8, 60), (22, 4), (34, 2)])   # 32, 8, and 4 or 2 lanes per cell
