@@ -47,12 +47,13 @@ struct Geometry {
     float wxf, wyf;        // binary32 cell widths (FP32 path)
     double sigma, sig2;    // sigma, sigma*sigma
     float sig2f;           // binary32 rounding of sigma*sigma
-    float band_lo, band_hi;   // binary32 estimates of r^2 outside decide an overlap (binary64 mode, pair_bands)
+    float lim;             // -(sigma^2 - band): binary32 estimates of r^2 below the band decide (binary64 mode, pair_bands)
     double d;              // maximum trial displacement
     float df;              // its binary32 rounding
     int nsel;              // trial moves per cell and sub-sweep (n_M)
     uint32_t key0, key1;   // Philox key = seed
     uint32_t flags;        // kNoParticleShuffle | kNoSetShuffle (Table 1 controls); 0 = the method
+    float bands;           // 2 band, the width in which they do not decide
     unsigned int* check;   // builds with -DHDMC_CHECK: device word that collects failed index checks
     // Rows of a strip of a larger grid (spatial decomposition, Sec. 6); a
     // whole system has row0 = 0 and both ranges [0, my-1].
@@ -68,10 +69,11 @@ struct Geometry {
 // 1.3 sigma^2), a tenth of the band.  Below sigma = 2^-40 the band no longer
 // shrinks, so that estimates which near the binary32 underflow range decide
 // nothing.
+constexpr float kBandFloor = 0x1p-80f;   // sigma^2 below which the band no longer shrinks
 inline void pair_bands(Geometry& g) {
-    const double band = 0x1p-15 * (g.sig2 > 0x1p-80 ? g.sig2 : 0x1p-80);
-    g.band_lo = (float)(g.sig2 - band);
-    g.band_hi = (float)(g.sig2 + band);
+    const double band = 0x1p-15 * (g.sig2 > (double)kBandFloor ? g.sig2 : (double)kBandFloor);
+    g.lim = -(float)(g.sig2 - band);
+    g.bands = (float)(2.0 * band);
 }
 
 // Device error word bits: a cell received more than its slots (bit 0); a

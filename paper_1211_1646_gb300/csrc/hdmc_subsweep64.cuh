@@ -154,8 +154,7 @@ __device__ __forceinline__ void subsweep_f64(const Geometry& g, double* __restri
         };
         if (dir23) pair23(__ffs(dir23) - 1, fx23, fy23);
         const double d = g.d, d52 = times_2m52(d);
-        const float lim = -g.band_lo, bands = g.band_hi - g.band_lo;   // certainly overlapping below band_lo
-        const f2x lo2 = pk(lim, lim), band2 = pk(-bands, -bands);      // possibly: up to band_hi
+        const f2x lo2 = pk(g.lim, g.lim), band2 = pk(-g.bands, -g.bands);   // certainly overlapping below 0, possibly below 2 bands
 
         int i = 0;
         auto trial = [&](int tt, auto slots) {
@@ -405,8 +404,12 @@ __device__ __forceinline__ void subsweep_lanes(const Geometry& g, double* __rest
     else any23 = __reduce_or_sync(kFull, has2);
     const bool crowd = __any_sync(kFull, n >= 2), crowdG = G < kSlots && __any_sync(kFull, n > G);
 
-    const float lim = -g.band_lo, bands = g.band_hi - g.band_lo;   // certainly overlapping below band_lo
-    const f2x lo2 = pk(lim, lim), band2 = pk(-bands, -bands);      // possibly: up to band_hi
+    // g.lim and g.bands; with two lanes a cell made from sigma^2 here (17.15 us a
+    // sub-sweep of 73,720 crowded cells, read from the parameters 17.30; with eight
+    // lanes and 16,500 cells 5.32 and 5.24)
+    const float bands = G == 2 ? fmaxf(g.sig2f, kBandFloor) * 0x1p-14f : g.bands;
+    const float lim = G == 2 ? 0.5f * bands - g.sig2f : g.lim;
+    const f2x lo2 = pk(lim, lim), band2 = pk(-bands, -bands);   // certainly overlapping below 0, possibly below 2 bands
     unsigned n_ac = 0, n_lf = 0;
     int i = 0, cur = (int)(perm & 3u);
     double px = sw.own[cur][0][grp], py = sw.own[cur][1][grp];   // disk `cur` before its trial
