@@ -56,7 +56,7 @@ extern "C" {
 #define HDMC_EOVERLAP 4  /* two disks closer than sigma */
 #define HDMC_ETIMEOUT 5  /* a bounded device wait gave up */
 #define HDMC_ENOMEM 6    /* allocation failed or workspace too small */
-#define HDMC_ECHECK 7    /* a kernel of a checked build computed a cell index outside the grid */
+#define HDMC_ECHECK 7    /* a kernel of a checked build computed a cell index outside the grid, or a warp vote missed lanes */
 
 /* ---- precision of the stored coordinates ---- */
 #define HDMC_FP64 0       /* binary64 cell-local offsets; bit-identical to the serial reference */
@@ -618,7 +618,10 @@ const char *hdmc_strerror(int code);
  * with -DHDMC_CHECK.  Such a build checks every cell index its kernels
  * compute against the grid; a bad index is replaced by 0 (so no access
  * leaves the buffer) and sets a bit of the handle's device error word, which
- * the next synchronising call reports as HDMC_ECHECK.  compute-sanitizer is
+ * the next synchronising call reports as HDMC_ECHECK.  It also checks that the
+ * votes and sums over a warp reach all its lanes (as does a build with
+ * -DHDMC_CHECK_WARPS alone, whose kernels are otherwise the product's).
+ * compute-sanitizer is
  * not available on every machine; this is its substitute for the kernels'
  * own index arithmetic.  Normal builds contain none of these checks. */
 #define HDMC_BUILD_CHECK 1

@@ -558,6 +558,7 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
                 hit |= slots_hit(g, cells, sn, dx, dy, dz, b == 31 ? 4 : 2, kSlots3 - 1, at);
             }
         }
+        checked_warp(g.check);
         const bool overlap = (__ballot_sync(kFull, hit) & gm) != 0;
         if (n > 0 && inside && !overlap) {
             if (L == 0) {
@@ -580,13 +581,10 @@ __device__ __forceinline__ void sub3_cells(const G3& g, T* __restrict__ cells, c
         p[8] = sw.own[o][2][grp];
     }
     // counters: one lane per cell
+    checked_warp(g.check);
     const bool count = L == 0 && n > 0;
-    const unsigned tr = __reduce_add_sync(kFull, count ? (unsigned)g.nsel : 0u);
-    const unsigned ac = __reduce_add_sync(kFull, count ? n_ac : 0u), lf = __reduce_add_sync(kFull, count ? n_lf : 0u);
-    if (lane < 4 && tr) {
-        const unsigned v = lane == 0 ? tr : lane == 1 ? ac : lane == 2 ? lf : tr - ac - lf;
-        atomicAdd(ctr + 4 * (blockIdx.x % kCtr3) + lane, (unsigned long long)v);
-    }
+    add_block_counters<1>(count ? (unsigned)g.nsel : 0u, count ? n_ac : 0u, count ? n_lf : 0u,
+                          ctr + 4 * (blockIdx.x % kCtr3));
 }
 
 template <typename T, int G>

@@ -1076,7 +1076,7 @@ const char* hdmc_strerror(int code) {
         case HDMC_EOVERLAP: return "overlapping disks";
         case HDMC_ETIMEOUT: return "bounded device wait timed out";
         case HDMC_ENOMEM: return "out of memory or workspace too small";
-        case HDMC_ECHECK: return "a kernel computed a cell index outside the grid (checked build)";
+        case HDMC_ECHECK: return "a kernel computed a cell index outside the grid, or a warp vote missed lanes (checked build)";
         default: return "unknown error";
     }
 }

@@ -253,11 +253,11 @@ __device__ __forceinline__ float pos_or_far(double v) { return is_empty(v) ? kFa
 // Per-block trial counters bpart[{trials, accepted, left, overlap}] of the
 // block's own slot: each warp adds its sums with fire-and-forget atomic
 // adds (no value returned, so nothing waits on the round trip; integer sums
-// do not depend on their order).  Lanes that the binary64 decisions of their
-// trials kept apart may arrive separately (measured with n_M = 8 in binary64:
-// a full-mask reduction then summed each part by itself, and only the part
-// with lane 0 was counted), so the sums are over the lanes that are here and
-// the first of them adds.
+// do not depend on their order).  The sums are over the lanes that are here and
+// the first of them adds, which is right however a warp arrives.  (Full-mask
+// sums, a __syncwarp() in front or not, counted parts of a warp by themselves
+// when a branch of the trials was compiled without its meeting point; a vote in
+// the same place named the same parts.)
 template <int ROWS>
 __device__ __forceinline__ void add_block_counters(unsigned int n_tr, unsigned int n_acc, unsigned int n_leave,
                                                    unsigned long long* __restrict__ bpart) {

@@ -79,8 +79,23 @@ inline void pair_bands(Geometry& g) {
 // Device error word bits: a cell received more than its slots (bit 0); a
 // computed cell index fell outside the grid (bit 1, builds with -DHDMC_CHECK
 // only, which check every cell index the kernels compute and replace a bad
-// one by 0 so that no access leaves the buffer).
-constexpr uint32_t kErrOverflow = 1u, kErrIndex = 2u;
+// one by 0 so that no access leaves the buffer); a full-mask vote did not
+// reach the whole warp (bit 2, the same builds).
+constexpr uint32_t kErrOverflow = 1u, kErrIndex = 2u, kErrWarp = 4u;
+
+// Warp check of a -DHDMC_CHECK or -DHDMC_CHECK_WARPS build (no code otherwise;
+// the latter leaves the rest of the kernels as they are), in front of the
+// votes and sums that need every lane: does a vote here reach the whole warp?
+// (The predicate is hidden from the compiler, which would fold a constant.)
+__device__ __forceinline__ void checked_warp(unsigned int* check) {
+#if (defined(HDMC_CHECK) || defined(HDMC_CHECK_WARPS)) && defined(__CUDA_ARCH__)
+    unsigned one;
+    asm volatile("mov.u32 %0, 1;" : "=r"(one));
+    if (__ballot_sync(0xffffffffu, one != 0u) != 0xffffffffu && check) atomicOr(check, kErrWarp);
+#else
+    (void)check;
+#endif
+}
 
 // Index check of a -DHDMC_CHECK build (no code otherwise).
 __host__ __device__ __forceinline__ long long checked_cell(unsigned int* check, long long idx, long long limit) {

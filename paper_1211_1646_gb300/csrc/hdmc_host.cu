@@ -19,7 +19,7 @@ int cuda_code(cudaError_t e) {
 }
 
 int error_code(unsigned int device_error) {
-    if (device_error & kErrIndex) return HDMC_ECHECK;
+    if (device_error & (kErrIndex | kErrWarp)) return HDMC_ECHECK;
     if (device_error & kErrOverflow) return HDMC_EOVERFLOW;
     return HDMC_OK;
 }

@@ -312,6 +312,7 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
                 n_tr = (unsigned)NSEL;
                 store_cell(ownp, own);
             }
+            checked_warp(g.check);
             add_block_counters<ROWS>(n_tr, n_acc, n_leave, bpart);
             return;
         }
@@ -435,6 +436,7 @@ __device__ __forceinline__ void subsweep_f32(const Geometry& g, float* __restric
             }
         }
     }
+    checked_warp(g.check);
     if (TRACK) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) net2 += __shfl_xor_sync(0xffffffffu, net2, o);

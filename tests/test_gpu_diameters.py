@@ -27,7 +27,7 @@ def _same(g, r):
     assert np.array_equal(g.counters(), r.counters())
 
 
-@pytest.mark.parametrize("sigma", [1e-6, 0.05, 300.0, 3000.0])
+@pytest.mark.parametrize("sigma", [1e-15, 1e-6, 0.05, 300.0, 3000.0])
 @pytest.mark.parametrize("prec,nx,ny,phi,cells,nsel,sweeps", [
     ("fp64", 94, 110, 0.70, "sigma", 4, 60),      # 8 lanes per cell
     ("fp64", 61, 62, 0.72, "sqrt2", 4, 100),      # 8 lanes, crowded cells
