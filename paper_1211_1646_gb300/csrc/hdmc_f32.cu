@@ -88,12 +88,14 @@ void launch_subsweep_f32_batch(const BatchCtx& c, void* arena, const SweepDraw* 
 
 void launch_shift_batch(const BatchCtx& c, int prec, const void* src, void* dst, const SweepDraw* draws, int j) {
     const dim3 grid(c.sh_blocks), block(kShiftBX, kShiftBY);
-    if (prec == 1)
-        launch_on(c, k_shift_batch<float>, grid, block, c.reps, c.sh_map, reinterpret_cast<const float*>(src),
-                  reinterpret_cast<float*>(dst), draws, c.R, j, c.sts);
-    else
-        launch_on(c, k_shift_batch<double>, grid, block, c.reps, c.sh_map, reinterpret_cast<const double*>(src),
-                  reinterpret_cast<double*>(dst), draws, c.R, j, c.sts);
+    auto run = [&](auto kernel, auto zero) {
+        using T = decltype(zero);
+        launch_on(c, kernel, grid, block, c.reps, c.sh_map, static_cast<const T*>(src), static_cast<T*>(dst), draws, c.R, j,
+                  c.sts);
+    };
+    if (prec == 1) run(k_shift_batch<float, false>, 0.0f);
+    else if (shift_early<double>((long long)c.sh_blocks * (kShiftBX * kShiftBY))) run(k_shift_batch<double, true>, 0.0);
+    else run(k_shift_batch<double, false>, 0.0);
 }
 
 void launch_hist_batch(const BatchCtx& c, int prec, const void* arena) {

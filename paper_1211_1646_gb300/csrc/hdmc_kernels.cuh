@@ -160,7 +160,19 @@ template <> struct ShiftParams<float> {
     }
 };
 
+// EARLY reads the own cell before the draw is known: faster where the latency of
+// the two reads binds (binary64, few cells), slower where the reads themselves do
+// and the cell of the other read is close by (us per shift in-step, both reads
+// after the draw -> EARLY): binary64 1024 disks 2.27 -> 2.22, 65,536 5.90 -> 5.70,
+// 115,850 6.03 -> 5.95, but 1M 29.2 -> 29.4, crowded 570,000 10.2 -> 11.3;
+// binary32 65,536 2.94 -> 2.98, 1M 10.95 -> 11.13, 4M 51.2 -> 52.5.
+constexpr long long kShiftEarlyCells = 200000;
 template <typename T>
+__host__ __device__ constexpr bool shift_early(long long cells) {
+    return sizeof(T) == 8 && cells <= kShiftEarlyCells;
+}
+
+template <typename T, bool EARLY>
 __device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* dst,
                                             const SweepDraw* __restrict__ draw, DevState* __restrict__ st, int bx,
                                             int by, int q) {
@@ -170,7 +182,7 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* 
     const bool live = hx < g.hx && hy < g.hy && cy >= g.slo && cy <= g.shi;   // a strip's halo rows are not its own
     const long long idx = (long long)q * g.cq + (long long)hy * g.hx + hx;
     Cell<T> o, b, r;
-    if (live) load_cell(src + 8 * idx, o);   // before the draw is known
+    if (EARLY && live) load_cell(src + 8 * idx, o);
     const int fdir = draw->fdir;
     const int ax = fdir >> 1;
     const int sgn = (fdir & 1) ? -1 : 1;
@@ -179,6 +191,7 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* 
     if (!live) return;
     const int ncx = ax ? cx : wrap(cx + sgn, g.mx);
     const int ncy = ax ? wrap(cy + sgn, g.my) : cy;
+    if (!EARLY) load_cell(src + 8 * idx, o);
     load_cell(src + 8 * storage_index(g, ncx, ncy), b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) r.x[j] = r.y[j] = T(kEmpty);
@@ -217,7 +230,7 @@ __device__ __forceinline__ void shift_cells(const Geometry& g, const T* src, T* 
     store_cell(dst + 8 * idx, r);
 }
 
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(kShiftBX * kShiftBY)
 k_shift(const Geometry g, const T* src, T* dst, const SweepDraw* __restrict__ draw,
         DevState* __restrict__ st) {
@@ -227,7 +240,7 @@ k_shift(const Geometry g, const T* src, T* dst, const SweepDraw* __restrict__ dr
     // the old cells a block reads from the neighbouring set are read by that
     // set's block at about the same time: the second read hits L2 even when
     // the state does not fit there
-    shift_cells<T>(g, src, dst, draw, st, blockIdx.x >> 2, blockIdx.y, blockIdx.x & 3);
+    shift_cells<T, EARLY>(g, src, dst, draw, st, blockIdx.x >> 2, blockIdx.y, blockIdx.x & 3);
 }
 
 // ---- contact histogram: Sec. 4 ------------------------------------------------------
@@ -760,7 +773,7 @@ k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short*
                               by * 4 + row, partial + 4 * (rd->part_off + local), sw[threadIdx.y]);
 }
 
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(kShiftBX * kShiftBY)
 k_shift_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
               const T* src, T* dst, const SweepDraw* __restrict__ draws, int R, int j,
@@ -772,7 +785,7 @@ k_shift_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __rest
     const int local = (int)blockIdx.x - rd->sh_block0;
     const int q = local & 3, rem = local >> 2;   // the four sets of a tile in adjacent blocks
     const int by = rem / rd->sh_gx, bx = rem - by * rd->sh_gx;
-    shift_cells<T>(rd->g, src + 8 * rd->cell_off, dst + 8 * rd->cell_off, draws + (size_t)j * R + r, sts + r, bx,
+    shift_cells<T, EARLY>(rd->g, src + 8 * rd->cell_off, dst + 8 * rd->cell_off, draws + (size_t)j * R + r, sts + r, bx,
                    by, q);
 }
 
@@ -801,8 +814,14 @@ template <typename T>
 void launch_shift_t(const LaunchCtx& c, const void* src, void* dst, const SweepDraw* draw) {
     const dim3 block(kShiftBX, kShiftBY);
     const dim3 sg = set_grid(c.g, block);
-    launch_on(c, k_shift<T>, dim3(4 * sg.x, sg.y, 1), block, c.g, reinterpret_cast<const T*>(src),
-              reinterpret_cast<T*>(dst), draw, c.st);
+    auto run = [&](auto kernel) {
+        launch_on(c, kernel, dim3(4 * sg.x, sg.y, 1), block, c.g, reinterpret_cast<const T*>(src),
+                  reinterpret_cast<T*>(dst), draw, c.st);
+    };
+    if constexpr (sizeof(T) == 8) {
+        if (shift_early<T>(c.g.C)) return run(k_shift<T, true>);
+    }
+    run(k_shift<T, false>);
 }
 
 template <typename T>
