@@ -4,7 +4,12 @@
 
 namespace hdmc {
 // A binary32 state of up to 64 MB stays in L2 (129 MB, with its other half)
-// from one sub-sweep to the next.
+// from one sub-sweep to the next.  Above, the loads come before the draws where
+// that measured faster (us per sub-sweep in-step, draws first -> loads first):
+// n_M = 4, 1.15M active cells 38.9 -> 37.3; run-time n_M = 12 117.1 -> 114.7;
+// crowded, 590,000 active cells, run-time n_M = 5 35.2 -> 34.7, but crowded
+// n_M = 4 25.7 -> 25.9, n_M = 8 42.4 -> 43.2, and n_M = 1 30.0 -> 30.5.  The
+// other n_M have the one form at every size.
 constexpr long long kAheadCells = 2000000;
 
 void launch_subsweep_f32(const LaunchCtx& c, void* cells, const SweepDraw* draw, int k) {
@@ -16,13 +21,13 @@ void launch_subsweep_f32(const LaunchCtx& c, void* cells, const SweepDraw* draw,
     const int nsel = c.g.nsel;
     const bool ahead = c.g.C <= kAheadCells;   // see subsweep_f32, phase 1
     if (c.g.dense) {   // cells that often hold three or four disks
-        if (ahead) return nsel == 4 ? run(k_subsweep_f32<2, 4, true>) : nsel == 8 ? run(k_subsweep_f32<2, 8, true>)
-                                                                                  : run(k_subsweep_f32<2, 0, true>);
-        return nsel == 4 ? run(k_subsweep_f32<2, 4, true, false>)
-                         : nsel == 8 ? run(k_subsweep_f32<2, 8, true, false>) : run(k_subsweep_f32<2, 0, true, false>);
+        if (nsel == 4) return run(k_subsweep_f32<2, 4, true>);
+        if (nsel == 8) return run(k_subsweep_f32<2, 8, true>);
+        return ahead ? run(k_subsweep_f32<2, 0, true>) : run(k_subsweep_f32<2, 0, true, false>);
     }
     if (!ahead && nsel == 4) return run(k_subsweep_f32<2, 4, false, false>);
     if (!ahead && nsel == 8) return run(k_subsweep_f32<2, 8, false, false>);
+    if (!ahead && nsel > 8) return run(k_subsweep_f32<2, 0, false, false>);
     // n_M fixed at compile time (directions drawn in one pass, trials
     // unrolled) up to kDirChunk; 100 sweeps of 2,585 active cells at n_M = 7 and
     // their pressure: 2.21 -> 1.70 ms
