@@ -43,9 +43,22 @@ void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long*
     launch_check_t<double>(c, cells, out);
 }
 
+// Two lanes per cell for few active cells over all replicas or crowded cells,
+// one thread per cell for many, as in a single system.  ms per 64 sweeps at n_M =
+// 4, two lanes / one thread (one thread with the loads before the draws, the form
+// before the lanes): 18,144 active cells 1.95 / 2.64 (3.46), 27,216 2.18 / 2.78
+// (3.65), 36,288 3.65 / 3.00 (4.08), 72,576 5.75 / 5.15 (6.50), 1.35M 82.8 / 62.9
+// (78.9); n_M = 8 2.66 / 3.57 (4.63), 2.97 / 3.71, 5.03 / 4.02, 8.02 / 7.07, 114.6
+// / 89.0 (107.3); crowded, 147,000 active cells 11.7 / 15.0 (16.0).
+constexpr long long kBatchLaneCells = 32768;
 void launch_subsweep_f64_batch(const BatchCtx& c, void* arena, const SweepDraw* draws, int j, int k) {
-    constexpr int G = 2;
-    launch_on(c, k_subsweep_f64_batch<G>, dim3(c.sub_blocks), dim3(32, 4 * G), c.reps, c.sub_map,
-              reinterpret_cast<double*>(arena), draws, c.R, j, k, c.partial);
+    auto run = [&](auto kernel, int warps) {
+        launch_on(c, kernel, dim3(c.sub_blocks), dim3(32, warps), c.reps, c.sub_map, reinterpret_cast<double*>(arena), draws,
+                  c.R, j, k, c.partial);
+    };
+    if (c.dense || (long long)c.sub_blocks * 128 <= kBatchLaneCells) return run(k_subsweep_lanes_batch<2>, 8);
+    if (c.nsel == 4) return run(k_subsweep_f64_batch<4>, 4);
+    if (c.nsel == 8) return run(k_subsweep_f64_batch<8>, 4);
+    run(k_subsweep_f64_batch<0>, 4);
 }
 }  // namespace hdmc

@@ -756,10 +756,11 @@ k_subsweep_f32_batch(const ReplicaDesc* __restrict__ reps, const unsigned short*
                                      partial + 4 * (rd->part_off + local), sdir, msd + r);
 }
 
-// Binary64: G lanes per cell, a block of G warps per set row and four rows.
+// Binary64: G lanes per cell, a block of G warps per set row and four rows; or
+// one thread per cell (launch_subsweep_f64_batch).
 template <int G>
 static __global__ void __launch_bounds__(128 * G)
-k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
+k_subsweep_lanes_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
                      double* __restrict__ arena, const SweepDraw* __restrict__ draws, int R, int j, int k,
                      unsigned long long* __restrict__ partial) {
     pdl_release();
@@ -771,6 +772,21 @@ k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short*
     const int row = threadIdx.y / G, part = threadIdx.y % G;
     subsweep_lanes<G>(rd->g, arena + 8 * rd->cell_off, draws + (size_t)j * R + r, k, bx * 32 + part * (32 / G),
                               by * 4 + row, partial + 4 * (rd->part_off + local), sw[threadIdx.y]);
+}
+
+template <int NSEL>
+static __global__ void __launch_bounds__(128, 4)
+k_subsweep_f64_batch(const ReplicaDesc* __restrict__ reps, const unsigned short* __restrict__ map,
+                     double* __restrict__ arena, const SweepDraw* __restrict__ draws, int R, int j, int k,
+                     unsigned long long* __restrict__ partial) {
+    pdl_release();
+    __shared__ uint4 sdir[kDirRows64][128];
+    const int r = map[blockIdx.x];
+    const ReplicaDesc* rd = reps + r;
+    const int local = (int)blockIdx.x - rd->sub_block0;
+    const int by = local / rd->sub_gx, bx = local - by * rd->sub_gx;
+    subsweep_f64<4, NSEL>(rd->g, arena + 8 * rd->cell_off, draws + (size_t)j * R + r, k, bx, by,
+                          partial + 4 * (rd->part_off + local), sdir);
 }
 
 template <typename T, bool EARLY>
