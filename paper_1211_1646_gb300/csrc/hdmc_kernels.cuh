@@ -261,10 +261,11 @@ k_shift(const Geometry g, const T* src, T* dst, const SweepDraw* __restrict__ dr
 // with its own roundings.  A cell two steps away is looked at only if some
 // lane has a disk within reach of it (a band of 0.02 sigma with cells of
 // sigma, nowhere with the paper's cells), its corners never.  What is left on
-// the binary64 pipe is seven instructions per queued pair.  A block does four
-// tiles of 32 x 8 cells before it adds its bins to the global ones.  One
-// histogram with its launch, N = 1M: binary32 120 -> 71 us, binary64 241 -> 111
-// us; the paper's cells (N = 1520^2) 196 -> 88 us.
+// the binary64 pipe is seven instructions per queued pair.  A block does a tile
+// of 32 x 8 cells, in large binary32 systems two, before it adds its bins to the
+// global ones.  One histogram with its launch, each pair estimated in both orders
+// -> now: 65,536 disks binary32 18.7 -> 10.5 us, binary64 29.2 -> 14.2; 1M 119 ->
+// 56, 245 -> 91; the paper's cells (N = 1520^2) 189 -> 73, 289 -> 90.
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(double v) { return approx_f32(v); }
 
@@ -279,7 +280,12 @@ __device__ __forceinline__ double widen(float v) {
 __device__ __forceinline__ double widen(double v) { return v; }
 
 constexpr int kHistQueue = 96;   // per-warp candidate queue (< 32 pending + 64 appended)
-constexpr int kHistTiles = 4;    // tiles of kHistBY set rows of a block
+
+// Tiles of kHistBY set rows of a block.  Fewer blocks add fewer bins, more fill
+// the chip: us with one / two / four tiles, binary32 65,536 disks 10.5 / 14.5 /
+// 22.7, 360,000 26.8 / 27.8 / 30.1, 640,000 41.0 / 37.8 / 43.3, 1M 61.0 / 56.1 /
+// 63.3; binary64 65,536 14.2 / 18.6 / 26.4, 1M 90.7 / 96.7 / 103.2.
+constexpr long long kHistTwoCells = 500000;   // binary32: two tiles above
 
 struct HistShared {
     unsigned int bins[kHistBins];
@@ -449,14 +455,14 @@ __device__ __forceinline__ void hist_tile(const Geometry& g, const T* __restrict
     __syncwarp();
 }
 
-template <typename T>
+template <typename T, int TILES>
 __global__ void __launch_bounds__(kHistBX * kHistBY)
 k_hist(const Geometry g, const T* __restrict__ cells, const double* __restrict__ edges2,
        unsigned long long* __restrict__ hist) {
     __shared__ HistShared S;
     hist_begin<T>(g, edges2, S);
 #pragma unroll 1
-    for (int t = 0; t < kHistTiles; ++t) hist_tile<T>(g, cells, S, blockIdx.x, blockIdx.y * kHistTiles + t, blockIdx.z);
+    for (int t = 0; t < TILES; ++t) hist_tile<T>(g, cells, S, blockIdx.x, blockIdx.y * TILES + t, blockIdx.z);
     hist_end(S, hist);
 }
 
@@ -853,8 +859,14 @@ template <typename T>
 void launch_hist_t(const LaunchCtx& c, const void* cells) {
     const dim3 block(kHistBX, kHistBY);
     const dim3 sg = set_grid(c.g, block);
-    k_hist<T><<<dim3(sg.x, (sg.y + kHistTiles - 1) / kHistTiles, sg.z), block, 0, c.stream>>>(c.g, reinterpret_cast<const T*>(cells), c.edges2,
-                                                              c.hist);
+    const T* a = reinterpret_cast<const T*>(cells);
+    if constexpr (sizeof(T) == 4) {
+        if (c.g.C > kHistTwoCells) {
+            k_hist<T, 2><<<dim3(sg.x, (sg.y + 1) / 2, sg.z), block, 0, c.stream>>>(c.g, a, c.edges2, c.hist);
+            return;
+        }
+    }
+    k_hist<T, 1><<<sg, block, 0, c.stream>>>(c.g, a, c.edges2, c.hist);
 }
 
 // ---- snapshot check ---------------------------------------------------------------------
