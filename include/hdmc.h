@@ -154,8 +154,8 @@ int hdmc_psi6(hdmc_t *h, double r_cut, double out[4], double *psi);
  * y), O the accumulated grid origin; cells use the binary32 widths in
  * HDMC_FP32_LOCAL mode.  cell (nullable, host int32[N]) receives each disk's
  * canonical cell index.  The coordinates are put together on the device in the
- * idle half of the state; where they do not fit it (crowded binary32 cells)
- * 20 bytes per disk are allocated for the duration of the call.  Synchronises. */
+ * idle half of the state, in parts where they do not fit it at once (crowded
+ * binary32 cells); nothing is allocated.  Synchronises. */
 int hdmc_positions(hdmc_t *h, double *xy, int32_t *cell);
 
 /* Raw state in the canonical layout described above: local[(4c+j)*2 + k]

@@ -1286,10 +1286,8 @@ int hdmc3_positions(hdmc3_t* h, double* xyz) {
     else run((const float*)h->cells[h->cur]);
     unsigned total = 0;
     int e2 = cuda_code(cudaGetLastError());
+    if (!e2) e2 = cuda_code(cudaMemcpyAsync(xyz, out, bytes, cudaMemcpyDeviceToHost, h->stream));
     if (!e2) e2 = cuda_code(cudaMemcpyAsync(&total, counts + nb, sizeof(total), cudaMemcpyDeviceToHost, h->stream));
-    if (!e2) e2 = cuda_code(cudaStreamSynchronize(h->stream));
-    const size_t got = sizeof(double) * 3 * (size_t)std::min<int64_t>(total, h->N);
-    if (!e2) e2 = cuda_code(cudaMemcpyAsync(xyz, out, got, cudaMemcpyDeviceToHost, h->stream));
     if (!e2) e2 = cuda_code(cudaStreamSynchronize(h->stream));
     if (e2) return e2;
     return (int64_t)total > h->N ? HDMC_EOVERFLOW : e;

@@ -522,40 +522,57 @@ int hdmc_psi6(hdmc_t* h, double r_cut, double out[4], double* psi) {
     return check_device(h);
 }
 
+// Bytes that one copy brings to the host together (three copies of a small
+// system's total, coordinates and cells take longer than the kernels: 1024 disks
+// 55 -> 44 us).
+constexpr size_t kExportOne = 65536;
+
 int hdmc_positions(hdmc_t* h, double* xy, int32_t* cell) {
     if (!h || !xy) return HDMC_EINVAL;
     if (h->nstrips) return HDMC_EINVAL;   // strips sweep in two phases (hdmc_strip_*)
-    // scratch between sweeps: the idle half of the double buffer, or where the
-    // coordinates of a crowded binary32 state do not fit it, a buffer of this call
+    // scratch between sweeps: the idle half of the double buffer; what does not
+    // fit it at once (a crowded binary32 state) is written and copied in parts
     const Geometry& g = h->g;
     const unsigned nb = export_blocks(g);
-    const size_t head = export_counts_bytes(nb), xy_bytes = sizeof(double) * 2 * (size_t)h->N;
-    const size_t need = head + xy_bytes + sizeof(int32_t) * (size_t)h->N;
+    const size_t head = export_counts_bytes(nb), each = 2 * sizeof(double) + (cell ? sizeof(int32_t) : 0);
+    if (h->lay.cells < head + each) return HDMC_EINVAL;   // not met: 16 cells hold 512 bytes
+    const size_t room = (h->lay.cells - head) / each;     // disks of a part
     char* buf = static_cast<char*>(h->cells[h->cur ^ 1]);
-    int e = HDMC_OK;
-    if (need > h->lay.cells) e = cuda_code(cudaMalloc((void**)&buf, need));
-    if (e) return e;
     unsigned* counts = reinterpret_cast<unsigned*>(buf);
     double* out = reinterpret_cast<double*>(buf + head);
-    int32_t* out_cell = reinterpret_cast<int32_t*>(buf + head + xy_bytes);
+    const size_t part = std::min(room, (size_t)h->N);
+    int32_t* out_cell = cell ? reinterpret_cast<int32_t*>(buf + head + 2 * sizeof(double) * part) : nullptr;
     ExportCtx x;
     x.wx = h->prec == HDMC_FP64 ? g.wx : (double)g.wxf;
     x.wy = h->prec == HDMC_FP64 ? g.wy : (double)g.wyf;
     x.Lx = h->prec == HDMC_FP64 ? h->Lx : (double)g.mx * x.wx;
     x.Ly = h->prec == HDMC_FP64 ? h->Ly : (double)g.my * x.wy;
-    x.limit = (unsigned)h->N;
     const LaunchCtx c = h->ctx(h->stream);
-    if (h->prec == HDMC_FP64) launch_export_f64(c, h->cells[h->cur], x, counts, out, out_cell);
-    else launch_export_f32(c, h->cells[h->cur], x, counts, out, out_cell);
     unsigned total = 0;
-    e = cuda_code(cudaGetLastError());
+    int e = HDMC_OK;
+    for (size_t p = 0; p < (size_t)h->N && !e; p += room) {
+        const size_t n = std::min(room, (size_t)h->N - p);
+        x.first = (unsigned)p;
+        x.limit = (unsigned)(p + n);
+        if (h->prec == HDMC_FP64) launch_export_f64(c, h->cells[h->cur], x, counts, out, out_cell);
+        else launch_export_f32(c, h->cells[h->cur], x, counts, out, out_cell);
+        e = cuda_code(cudaGetLastError());
+        if (!e && n == (size_t)h->N && head + each * n <= kExportOne) {   // a small system: one copy
+            char one[kExportOne];
+            const size_t skip = sizeof(unsigned) * nb;   // from the total on
+            e = cuda_code(cudaMemcpyAsync(one, buf + skip, head + each * n - skip, cudaMemcpyDeviceToHost, h->stream));
+            if (!e) e = cuda_code(cudaStreamSynchronize(h->stream));
+            if (e) return e;
+            std::memcpy(&total, one, sizeof(total));
+            std::memcpy(xy, one + head - skip, 2 * sizeof(double) * n);
+            if (cell) std::memcpy(cell, one + head - skip + 2 * sizeof(double) * n, sizeof(int32_t) * n);
+            return (int64_t)total == h->N ? HDMC_OK : HDMC_EOVERFLOW;
+        }
+        if (!e) e = cuda_code(cudaMemcpyAsync(xy + 2 * p, out, 2 * sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
+        if (!e && cell) e = cuda_code(cudaMemcpyAsync(cell + p, out_cell, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, h->stream));
+    }
     if (!e) e = cuda_code(cudaMemcpyAsync(&total, counts + nb, sizeof(total), cudaMemcpyDeviceToHost, h->stream));
     if (!e) e = cuda_code(cudaStreamSynchronize(h->stream));
-    const size_t got = (size_t)std::min<int64_t>(total, h->N);
-    if (!e) e = cuda_code(cudaMemcpyAsync(xy, out, sizeof(double) * 2 * got, cudaMemcpyDeviceToHost, h->stream));
-    if (!e && cell) e = cuda_code(cudaMemcpyAsync(cell, out_cell, sizeof(int32_t) * got, cudaMemcpyDeviceToHost, h->stream));
-    if (!e) e = cuda_code(cudaStreamSynchronize(h->stream));
-    if (need > h->lay.cells) cudaFree(buf);
     if (e) return e;
     return (int64_t)total == h->N ? HDMC_OK : HDMC_EOVERFLOW;
 }

@@ -303,7 +303,7 @@ void launch_check_f64(const LaunchCtx& c, const void* cells, unsigned long long*
 // Export of the global coordinates (hdmc_export.cuh).
 struct ExportCtx {
     double wx, wy, Lx, Ly;   // cell widths and box of the coordinate type
-    unsigned limit;          // disks written at most
+    unsigned first, limit;   // disks written: first <= number < limit
 };
 constexpr int kExportB = 256;              // canonical cells per block
 unsigned export_blocks(const Geometry& g);
