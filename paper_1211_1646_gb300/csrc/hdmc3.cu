@@ -436,12 +436,29 @@ __global__ void __launch_bounds__(kExportB) k_export3(const G3 g, const T* __res
     }
 }
 
+// Adds the counter slots to the counters of the state and empties them (one
+// block of 4 kCtr3 threads).
+static_assert(4 * kCtr3 == 256, "threads of k_check3");
+__device__ __forceinline__ void fold_counters3(Book3* book) {
+    __shared__ unsigned long long sum[4 * kCtr3];
+    const int i = (int)threadIdx.x;
+    sum[i] = book->ctr[i];
+    book->ctr[i] = 0;
+    for (int o = 2 * kCtr3; o >= 4; o >>= 1) {
+        __syncthreads();
+        if (i < o) sum[i] += sum[i + o];
+    }
+    if (i < 4) book->st.ctr[i] += sum[i];
+}
+
 // Check of a cell image (snapshot load): occupied slots form a prefix of
 // each cell (slot 3 occupied before the secondary half is read), occupied
 // coordinates lie in [0, w) on every axis, empty slots hold kEmpty in all
-// three coordinates.  out[0] += spheres, out[1] |= 1 on a bad cell.
+// three coordinates.  out[0] += spheres, out[1] |= 1 on a bad cell.  The first
+// block also folds the counter slots, which a loaded state does not take over.
 template <typename T>
-__global__ void __launch_bounds__(256) k_check3(G3 g, const T* __restrict__ cells, unsigned long long* out) {
+__global__ void __launch_bounds__(256) k_check3(G3 g, const T* __restrict__ cells, unsigned long long* out, Book3* book) {
+    if (blockIdx.x == 0) fold_counters3(book);
     const unsigned s = blockIdx.x * 256 + threadIdx.x;
     unsigned n = 0;
     bool bad = false;
@@ -482,15 +499,15 @@ struct hdmc3_handle {
     void* cells[2];            // current state and shift target
     int cur;
     Draw3* table;              // kDrawChunk3 sweep draws + 1 extra entry
-    Dev3* st;
-    unsigned long long* ctr;   // kCtr3 x 4 trial counters since creation or load
+    Book3* book;
+    Dev3* st;                  // &book->st
+    Book3* copy;               // the host's copy (pinned), valid after read_book3 or collect_book3
     unsigned long long* hist;  // kHistBins accumulator
     double* edges2;            // kHistBins + 1 squared bin edges
     float* binf;               // binary32 bin bounds that decide a bin for certain (certified_bins)
     float lo2f, hi2f;
     int64_t samples;
     uint64_t sweeps, shifts;
-    uint32_t* next;            // device: index of the next sweep to draw
     cudaStream_t cap;          // private stream used only to record graphs
     std::map<std::pair<int, int>, cudaGraphExec_t> graphs;   // (sweeps, buffer) -> graph
     void drop_graphs() {
@@ -513,12 +530,19 @@ int finish3(hdmc3_t* h) {
     return error_code(err);
 }
 
-// Adds the counter slots to the counters of st (the handle's stream is idle).
-int add_counters3(hdmc3_t* h, Dev3& st) {
-    unsigned long long c[4 * kCtr3];
-    const cudaError_t e = cudaMemcpy(c, h->ctr, sizeof(c), cudaMemcpyDeviceToHost);
+// The bookkeeping as copied to the host, the counter slots added to the counters.
+Dev3 collect_book3(const hdmc3_t* h) {
+    Dev3 st = h->copy->st;
+    for (int i = 0; i < 4 * kCtr3; ++i) st.ctr[i & 3] += h->copy->ctr[i];
+    return st;
+}
+
+// Waits for the handle's stream and reads its bookkeeping.
+int read_book3(hdmc3_t* h, Dev3& st) {
+    cudaError_t e = cudaMemcpyAsync(h->copy, h->book, sizeof(Book3), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_code(e);
-    for (int i = 0; i < 4 * kCtr3; ++i) st.ctr[i & 3] += c[i];
+    st = collect_book3(h);
     return HDMC_OK;
 }
 
@@ -704,7 +728,7 @@ void launch_sub3(hdmc3_t* h, cudaStream_t stream, int cur, int jd, int k, bool p
     const LaunchCtx c = ctx3(stream, pdl);
     auto run = [&](auto kernel, auto* cells, unsigned G) {
         const unsigned per = kSubB3 / G;
-        launch_on(c, kernel, dim3((h->g.cq + per - 1) / per), dim3(kSubB3), h->g, cells, h->table, jd, k, h->ctr);
+        launch_on(c, kernel, dim3((h->g.cq + per - 1) / per), dim3(kSubB3), h->g, cells, h->table, jd, k, h->book->ctr);
     };
     // Lanes per cell: few active cells leave the chip idle and the chain of
     // one cell update binds, so its work is spread over a warp; many are bound
@@ -745,11 +769,10 @@ void free3(hdmc3_t* h) {
     cudaFree(h->cells[0]);
     cudaFree(h->cells[1]);
     cudaFree(h->table);
-    cudaFree(h->st);
+    cudaFree(h->book);
+    cudaFreeHost(h->copy);
     h->drop_graphs();
     if (h->cap) cudaStreamDestroy(h->cap);
-    cudaFree(h->ctr);
-    cudaFree(h->next);
     cudaFree(h->hist);
     cudaFree(h->edges2);
     cudaFree(h->binf);
@@ -757,7 +780,7 @@ void free3(hdmc3_t* h) {
 }
 
 void launch_draws3(hdmc3_t* h, cudaStream_t stream, int count) {
-    k_draws3<<<1, kDrawChunk3, 0, stream>>>(h->g, h->table, 0u, h->next, count, 1);
+    k_draws3<<<1, kDrawChunk3, 0, stream>>>(h->g, h->table, 0u, &h->st->next, count, 1);
 }
 
 // K sweeps on s, starting from buffer cur.  The draws kernel and the first
@@ -958,17 +981,15 @@ int hdmc3_save(hdmc3_t* h, void* buf, size_t bytes) {
     std::memset(b, 0, L.cells);
     std::memcpy(b, &hd, sizeof(hd));
     const cudaStream_t s = h->stream;
-    int e = cuda_code(cudaMemcpyAsync(b + L.state, h->st, sizeof(Dev3), cudaMemcpyDeviceToHost, s));
+    int e = cuda_code(cudaMemcpyAsync(h->copy, h->book, sizeof(Book3), cudaMemcpyDeviceToHost, s));
     if (!e)
         e = cuda_code(cudaMemcpyAsync(b + L.hist, h->hist, sizeof(unsigned long long) * kHistBins,
                                       cudaMemcpyDeviceToHost, s));
     if (!e) e = cuda_code(cudaMemcpyAsync(b + L.cells, h->cells[h->cur], L.cell_bytes, cudaMemcpyDeviceToHost, s));
     if (!e) e = cuda_code(cudaStreamSynchronize(s));
     if (e) return e;
-    Dev3 st;
-    std::memcpy(&st, b + L.state, sizeof(st));
-    e = add_counters3(h, st);
-    if (e) return e;
+    Dev3 st = collect_book3(h);
+    st.next = 0;   // a snapshot's header has the sweeps
     std::memcpy(b + L.state, &st, sizeof(st));
     return error_code(st.error);
 }
@@ -1005,8 +1026,8 @@ int hdmc3_load(hdmc3_t* h, const void* buf, size_t bytes) {
     if (!e) e = cuda_code(cudaMemsetAsync(res, 0, 2 * sizeof(unsigned long long), s));
     if (!e) {
         const unsigned blocks = (g.C + 255) / 256;
-        if (h->prec == HDMC_FP64) k_check3<double><<<blocks, 256, 0, s>>>(g, (const double*)idle, res);
-        else k_check3<float><<<blocks, 256, 0, s>>>(g, (const float*)idle, res);
+        if (h->prec == HDMC_FP64) k_check3<double><<<blocks, 256, 0, s>>>(g, (const double*)idle, res, h->book);
+        else k_check3<float><<<blocks, 256, 0, s>>>(g, (const float*)idle, res, h->book);
         e = cuda_code(cudaGetLastError());
     }
     if (!e) e = cuda_code(cudaMemcpyAsync(r, res, sizeof(r), cudaMemcpyDeviceToHost, s));
@@ -1014,10 +1035,8 @@ int hdmc3_load(hdmc3_t* h, const void* buf, size_t bytes) {
     if (e) return e;
     if (r[1] != 0 || r[0] != (unsigned long long)h->N) return HDMC_EINVAL;
     // commit
+    st.next = (uint32_t)hd.sweeps;   // k_check3 has emptied the counter slots
     e = cuda_code(cudaMemcpyAsync(h->st, &st, sizeof(Dev3), cudaMemcpyHostToDevice, s));
-    const uint32_t next = (uint32_t)hd.sweeps;
-    if (!e) e = cuda_code(cudaMemcpyAsync(h->next, &next, sizeof(next), cudaMemcpyHostToDevice, s));
-    if (!e) e = cuda_code(cudaMemsetAsync(h->ctr, 0, sizeof(unsigned long long) * 4 * kCtr3, s));
     if (!e)
         e = cuda_code(cudaMemcpyAsync(h->hist, b + L.hist, sizeof(unsigned long long) * kHistBins,
                                       cudaMemcpyHostToDevice, s));
@@ -1077,17 +1096,14 @@ int hdmc3_create(hdmc3_t** out, int64_t N, double Lx, double Ly, double Lz, doub
     cudaError_t ce = cudaMalloc(&h->cells[0], bytes);
     if (ce == cudaSuccess) ce = cudaMalloc(&h->cells[1], bytes);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->table, sizeof(Draw3) * (kDrawChunk3 + 1));
-    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->st, sizeof(Dev3));
+    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->book, sizeof(Book3));
+    if (ce == cudaSuccess) ce = cudaMemset(h->book, 0, sizeof(Book3));
+    if (ce == cudaSuccess) ce = cudaMallocHost((void**)&h->copy, sizeof(Book3));
     if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
-    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->next, sizeof(uint32_t));
-    if (ce == cudaSuccess) ce = cudaMemset(h->next, 0, sizeof(uint32_t));
-    if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->ctr, sizeof(unsigned long long) * 4 * kCtr3);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->hist, sizeof(unsigned long long) * kHistBins);
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->edges2, sizeof(double) * (kHistBins + 1));
     if (ce == cudaSuccess) ce = cudaMalloc((void**)&h->binf, sizeof(float) * (2 * kHistBins + 2));
     if (ce == cudaSuccess) ce = cudaMemcpy(h->cells[0], raw.data(), bytes, cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) ce = cudaMemset(h->st, 0, sizeof(Dev3));
-    if (ce == cudaSuccess) ce = cudaMemset(h->ctr, 0, sizeof(unsigned long long) * 4 * kCtr3);
     if (ce == cudaSuccess) ce = cudaMemset(h->hist, 0, sizeof(unsigned long long) * kHistBins);
     double E[kHistBins + 1];
     squared_edges(sigma, E);
@@ -1102,6 +1118,7 @@ int hdmc3_create(hdmc3_t** out, int64_t N, double Lx, double Ly, double Lz, doub
         free3(h);
         return cuda_code(ce);
     }
+    h->st = &h->book->st;
     h->g.check = &h->st->error;
     h->lo2f = (float)(E[0] * (1.0 - 1.0e-4));
     h->hi2f = (float)(E[kHistBins] * (1.0 + 1.0e-4));
@@ -1295,23 +1312,19 @@ int hdmc3_positions(hdmc3_t* h, double* xyz) {
 
 int hdmc3_counters(hdmc3_t* h, uint64_t out[4]) {
     if (!h || !out) return HDMC_EINVAL;
-    const int e = finish3(h);
     Dev3 st;
-    const cudaError_t ce = cudaMemcpy(&st, h->st, sizeof(st), cudaMemcpyDeviceToHost);
-    if (ce != cudaSuccess) return cuda_code(ce);
-    const int ec = add_counters3(h, st);
-    if (ec) return ec;
+    const int e = read_book3(h, st);
+    if (e) return e;
     for (int k = 0; k < 4; ++k) out[k] = st.ctr[k];
-    return e;
+    return error_code(st.error);
 }
 
 int hdmc3_info(hdmc3_t* h, int32_t m[3], double w[3], double origin[3], uint64_t* sweeps_done,
                uint64_t* shifts_done) {
     if (!h) return HDMC_EINVAL;
-    const int e = finish3(h);
     Dev3 st;
-    const cudaError_t ce = cudaMemcpy(&st, h->st, sizeof(st), cudaMemcpyDeviceToHost);
-    if (ce != cudaSuccess) return cuda_code(ce);
+    const int e = read_book3(h, st);
+    if (e) return e;
     for (int a = 0; a < 3; ++a) {
         if (m) m[a] = h->g.m[a];
         if (w) w[a] = h->g.w[a];
@@ -1319,7 +1332,7 @@ int hdmc3_info(hdmc3_t* h, int32_t m[3], double w[3], double origin[3], uint64_t
     }
     if (sweeps_done) *sweeps_done = h->sweeps;
     if (shifts_done) *shifts_done = h->shifts;
-    return e;
+    return error_code(st.error);
 }
 
 int hdmc3_set_move_size(hdmc3_t* h, double d) {

@@ -73,7 +73,14 @@ struct Dev3 {
     unsigned long long ctr[4];   // counters of a loaded snapshot (the slots hold the rest)
     double origin[3];
     unsigned int error;          // bit 0: a cell received more than 8 spheres
-    unsigned int pad;
+    uint32_t next;               // index of the next sweep to draw (0 in a snapshot)
+};
+
+// What the host reads and loads of a system besides its cells and histogram,
+// in one copy.
+struct Book3 {
+    Dev3 st;
+    alignas(256) unsigned long long ctr[4 * kCtr3];   // trial counters since creation or load
 };
 
 __host__ __device__ inline unsigned sidx3(const G3& g, int cx, int cy, int cz) {
