@@ -110,7 +110,6 @@ __device__ __forceinline__ T sel3(int ax, T a, T b, T c) {
 template <typename T> struct Shift3 {
     int ax;
     T w, sd, sw, wprev;
-    __device__ __forceinline__ bool inside(T dp) const { return Prm<T>::ge0(dp) && Prm<T>::lt(dp, w); }
     // Is a sphere with moving coordinate x inside its old cell after the
     // shift, and its new coordinate: x - sd, for a migrant (to the cell on the
     // other side of f) one width further and clamped into [0, w).

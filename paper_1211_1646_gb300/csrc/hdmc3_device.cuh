@@ -1,7 +1,7 @@
 // hdmc3_device.cuh -- shared definitions of the three-dimensional (hard
 // sphere) kernels: geometry, per-sweep draws, device bookkeeping, the
-// set-major cell index and the two-half cell layout, slot shuffles and the
-// precision-specific arithmetic of a trial.
+// set-major cell index and the two-half cell layout, and the
+// precision-specific arithmetic of an overlap test.
 //
 // Device layout: the cells of one set are contiguous (set-major), row-major
 // over the half-resolution grid within a set, as in two dimensions.  A cell
@@ -103,14 +103,12 @@ __device__ __forceinline__ uint32_t factorial8(int n) {
 template <typename T> struct Ar3;
 template <> struct Ar3<double> {
     __device__ static double w(const G3& g, int a) { return g.w[a]; }
-    __device__ static double trial(const G3& g, double x, double u) { return x + g.d * u; }
     __device__ static bool hit(const G3& g, double dx, double dy, double dz) {
         return (dx * dx + dy * dy) + dz * dz < g.sig2;
     }
 };
 template <> struct Ar3<float> {
     __device__ static float w(const G3& g, int a) { return g.wf[a]; }
-    __device__ static float trial(const G3& g, float x, float u) { return fmaf(g.df, u, x); }
     __device__ static bool hit(const G3& g, float dx, float dy, float dz) {
         return fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -g.sig2f))) < 0.0f;
     }
@@ -122,41 +120,6 @@ __device__ __forceinline__ T pick8(const T (&v)[8], int i) {
 #pragma unroll
     for (int j = 1; j < 8; ++j) r = i == j ? v[j] : r;
     return r;
-}
-
-template <typename T>
-__device__ __forceinline__ void put8(T (&v)[8], int i, T x) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
-}
-
-// Swap slots J and r (r <= J) of the three coordinate arrays.
-template <int J, typename T>
-__device__ __forceinline__ void swap_slot3(T (&x)[8], T (&y)[8], T (&z)[8], int r) {
-    const T ax = pick8(x, r), ay = pick8(y, r), az = pick8(z, r);
-#pragma unroll
-    for (int s = 0; s < J; ++s) {
-        x[s] = s == r ? x[J] : x[s];
-        y[s] = s == r ? y[J] : y[s];
-        z[s] = s == r ? z[J] : z[s];
-    }
-    x[J] = ax;
-    y[J] = ay;
-    z[J] = az;
-}
-
-// Fisher-Yates decode of k in [0, n!): for j = n-1 down to 1 swap slots j and
-// k mod (j+1), then k /= (j+1).
-template <typename T>
-__device__ __forceinline__ void shuffle3(T (&x)[8], T (&y)[8], T (&z)[8], int n, uint32_t k) {
-#define HDMC3_STEP(J)                                        \
-    if (J < n) {                                             \
-        const int r = (int)(k % (uint32_t)(J + 1));          \
-        k /= (uint32_t)(J + 1);                              \
-        swap_slot3<J>(x, y, z, r);                           \
-    }
-    HDMC3_STEP(7) HDMC3_STEP(6) HDMC3_STEP(5) HDMC3_STEP(4) HDMC3_STEP(3) HDMC3_STEP(2) HDMC3_STEP(1)
-#undef HDMC3_STEP
 }
 
 __device__ __forceinline__ int wrap3(int c, int m) { return c < 0 ? c + m : (c >= m ? c - m : c); }
@@ -213,23 +176,6 @@ template <typename T>
 __device__ __forceinline__ void ld_cell3(const T* cells, const G3& g, unsigned s, T (&x)[8], T (&y)[8], T (&z)[8]) {
     ld_half3<0>(cells + primary3(s), x, y, z);
     ld_rest3(cells, g, s, x, y, z);
-}
-
-// Writes the primary half, and the secondary half when `full` (4 or more
-// spheres: readers then take slot 3 as occupied and read it).
-template <typename T>
-__device__ __forceinline__ void st_cell3(T* cells, const G3& g, unsigned s, const T (&x)[8], const T (&y)[8],
-                                         const T (&z)[8], bool full) {
-    T* p = cells + primary3(s);
-    st4(p, x);
-    st4(p + 4, y);
-    st4(p + 8, z);
-    if (full) {
-        T* q = cells + secondary3(g, s);
-        st4(q, x + 4);
-        st4(q + 4, y + 4);
-        st4(q + 8, z + 4);
-    }
 }
 
 // Slot j of cell s (coordinate a at offset 4a); slots 4..7 may be read only

@@ -244,7 +244,7 @@ constexpr int kDir3 = 8;       // trial directions drawn ahead per cell
 template <typename T, int G> struct Warp3 {
     static constexpr int kCells = 32 / G;
     // kept directions, a ring: fewer than kDir3 left over, 2 G more per round
-    static constexpr int kRing = G <= 4 ? 16 : G <= 8 ? 32 : G <= 16 ? 64 : 128;
+    static constexpr int kRing = G <= 4 ? 16 : G <= 8 ? 32 : 128;
     static_assert(kRing >= kDir3 - 1 + 2 * G, "direction ring");
     // the cell last: the lanes of a warp read neighbouring banks
     T dir[kRing][3][kCells];
