@@ -142,17 +142,16 @@ def profiled_traffic_spheres():
 # two attempts per block; per attempt 12 for three 21-bit fields and their
 # conversion, 4 for the ball test; 6/pi attempts per kept direction); trial
 # position and containment (3 FMAs, 6 compares); the other spheres of the
-# cell (0.37 on average, 7 each); the gathered candidates (12.5 on average at
-# n_M = 4, about 11 tested before a hit ends the scan, 7 each); the cell's
-# gather shared by its n_M = 4 trials (31 occupied neighbour slots at 13
-# each, reach box 20); the shuffle shared likewise (a Philox block and the
-# decode for the 27 % of cells with n >= 2).
+# cell (0.37 on average, 7 each: 3 differences, 3 FMAs, 1 compare); the spheres
+# of the 26 neighbour cells that are within reach of the cell's trials (12.5 on
+# average at n_M = 4, about 11 tested before a hit decides, 7 each); the
+# shuffle shared by the cell's n_M = 4 trials (a Philox block and the decode for
+# the 27 % of cells with n >= 2).
 SPHERE_ALU_OPS_PER_TRIAL = {
     "direction": (80.0 / 2 + 12 + 4) * 6 / math.pi,
     "trial_and_containment": 9.0,
     "own_cell": 0.37 * 7,
     "candidates": 11 * 7.0,
-    "gather": (31 * 13 + 20) / 4.0,
     "shuffle": 0.27 * 100 / 4.0,
 }
 

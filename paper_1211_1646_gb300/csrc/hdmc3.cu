@@ -731,12 +731,17 @@ void launch_sub3(hdmc3_t* h, cudaStream_t stream, int cur, int jd, int k, bool p
     };
     // Lanes per cell: few active cells leave the chip idle and the chain of
     // one cell update binds, so its work is spread over a warp; many are bound
-    // by instructions, of which wide groups need more.  us per sub-sweep at
-    // n_M = 4 with 32 / 8 / 4 / 2 lanes, binary32 then binary64 (plain launches):
-    //     2,197 active cells   6.2 / 6.7 / 8.2 / 8.6       9.2 / 11.6 / 13.2 / 17.1
-    //     7,000               10.3 / 8.3 / 8.5 / 10.3     16.0 / 14.1 / 15.7 / 18.6
-    //    32,768               29.0 / 19.3 / 15.7 / 16.2   46.8 / 34.7 / 29.8 / 31.8
-    //   132,651              103.2 / 55.4 / 39.7 / 37.1   172 / 108 / 93.2 / 93.9
+    // by instructions, of which wide groups need more.  us per sub-sweep in-step
+    // with 32 / 8 / 4 / 2 lanes, binary32 at n_M = 4, binary64 at n_M = 4 (no
+    // form with two lanes), then at 8:
+    //       216 active cells   3.87 / 4.83 / 5.84 / 7.37   4.92 / 9.11 / 10.9   7.31 / 15.8 / 18.0
+    //     2,197                4.64 / 6.01 / 5.39 / 6.11   6.82 / 10.6 / 9.49   9.44 / 15.9 / 14.0
+    //     4,096                6.41 / 7.10 / 7.40 / 6.71   9.15 / 12.2 / 13.1   12.2 / 18.1 / 19.5
+    //     6,859                9.79 / 6.97 / 7.79 / 7.92   11.6 / 12.2 / 14.2   15.7 / 18.1 / 20.4
+    //    12,167                13.8 / 6.77 / 7.57 / 8.20   17.1 / 11.5 / 13.4   23.4 / 17.5 / 19.4
+    //    17,576                18.8 / 9.22 / 7.83 / 9.05   23.3 / 17.1 / 14.0   31.5 / 24.8 / 21.2
+    //    32,768                34.0 / 14.7 / 12.4 / 12.0   41.4 / 27.0 / 23.3   55.9 / 39.3 / 33.7
+    //   140,608                 142 / 46.4 / 35.8 / 31.1    168 / 92.0 / 76.8    223 /  133 /  106
     const unsigned cq = h->g.cq;
     if (h->prec == HDMC_FP64) {
         double* a = (double*)h->cells[cur];

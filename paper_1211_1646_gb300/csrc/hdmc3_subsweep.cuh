@@ -8,16 +8,16 @@
 // are rare (flagged per warp, read when present).
 //
 // What binds it: with few active cells the chain of one cell update (loads,
-// Philox, n_M dependent trials), which wide groups shorten; with many the
-// instructions (binary32: issue and the L1 wavefronts of the cell loads, 48 %
-// of peak) and in binary64 also the binary64 pipe, which has two instructions
-// per trial coordinate.  One thread per cell, which first gathered the
-// neighbours within reach of its trials into shared memory, took (us per
-// sub-sweep, n_M = 4, before -> now, the latter as programmatic dependents):
-//     216 active cells (N = 2048)       binary32 14.1 ->  4.1   binary64  46.3 ->  5.1
-//   2,197             (N = 16384)                14.4 ->  4.7             45.6 ->  7.0
-//  32,768             (N = 256,000)              16.7 -> 14.7             53.6 -> 29.8
-// 132,651             (N = 1,048,576)            39.4 -> 32.9            165.3 -> 77.0
+// Philox, n_M dependent trials), which wide groups shorten; with many latency at
+// 10 to 12 warps per SM (168 registers) beside the instructions, and in binary64
+// also the binary64 pipe, which has two instructions per trial coordinate.  One
+// thread per cell, which first gathered the neighbours within reach of its trials
+// into shared memory, took (us per sub-sweep in-step, n_M = 4, phi = 0.47, before
+// -> now):
+//     216 active cells (N = 2048)       binary32 14.4 ->  3.9   binary64  47.6 ->  4.9
+//   2,197             (N = 16384)                14.3 ->  4.6             46.6 ->  6.8
+//  32,768             (N = 256,000)              16.5 -> 11.7             53.4 -> 23.4
+// 140,608             (N = 1,048,576)            39.5 -> 30.8            166.5 -> 76.6
 #pragma once
 
 #include "hdmc3_device.cuh"
@@ -237,7 +237,7 @@ __device__ __forceinline__ bool slots_hit(const G3& g, const T* cells, unsigned 
     return hit;
 }
 
-constexpr int kSubB3 = 32;     // threads of a sub-sweep block: one warp, no block barrier (blocks of 4 warps: 41.0 us)
+constexpr int kSubB3 = 32;     // threads of a sub-sweep block: one warp, no block barrier (blocks of 4 warps: 41 instead of 37 us at 132,651 active cells)
 constexpr int kDir3 = 8;       // trial directions drawn ahead per cell
 
 // Shared memory of one warp's cells.
