@@ -66,7 +66,7 @@ def ncu_case(args):
     build.build()
     if args.ncu_case == "batch64":
         b = hdmc.Batch(workloads.batch64(), precision="fp32")
-        b.set_rows(1)
+        b.set_rows(2)
         hdmc.hdmc_batch_set_nselect(b.b, [8] * b.R)   # the autotuner's choice for this workload
         b.sweep(3)
         b.sample()

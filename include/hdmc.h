@@ -73,6 +73,9 @@ extern "C" {
  * rule gives fewer than 4 cells or cells narrower than sigma. */
 #define HDMC_CELLS_SQRT2 0x100
 
+/* Both coordinates of an unused slot.  Lengths may be in any unit in which
+ * sigma stays below 4000: in binary32 and in the contact histogram a disk of
+ * that size would reach the slot's place. */
 #define HDMC_EMPTY_SLOT (-1.0e4)
 #define HDMC_HIST_BINS 200 /* contact histogram: bins of 1e-4 sigma over [sigma, 1.02 sigma) (Sec. 4) */
 
@@ -621,9 +624,9 @@ const char *hdmc_strerror(int code);
  * the next synchronising call reports as HDMC_ECHECK.  It also checks that the
  * votes and sums over a warp reach all its lanes (as does a build with
  * -DHDMC_CHECK_WARPS alone, whose kernels are otherwise the product's).
- * compute-sanitizer is
- * not available on every machine; this is its substitute for the kernels'
- * own index arithmetic.  Normal builds contain none of these checks. */
+ * compute-sanitizer is not available on every machine; this is its substitute
+ * for the kernels' own index arithmetic.  Normal builds contain none of these
+ * checks. */
 #define HDMC_BUILD_CHECK 1
 int hdmc_build_flags(void);
 

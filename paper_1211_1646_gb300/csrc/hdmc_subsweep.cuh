@@ -18,12 +18,12 @@ namespace hdmc {
 //      in shared memory, kDirChunk at a time).  They depend on the draw table
 //      alone, so with AHEAD they come before pdl_wait: as a programmatic
 //      dependent the kernel draws them while the previous kernel's last blocks
-//      run.  Where the state does not fit L2 the loads go first and the draws
-//      cover their latency.  us per sub-sweep in-step at n_M = 4, loads first
-//      -> draws first: 270 active cells 1.84 -> 1.69, 9k 3.6 -> 2.6, 73k 4.05 ->
-//      3.2, 293k 10.6 either way (n_M = 8 16.4 -> 15.8), 1.15M (147 MB) 37.3 ->
-//      38.9; crowded 9k 4.0 -> 2.7.  Draws first only in the blocks of the
-//      first wave: 11.0 at 293k;
+//      run.  Where the state does not fit L2 the loads may go first, the draws
+//      covering their latency (launch_subsweep_f32).  us per sub-sweep in-step
+//      at n_M = 4, loads first -> draws first: 270 active cells 1.84 -> 1.69, 9k
+//      3.6 -> 2.6, 73k 4.05 -> 3.2, 293k 10.6 either way (n_M = 8 16.4 -> 15.8),
+//      1.15M (147 MB) 37.3 -> 38.9; crowded 9k 4.0 -> 2.7.  Draws first only in
+//      the blocks of the first wave: 11.0 at 293k;
 //   2. load the own cell and the 8 neighbouring cells (they belong to other
 //      sets and are not written by this launch);
 //   3. shuffle the disks with the draw in field 0 of the stream's first block,
